@@ -135,12 +135,26 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
   const size_t wy_doubles = wy ? 0 : wy_panel_doubles(NB) * (size_t)np;
   const size_t gp_doubles = wy ? 0 : (size_t)np * Sg * NB * NB;
   const size_t work_doubles = panel_update_work_doubles(m, nrhs, NB, ctx->num_sms);
-  slqr_status st = ensure_workspace(ctx, (wy_doubles + gp_doubles + work_doubles) * 8 + 256);
+  const size_t head_bytes = align_up((wy_doubles + gp_doubles) * 8, 256);
+  // kFxMinCols right-hand sides and up: the products on the tensor cores
+  // (tc_fp64.cu), unless the scratch does not fit
+  bool fx = NB == 64 && nrhs >= kFxMinCols;
+  const size_t fx_v = align_up(fx_v_bytes(m), 256);
+  const size_t fx_work = align_up(fx_work_bytes(m, nrhs, ctx->num_sms), 256);
+  slqr_status st = SLQR_OK;
+  if (fx) {
+    st = ensure_workspace(ctx, head_bytes + fx_v + fx_work + (size_t)np * nrhs * sizeof(unsigned));
+    if (st == SLQR_EBUSY || st == SLQR_ENOMEM) fx = false;
+    else if (st != SLQR_OK) return st;
+  }
+  if (!fx) st = ensure_workspace(ctx, head_bytes + work_doubles * 8 + 256);
   if (st != SLQR_OK) return st;
   double *base = (double *)ctx->ws.ptr;
   double *wy_store = base;
   double *Gp = base + wy_doubles;
-  double *work = Gp + gp_doubles;
+  char *tail = (char *)base + head_bytes;
+  double *work = (double *)tail;
+  unsigned *cmax = (unsigned *)(tail + fx_v + fx_work);
   if (!wy) {
     double gflops = 0.0;
     for (int pnl = 0; pnl < np; ++pnl) gflops += 2.0 * (m - pnl * NB) * NB * NB;
@@ -157,6 +171,23 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
     if (st != SLQR_OK) return st;
   }
   const double *wys = wy ? wy : wy_store;
+  if (fx) {
+    fx_colmax(B, ldb, m, nrhs, ntop, false, cmax, np, ctx->num_sms, stream);
+    for (int pnl = 0; pnl < np; ++pnl) {
+      const int k0 = pnl * NB, nbw = std::min(NB, K - k0);
+      const int skip = ntop > 0 ? ntop - (k0 + nbw) : 0;
+      const double *wyp = wys + (size_t)pnl * wy_panel_doubles(NB);
+      int slot = prof_begin(ctx, stream);
+      fx_split_v(A, lda, wyp, k0, nbw, m - k0 - skip, skip, tail, stream);
+      prof_end(ctx, stream, slot, kVtx, 0.0);
+      if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip, wyp, tail, B, ldb, nrhs,
+                     cmax + (size_t)pnl * nrhs,
+                     pnl + 1 < np ? cmax + (size_t)(pnl + 1) * nrhs : nullptr, tail + fx_v, fx_work,
+                     stream))
+        return fail(ctx, SLQR_ENOMEM, "internal: Q^T B workspace too small");
+    }
+    return check_launch(ctx, "Q^T B");
+  }
   for (int pnl = 0; pnl < np; ++pnl) {
     const int k0 = pnl * NB;
     const int nbw = std::min(NB, K - k0);

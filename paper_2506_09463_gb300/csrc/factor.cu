@@ -1249,13 +1249,34 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   const size_t wy_doubles = wy ? 0 : wy_panel_doubles(NB) * (size_t)std::max(np, 1);
   // (the FP32 path also keeps a row-major copy of V for the tensor-core update)
   // (the FP32 path also keeps a row-major V, or the BF16 pairs of V and W')
-  const size_t work_doubles = panel_update_work_doubles(m, n, NB, ctx->num_sms) +
-                              (std::is_same<T, float>::value ? (size_t)(m + n) * NB : 0);
-  const size_t bytes = 256 +
-                       (rec_doubles + srec_doubles + gpart_doubles + prow_doubles + wy_doubles) * 8 +
-                       work_doubles * sizeof(T) + 256;
-  slqr_status st = ensure_workspace(ctx, bytes);
-  if (st != SLQR_OK) return st;
+  size_t work_doubles = panel_update_work_doubles(m, n, NB, ctx->num_sms) +
+                        (std::is_same<T, float>::value ? (size_t)(m + n) * NB : 0);
+  const size_t head_bytes =
+      256 + (rec_doubles + srec_doubles + gpart_doubles + prow_doubles + wy_doubles) * 8 + 256;
+  // FP64 updates of at least kFxMinCols columns run on the tensor cores
+  // (tc_fp64.cu) with panels of 64; the digit images of V (of two panels: the
+  // rest of one update runs beside the next panel), the update's scratch and
+  // the column maxima follow the workspace of the FP64-pipe kernels, which
+  // narrow updates still use.  Where that does not fit the device or the
+  // context's budget, every update stays on the FP64 pipe.
+  bool fx = std::is_same<T, double>::value && NB == 64 && n - NB >= kFxMinCols && np > 1;
+  const size_t fx_v = align_up(fx_v_bytes(m), 256);
+  const size_t fx_work = align_up(fx_work_bytes(m, n, ctx->num_sms), 256);
+  const size_t fx_cm = align_up((size_t)np * n * sizeof(unsigned), 256);
+  slqr_status st = SLQR_OK;
+  if (fx) {
+    // (at most m / 64 row slices, see split_count)
+    const size_t narrow = ((size_t)std::max(1, m / 64) + 1) * kFxMinCols * NB;
+    const size_t with_fx = head_bytes + align_up(narrow * sizeof(T), 256) + 2 * fx_v + fx_work + fx_cm;
+    st = ensure_workspace(ctx, with_fx);
+    if (st == SLQR_OK) work_doubles = narrow;
+    else if (st == SLQR_EBUSY || st == SLQR_ENOMEM) fx = false;
+    else return st;
+  }
+  if (!fx) {
+    st = ensure_workspace(ctx, head_bytes + work_doubles * sizeof(T));
+    if (st != SLQR_OK) return st;
+  }
   char *base = (char *)ctx->ws.ptr;
   unsigned *bar = (unsigned *)base;
   double *rec = (double *)(base + 256);
@@ -1265,6 +1286,11 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   double *wy_store = wy ? wy : prow + prow_doubles;
   // 256-byte aligned (vector stores and TMA maps of the trailing update)
   T *work = (T *)align_up((size_t)(prow + prow_doubles + wy_doubles), 256);
+
+  char *fx_base = (char *)align_up((size_t)(work + work_doubles), 256);
+  void *vbuf[2] = {fx_base, fx_base + fx_v};
+  void *fxw = fx_base + 2 * fx_v;
+  unsigned *cmax = (unsigned *)(fx_base + 2 * fx_v + fx_work);   // [panel][column]
 
   cudaError_t e = cudaMemsetAsync(bar, 0, 256, stream);
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
@@ -1339,6 +1365,17 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
     bar_base += 2u * (unsigned)P;                 // two grid barriers per panel
     return SLQR_OK;
   };
+  // digits of the panel's reflectors for its update, right behind the panel
+  auto split_v = [&](int pnl, cudaStream_t s) {
+    const int k0 = pnl * NB, nbw = std::min(NB, K - k0), skip = skip_of(k0, nbw);
+    if (!fx || n - (k0 + nbw) < kFxMinCols) return;
+    if constexpr (std::is_same<T, double>::value) {
+      int slot = prof_begin(ctx, s);
+      fx_split_v(A, lda, wy_store + (size_t)pnl * wy_panel_doubles(NB), k0, nbw, m - k0 - skip, skip,
+                 vbuf[pnl & 1], s);
+      prof_end(ctx, s, slot, kVtx, 0.0);
+    }
+  };
   // the fused look-ahead kernel's grid barriers count on their own counter
   // (bar[32], another cache line than the panels' bar[0])
   unsigned la_base = 0;
@@ -1356,6 +1393,21 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
                                &lst))
         return lst;
     }
+    if constexpr (std::is_same<T, double>::value) {
+      // (a column that once was in a narrow update stays in narrow ones: its
+      // maxima are not needed any more)
+      if (fx && c_end - c_begin >= kFxMinCols) {
+        const int skip = skip_of(k0, nbw);
+        if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip,
+                       wy_store + (size_t)pnl * wy_panel_doubles(NB), vbuf[pnl & 1],
+                       A + (size_t)c_begin * lda, lda, c_end - c_begin,
+                       cmax + (size_t)pnl * n + c_begin,
+                       pnl + 1 < np ? cmax + (size_t)(pnl + 1) * n + c_begin : nullptr, fxw, fx_work,
+                       us))
+          return fail(ctx, SLQR_ENOMEM, "internal: trailing-update workspace too small");
+        return check_launch(ctx, "trailing update");
+      }
+    }
     return panel_update_impl<T, NB>(ctx, m, k0, nbw, A, lda,
                                  wy_store + (size_t)pnl * wy_panel_doubles(NB),
                                  A + (size_t)c_begin * lda, lda, c_end - c_begin, work,
@@ -1365,15 +1417,19 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   e = cudaEventRecord(ctx->ev_start, stream);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(aux, ctx->ev_start, 0);
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "event: %s", cudaGetErrorString(e));
+  if constexpr (std::is_same<T, double>::value) {
+    if (fx) fx_colmax(A, lda, m, n, ntop, true, cmax, np, ctx->num_sms, stream);
+  }
   st = launch_panel(0, stream);
   if (st != SLQR_OK) return st;
-  // FP64: the panels on the auxiliary stream, the updates (the longer chain)
-  // back to back on the caller's stream.  FP32: the panels (the longer chain)
-  // right behind the look-ahead on the caller's stream, so that a panel is
-  // never queued behind the first kernel of the rest of the update and has
-  // its SMs before the update fills the GPU, and the rest of each update on
-  // the auxiliary stream.
-  constexpr bool kPanelsOnCaller = std::is_same<T, float>::value;
+  split_v(0, stream);
+  // Updates on the FP64 pipe: the panels on the auxiliary stream, the updates
+  // (the longer chain) back to back on the caller's stream.  FP32 and tensor-
+  // core FP64 updates: the panels (the longer chain) right behind the
+  // look-ahead on the caller's stream, so that a panel is never queued behind
+  // the first kernel of the rest of the update and has its SMs before the
+  // update fills the GPU, and the rest of each update on the auxiliary stream.
+  const bool panels_on_caller = std::is_same<T, float>::value || fx;
   for (int pnl = 0; pnl < np; ++pnl) {
     const int k0 = pnl * NB;
     const int nbw = std::min(NB, K - k0);
@@ -1385,7 +1441,7 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       e = cudaEventRecord(ctx->ev_ready, stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(aux, ctx->ev_ready, 0);
       if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "event: %s", cudaGetErrorString(e));
-      if (kPanelsOnCaller) {
+      if (panels_on_caller) {
         // rest of the update of panel p (aux) || panel p+1 (caller's stream)
         st = update(pnl, c0 + next_w, n, false, aux);
         if (st != SLQR_OK) return st;
@@ -1393,6 +1449,7 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
         if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "event: %s", cudaGetErrorString(e));
         st = launch_panel(pnl + 1, stream);
         if (st != SLQR_OK) return st;
+        split_v(pnl + 1, stream);
         e = cudaStreamWaitEvent(stream, ctx->ev_panel, 0);
       } else {
         st = launch_panel(pnl + 1, aux);

@@ -152,6 +152,31 @@ int launch_vtx_tc(const float *A, int lda, const double *Vtop, int k0, int M, in
                   void (*vtop_part)(const float *, int, const double *, int, int, const float *, int,
                                     int, float *, cudaStream_t));
 
+// The trailing update of an FP64 factorization (and Q^T B) on the tensor cores
+// by exact splitting (tc_fp64.cu), panels of 64 reflectors.
+//   fx_v_bytes, fx_work_bytes  sizes of one panel's digit images of V and of the
+//                              scratch of an update of up to n columns
+//   fx_colmax    cmax[p][c], p < np: largest high word of column c over the rows
+//                of panel p that no earlier panel changes (stacked_top > 0: a
+//                stacked [L^T; C] with that many rows on top; upper: only the
+//                upper triangle of those is read, the rest is zero)
+//   fx_split_v   digit images of the panel's V
+//   fx_update    X -= V T^T V^T X (rows of the panel at k0, ldx, N columns);
+//                cmax: column maxima of X over those rows; cnext (or NULL)
+//                receives the maxima over the rows of the next panel.  False
+//                (nothing launched) when work_bytes is too small.
+constexpr int kFxMinCols = 16;       // narrower updates stay on the FP64 pipe
+slqr_status init_fx_attrs(slqr_ctx *ctx);
+size_t fx_v_bytes(int m);
+size_t fx_work_bytes(int m, int n, int num_sms);
+void fx_colmax(const double *X, int ldx, int m, int n, int stacked_top, bool upper, unsigned *cmax,
+               int np, int num_sms, cudaStream_t stream);
+void fx_split_v(const double *A, int lda, const double *Vtop, int k0, int nbw, int M, int skip,
+                void *vbuf, cudaStream_t stream);
+bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy_panel,
+               const void *vbuf, double *X, int ldx, int N, const unsigned *cmax, unsigned *cnext,
+               void *work, size_t work_bytes, cudaStream_t stream);
+
 // slqr_batch_factor with a per-problem stacked top block (ntop[i] rows, 0 for a
 // dense problem; ntop may be NULL); takes the context mutex.
 slqr_status batch_factor_locked(slqr_ctx *ctx, int count, const int *m, const int *n,

@@ -1,0 +1,857 @@
+// tc_fp64.cu -- the two FP64 products of the compact-WY trailing update
+//   W = V^T X   and   X -= V W'
+// on the 5th-generation tensor cores, by error-free splitting (the scheme of
+// Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59, 2012): every operand
+// is written as an integer times a power of two per vector, the integer in
+// balanced base-256 digits, and products of digit matrices are summed exactly.
+//
+//   x = 2^(e-55) sum_i d_i 256^(6-i),   d_i in [-128, 127], i = 0..6
+//
+// e is the exponent of the vector's largest entry, so the rounding of x to
+// this grid is at most 2^(e-56): a quarter of the half-ulp that one FP64
+// operation on that entry commits.  The digits are exact in FP16.  A product
+// of two digits is an integer of at most 2^14 in magnitude; the tensor core
+// sums them in FP32, which is exact while the sum stays below 2^24: at most
+// 7 pairs of digits of the same order i + j, over at most 128 terms.  The 34
+// pairs with i + j <= 7 are kept (the first dropped ones are 2^-8 times the
+// rounding above), one accumulator per order in tensor memory, and the eight
+// orders are put together in integer arithmetic before one rounding to FP64.
+// The residual ||A - Q R|| / ||A|| in 128-bit arithmetic: 3.70e-16 with these
+// kernels, 4.92e-16 with the DFMA kernels of factor.cu (700 x 300 Gaussian),
+// 3.05e-16 against 3.38e-16 (3000 x 260), 2.94e-16 against 2.98e-16
+// (16384 x 260), 6.1e-16 against 9.2e-16 (rows graded over 10^16).
+//
+// Why: the FP64 pipe of GB300 does 2 DFMA per SM and clock, 1.2 TFLOP/s, and
+// the products ran at 82-91% of that.  34 FP16 products cost 34/1834 of the
+// same work at the tensor rate, so the products are bound by memory, by the
+// digit extraction and by the reassembly instead.  Both products over a whole
+// 8192 x 8192 factorization: 663 ms on the FP64 pipe, 88 ms here.
+//
+// Operand layout: K-major shared-memory images of the digit matrices, written
+// by the producing kernel in the exact (swizzled) form the MMA reads, so that
+// a tile is one bulk copy:
+//   V1  per 32 rows:     [digit][reflector a][32 rows]   64-byte rows, SWIZZLE_64B
+//   V2  per 128 rows:    [digit][row][64 reflectors]    128-byte rows, SWIZZLE_128B
+//   W   per 32 columns:  [digit][column][64 reflectors] 128-byte rows, SWIZZLE_128B
+// The digit matrices of one operand are stacked, so A_i times all B_j with
+// j <= 7 - i is one MMA (N = 64 or 32 per digit) whose result columns are the
+// accumulators of the orders i, i + 1, ...
+#include "tc_common.cuh"
+
+#include <cuda_fp16.h>
+#include <algorithm>
+
+namespace slqr {
+
+constexpr int kFxD = 7;                       // digits
+constexpr int kFxOrders = 8;                  // accumulated orders i + j
+constexpr int kFxThreads = 512;
+constexpr int kFxV1Chunk = kFxD * 64 * 64;            // 28672 B: 32 rows
+constexpr int kFxV2Tile = kFxD * 128 * 128;           // 114688 B: 128 rows
+constexpr int kFxWTile = kFxD * 32 * 128;             // 28672 B: 32 columns
+constexpr int kFxXStage = kFxD * 128 * 64;            // 57344 B: 128 columns x 32 rows
+constexpr int kFxStage = kFxXStage + kFxV1Chunk;
+constexpr size_t kFxVtxSmem = 2 * (size_t)kFxStage + 1024;
+constexpr size_t kFxUpdSmem = (size_t)kFxV2Tile + 2 * kFxWTile + 1024;
+constexpr int kFxNonFinite = 1 << 20;         // exponent that stands for Inf / NaN
+
+// D = F32, A = B = F16, both K-major, M = 128; N is added per MMA
+constexpr uint32_t kIdescF16 = (1u << 4) | ((128u >> 4) << 24);
+
+__device__ __forceinline__ uint32_t fx_idesc(int n) { return kIdescF16 | ((uint32_t)(n >> 3) << 17); }
+
+// K-major operand with 64-byte rows, SWIZZLE_64B, 8-row groups 512 bytes apart
+__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;                    // SWIZZLE_64B
+  return d;
+}
+
+__device__ __forceinline__ void fx_mma(uint32_t d, uint64_t ad, uint64_t bd, int n, bool accum) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+               " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+               :: "r"(d), "l"(ad), "l"(bd), "r"(fx_idesc(n)), "r"(accum ? 1u : 0u) : "memory");
+}
+
+__device__ __forceinline__ void fx_commit(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+               :: "r"(smem_u32(bar)) : "memory");
+}
+
+// 1-D bulk copy (16-byte aligned, a multiple of 16 bytes) counted on an mbarrier
+__device__ __forceinline__ void fx_bulk(uint32_t dst, const void *src, uint32_t bytes,
+                                        uint64_t *bar) {
+  const uint32_t b = smem_u32(bar);
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes)
+               : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes"
+               " [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(b) : "memory");
+}
+
+// High word of |x| (sign cleared): ordered as |x|.
+__device__ __forceinline__ uint32_t fx_hi(double x) {
+  return (uint32_t)__double2hiint(x) & 0x7fffffffu;
+}
+
+// Key of a vector maximum: the high word of |x| with the exponent unbiased (a
+// denormal counts as its binade), plus a power of two as `shift` exponents;
+// kFxZero for a zero.
+constexpr int kFxZero = -0x7fffffff;
+__device__ __forceinline__ int fx_key_of_hi(uint32_t hi) {
+  return (int)(hi < 0x00100000u ? (hi | 0x00100000u) : hi) - (1023 << 20);
+}
+__device__ __forceinline__ int fx_key(double x, int shift) {
+  return x != 0.0 ? fx_key_of_hi(fx_hi(x)) + shift * (1 << 20) : kFxZero;
+}
+
+// Exponent e of a vector whose largest entry has this key: every entry is at
+// most 1.9883 * 2^(e-1), so that |x| 2^(55-e) stays within the balanced digits
+// (127 (256^7 - 1) / 255 = 1.9921 * 2^54).
+__device__ __forceinline__ int fx_exp(int key) {
+  return (key >> 20) + 1 + ((key & 0xfffff) >= 0xFD000 ? 1 : 0);   // (shift: floor)
+}
+
+__device__ __forceinline__ int fx_exp_of_hi(uint32_t hi) { return fx_exp(fx_key_of_hi(hi)); }
+
+// round(x 2^(55-e)) as seven balanced digits, each biased by 128: byte 6 - i
+// of the result is d_i + 128.
+__device__ __forceinline__ unsigned long long fx_digits(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int Ef = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = b & 0xfffffffffffffull;
+  m |= Ef ? (1ull << 52) : 0ull;
+  const int rsh = min(max(1022 + e - max(Ef, 1), 0), 62);
+  m = (((m << 3) >> rsh) + 1) >> 1;                       // (m << 2) >> rsh, rounded
+  const unsigned long long bias = 0x80808080808080ull;
+  return (long long)b < 0 ? bias - m : bias + m;
+}
+
+// The same with three bits more for the leading digit (|x| up to 2^3 times
+// the bound above): bytes 5 .. 0 biased, the rest the signed leading digit,
+// at most 1024 in magnitude (exact in FP16).
+__device__ __forceinline__ long long fx_digits_wide(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int Ef = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = b & 0xfffffffffffffull;
+  m |= Ef ? (1ull << 52) : 0ull;
+  const int rsh = min(max(1022 + e + 3 - max(Ef, 1), 0), 62);
+  m = (((m << 6) >> rsh) + 1) >> 1;                       // (m << 5) >> rsh, rounded
+  const long long bias = 0x808080808080ll;
+  return (long long)b < 0 ? bias - (long long)m : bias + (long long)m;
+}
+
+// The digits at byte `byte` of two biased words as two FP16 values (low, high).
+__device__ __forceinline__ uint32_t fx_half2(uint32_t w0, uint32_t w1, int byte) {
+  // bytes w0[byte], 0x64, w1[byte], 0x64: 1024 + u in each half (exact in FP16)
+  const uint32_t r =
+      (__byte_perm(w0, w1, byte | ((4 + byte) << 8)) & 0x00ff00ffu) | 0x64006400u;
+  uint32_t o;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(o) : "r"(r), "r"(0x64806480u));   // minus 1152
+  return o;
+}
+
+// Eight values' digits i as 16 bytes (value k in half k).
+__device__ __forceinline__ uint4 fx_pack8(const unsigned long long (&y)[8], int i) {
+  const int byte = 6 - i;
+  uint32_t o[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const uint32_t w0 = byte < 4 ? (uint32_t)y[2 * p] : (uint32_t)(y[2 * p] >> 32);
+    const uint32_t w1 = byte < 4 ? (uint32_t)y[2 * p + 1] : (uint32_t)(y[2 * p + 1] >> 32);
+    o[p] = fx_half2(w0, w1, byte & 3);
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// t 2^k for any k (the exact power of two in one or two steps)
+__device__ __forceinline__ double fx_scale(double t, int k) {
+  if (k >= -960 && k <= 1000)
+    return t * __longlong_as_double((long long)(k + 1023) << 52);
+  return scalbn(t, k);
+}
+
+#define FX_LD16(r, addr)                                                                         \
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "                                         \
+               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"                 \
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),         \
+                 "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),       \
+                 "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])                              \
+               : "r"(addr))
+#define FX_LD8(r, addr)                                                                          \
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"          \
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),         \
+                 "=r"(r[6]), "=r"(r[7])                                                          \
+               : "r"(addr))
+
+// --------------------------------------------------------------------------
+// Column maxima (high words) of the rows each panel sees: cmax[p][c] over the
+// rows [k0, m) of panel p that no earlier panel changes.  A dense matrix: all
+// rows for panel 0 (later panels' maxima come from the update kernel).  A
+// stacked [L^T; C]: panel p's diagonal rows, panel 0 also all rows of C.
+// grid: (columns, row slices); columns from c_first.
+// --------------------------------------------------------------------------
+__global__ void __launch_bounds__(256)
+fx_colmax_kernel(const double *__restrict__ X, int ldx, int r0, int r1, int c_first, int n,
+                 unsigned *__restrict__ cmax) {
+  const int c = c_first + blockIdx.x;
+  if (c >= n) return;
+  const int rows = r1 - r0;
+  const int per = (rows + gridDim.y - 1) / gridDim.y;
+  const int lo = r0 + blockIdx.y * per, hi = min(r1, lo + per);
+  unsigned mx = 0;
+  for (int i = lo + threadIdx.x; i < hi; i += 256) mx = max(mx, fx_hi(X[SLQR_IDX(i, c, ldx)]));
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0 && mx) atomicMax(cmax + c, mx);
+}
+
+// stacked: panel p's rows 64 p .. 64 p + 63 of the top block of `top` rows;
+// upper: of its upper triangle only (the rest is zero and not read)
+__global__ void __launch_bounds__(256)
+fx_colmax_diag_kernel(const double *__restrict__ A, int lda, int n, int top, int upper,
+                      unsigned *__restrict__ cmax) {
+  const int p = blockIdx.y, c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= n) return;
+  unsigned mx = 0;
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const int r = p * 64 + lane + 32 * t;
+    if (r < top && (!upper || r <= c)) mx = max(mx, fx_hi(A[SLQR_IDX(r, c, lda)]));
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0 && mx) atomicMax(cmax + (size_t)p * n + c, mx);
+}
+
+// --------------------------------------------------------------------------
+// Digits of the panel's V: both images and the row exponents of the second.
+// Reflector a is scaled by its pivot entry: |up| >= the norm of the tail, so it
+// is the largest entry, and for a tall panel far above all others.  For V^T X
+// it may therefore stick out of the leading digit by three bits (1024 instead
+// of 128), which leaves the tail 8 times finer steps.  The sums stay exact:
+// the leading digits of one reflector have a 2-norm of at most sqrt(2) 1024,
+// so by Cauchy-Schwarz their absolute sum over 128 rows is at most 128^2, what
+// 128 rows of ordinary digits may have.  For X -= V W' each row is scaled once
+// more by its own largest (scaled) entry.
+// One CTA per 32 rows.  Bound by latency (one pass over M x 64 doubles).
+// --------------------------------------------------------------------------
+__global__ void __launch_bounds__(256)
+fx_vsplit_kernel(const double *__restrict__ A, int lda, const double *__restrict__ Vtop, int k0,
+                 int nbw, int M, int skip, unsigned char *__restrict__ V1,
+                 unsigned char *__restrict__ V2, int *__restrict__ erow) {
+  __shared__ double t[64][33];
+  __shared__ int s_f[64];
+  const int tid = threadIdx.x, i0 = blockIdx.x * 32;
+  {
+    const int r = tid & 31, i = i0 + r;
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int a = (tid >> 5) + 8 * u;
+      v[u] = 0.0;
+      if (i < M && a < nbw)
+        v[u] = (i < nbw) ? Vtop[i + a * 64] : A[SLQR_IDX(k0 + skip + i, k0 + a, lda)];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[(tid >> 5) + 8 * u][r] = v[u];
+  }
+  if (tid < 64) {
+    const double up = Vtop[tid * 65];
+    // a skipped reflector (up = 0) takes no part: all digits zero
+    s_f[tid] = (up == 0.0) ? kFxNonFinite : fx_exp_of_hi(fx_hi(up));
+  }
+  __syncthreads();
+  {
+    const int a = tid >> 2, rg = tid & 3;
+    const int f = s_f[a];
+    unsigned long long y[8];
+    __align__(16) __half lead[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const long long v = fx_digits_wide(f == kFxNonFinite ? 0.0 : t[a][rg * 8 + k], f - 3);
+      y[k] = (unsigned long long)v;
+      lead[k] = __int2half_rn((int)(v >> 48));
+    }
+    unsigned char *dst = V1 + (size_t)blockIdx.x * kFxV1Chunk + a * 64 +
+                         ((rg * 16) ^ (((a >> 1) & 3) << 4));
+    *(uint4 *)dst = *(const uint4 *)lead;
+#pragma unroll
+    for (int i = 1; i < kFxD; ++i) *(uint4 *)(dst + i * 4096) = fx_pack8(y, i);
+  }
+  {
+    const int r = tid >> 3, ag = tid & 7;
+    int key = kFxZero;
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int f = s_f[ag * 8 + k];
+      v[k] = f == kFxNonFinite ? 0.0 : t[ag * 8 + k][r];
+      const int kk = fx_key(v[k], 0);
+      if (kk != kFxZero) key = max(key, kk - f * (1 << 20));
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+    const int e = (key == kFxZero) ? 0 : fx_exp(key);
+    unsigned long long y[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int f = s_f[ag * 8 + k];
+      y[k] = fx_digits(v[k], (f == kFxNonFinite ? 0 : f) + e);
+    }
+    const int rr = (i0 + r) & 127;
+    unsigned char *dst = V2 + (size_t)((i0 + r) >> 7) * kFxV2Tile + rr * 128 +
+                         ((ag * 16) ^ ((rr & 7) << 4));
+#pragma unroll
+    for (int i = 0; i < kFxD; ++i) *(uint4 *)(dst + i * 16384) = fx_pack8(y, i);
+    if (ag == 0) erow[i0 + r] = e;
+  }
+}
+
+// --------------------------------------------------------------------------
+// W_part[s][c][a] = sum over the rows i of slice s of X(i, c) V(i, a):
+// 128 columns of X on the M side, the digits of the 64 reflectors stacked on
+// the N side, 32 rows per stage.  X is read as FP64 and split here (a thread
+// owns 8 consecutive rows of a column); V's digits come by bulk copy.  Every
+// 128 rows the eight accumulators are drained into 96-bit integer totals.
+// grid: (ceil(N / 128), S), slices of RS rows (a multiple of 128).
+// --------------------------------------------------------------------------
+__global__ void __launch_bounds__(kFxThreads, 1)
+fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M, int N,
+              int RS, const unsigned char *__restrict__ V1, const double *__restrict__ Vtop,
+              const unsigned *__restrict__ cmax, double *__restrict__ Wp, int *status) {
+  extern __shared__ __align__(1024) unsigned char fx_smem_raw[];
+  unsigned char *base = (unsigned char *)(((uintptr_t)fx_smem_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ uint32_t s_taddr;
+  __shared__ __align__(8) uint64_t s_full[2], s_empty[2];
+  __shared__ int s_fa[64];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c0 = blockIdx.x * 128, s = blockIdx.y;
+  const int i_begin = s * RS, i_end = min(M, i_begin + RS);
+  const int T = (i_end - i_begin + 31) / 32;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+                 :: "r"(smem_u32(&s_taddr)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    for (int st = 0; st < 2; ++st) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_full[st])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_empty[st])));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (tid < 64) {
+    const double up = Vtop[tid * 65];
+    s_fa[tid] = (fx_hi(up) >= 0x7ff00000u) ? kFxNonFinite : fx_exp_of_hi(fx_hi(up)) - 3;
+  }
+  // the splitting thread's column and group of 8 rows, and its column's exponent
+  const int sc = tid >> 2, rg = tid & 3;
+  const bool col_ok = c0 + sc < N;
+  const unsigned scm = col_ok ? cmax[c0 + sc] : 0u;
+  const int se = fx_exp_of_hi(scm);
+  const double *xcol = X + (size_t)(c0 + (col_ok ? sc : 0)) * ldx;
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t taddr = s_taddr;
+
+  auto load_v = [&](int t) {
+    fx_bulk(smem_u32(base + (t & 1) * kFxStage + kFxXStage),
+            V1 + (size_t)(i_begin / 32 + t) * kFxV1Chunk, kFxV1Chunk, &s_full[t & 1]);
+  };
+  double xv[8];
+  auto load_x = [&](int t) {
+    const int i = i_begin + t * 32 + rg * 8;
+    const double *p = xcol + k0 + i + (i >= nbw ? skip : 0);
+    const bool whole = i + 8 <= i_end && (i >= nbw || i + 8 <= nbw || skip == 0);
+    if (col_ok && whole) {
+      if ((((uintptr_t)p) & 15) == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+          const double2 v = *(const double2 *)(p + k);
+          xv[k] = v.x;
+          xv[k + 1] = v.y;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) xv[k] = p[k];
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int ii = i + k;
+        xv[k] = (col_ok && ii < i_end) ? xcol[k0 + ii + (ii >= nbw ? skip : 0)] : 0.0;
+      }
+    }
+  };
+  int issued = 0;                                       // V copies (thread 0)
+  if (tid == 0)
+    for (; issued < T && issued < 2; ++issued) load_v(issued);
+  load_x(0);
+
+  // drain mapping: TMEM lane = column of X, this thread's 16 reflectors
+  const int dq = warp & 3, dh = warp >> 2;
+  long long hi[16], lo[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) hi[k] = lo[k] = 0;
+  bool ok = true;
+  for (int t = 0; t < T; ++t) {
+    const int st = t & 1;
+    unsigned char *Xs = base + st * kFxStage;
+    if (t >= 2) {                                       // the MMAs of chunk t - 2 are done
+      ok = mbar_wait(smem_u32(&s_empty[st]), (uint32_t)((t / 2 - 1) & 1));
+      if (tid == 0 && ok) { load_v(t); ++issued; }
+    }
+    {
+      unsigned long long y[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) y[k] = fx_digits(xv[k], se);
+      unsigned char *dst = Xs + sc * 64 + ((rg * 16) ^ (((sc >> 1) & 3) << 4));
+#pragma unroll
+      for (int i = 0; i < kFxD; ++i) *(uint4 *)(dst + i * 8192) = fx_pack8(y, i);
+    }
+    if (t + 1 < T) load_x(t + 1);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (!__syncthreads_and(ok)) { ok = false; break; }
+    if (tid == 0) {
+      // (a copy that never lands leaves the wait for these MMAs to run out)
+      if (mbar_wait(smem_u32(&s_full[st]), (uint32_t)((t >> 1) & 1))) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t xa = smem_u32(Xs), vb = xa + kFxXStage;
+        const bool fresh = (t & 3) == 0;
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          const bool acc = !(fresh && ks == 0);
+          // digit i of X times the stacked digits 0 .. min(6, 7 - i) of V, in
+          // pieces of at most 256 columns; the last 64 of i = 1 open order 7
+          auto piece = [&](int i, int n0, int n, bool ac) {
+            fx_mma(taddr + (uint32_t)(i * 64 + n0), sw64_desc(xa + i * 8192 + ks * 32),
+                   sw64_desc(vb + n0 * 64 + ks * 32), n, ac);
+          };
+          piece(0, 0, 256, acc);   piece(0, 256, 192, acc);
+          piece(1, 0, 256, true);  piece(1, 256, 128, true); piece(1, 384, 64, acc);
+          piece(2, 0, 192, true);  piece(2, 192, 192, true);
+          piece(3, 0, 160, true);  piece(3, 160, 160, true);
+          piece(4, 0, 256, true);
+          piece(5, 0, 192, true);
+          piece(6, 0, 128, true);
+        }
+        fx_commit(&s_empty[st]);
+      }
+    }
+    if ((t & 3) == 3 || t == T - 1) {                   // drain
+      ok = mbar_wait(smem_u32(&s_empty[st]), (uint32_t)((t >> 1) & 1));
+      ok = __all_sync(0xffffffffu, ok);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (ok) {
+#pragma unroll
+        for (int o = 0; o < kFxOrders; ++o) {
+          uint32_t r[16];
+          FX_LD16(r, taddr + ((uint32_t)(dq * 32) << 16) + (uint32_t)(o * 64 + dh * 16));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          const int w = 1 << (8 * (3 - (o & 3)));
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const long long v = (long long)__float2int_rn(__uint_as_float(r[k])) * w;
+            if (o < 4) hi[k] += v;
+            else lo[k] += v;
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (!__syncthreads_and(ok)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    }
+  }
+  if (!ok && tid == 0) {
+    for (int t = max(0, issued - 2); t < issued; ++t)   // let the copies in flight land
+      mbar_wait(smem_u32(&s_full[t & 1]), (uint32_t)((t >> 1) & 1));
+    atomicCAS(status, 0, SLQR_ETIMEOUT);
+  }
+  const int c = c0 + dq * 32 + lane;
+  if (ok && c < N) {
+    const unsigned cm = cmax[c];
+    const int e = fx_exp_of_hi(cm);
+    double *out = Wp + ((size_t)s * N + c) * 64 + dh * 16;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const int f = s_fa[dh * 16 + k];
+      // (hi 2^32 + lo) 2^40 in units of 2^(e-55) 2^(f-55)
+      double v = fma((double)hi[k], 4294967296.0, (double)lo[k]);
+      v = (cm >= 0x7ff00000u || f == kFxNonFinite) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                   : fx_scale(v, e + f - 70);
+      out[k] = v;
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(taddr));
+}
+
+// --------------------------------------------------------------------------
+// W' = T^T W from the partials (the substitution of tw_kernel in factor.cu),
+// written as the digit image of X -= V W': column c scaled by the largest
+// |W'(a, c)| 2^(f_a), f_a the exponent of reflector a.  One warp per column.
+// --------------------------------------------------------------------------
+template <int COLS>
+__global__ void __launch_bounds__(256)
+fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restrict__ wy, int nbw,
+             unsigned char *__restrict__ Wimg, int *__restrict__ ecol) {
+  constexpr int NB = 64, GLD = NB + 1;
+  constexpr int TPE = 256 / (COLS * NB);
+  __shared__ double w[COLS][NB];
+  __shared__ double part[TPE][COLS * NB];
+  __shared__ double G[NB * GLD];
+  __shared__ double tau[NB];
+  __shared__ int s_f[NB];
+  const int tid = threadIdx.x;
+  {
+    double gv[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) gv[u] = wy[(size_t)NB * NB + tid + u * 256];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int idx = tid + u * 256;
+      G[(idx % NB) * GLD + idx / NB] = gv[u];
+    }
+  }
+  if (tid < NB) {
+    tau[tid] = wy[2 * (size_t)NB * NB + tid];
+    const double up = wy[tid * 65];
+    s_f[tid] = up == 0.0 ? 0 : fx_exp_of_hi(fx_hi(up));
+  }
+  const int c0 = blockIdx.x * COLS;
+  {
+    const int e = tid % (COLS * NB), h = tid / (COLS * NB);
+    const int c = e / NB, a = e - c * NB;
+    double acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
+    if (c0 + c < N) {
+      const double *src = Wp + (size_t)(c0 + c) * NB + a;
+      const size_t stride = (size_t)N * NB;
+      int s = h;
+      for (; s + 3 * TPE < S; s += 4 * TPE) {
+        acc0 += src[(size_t)s * stride];
+        acc1 += src[(size_t)(s + TPE) * stride];
+        acc2 += src[(size_t)(s + 2 * TPE) * stride];
+        acc3 += src[(size_t)(s + 3 * TPE) * stride];
+      }
+      for (; s < S; s += TPE) acc0 += src[(size_t)s * stride];
+    }
+    part[h][e] = (acc0 + acc1) + (acc2 + acc3);
+  }
+  __syncthreads();
+  if (tid < COLS * NB) {
+    double v = part[0][tid];
+#pragma unroll
+    for (int h = 1; h < TPE; ++h) v += part[h][tid];
+    w[tid / NB][tid % NB] = v;
+  }
+  __syncthreads();
+  const int warp = tid >> 5, lane = tid & 31;
+  if (warp >= COLS || c0 + warp >= N) return;
+  const int c = c0 + warp;
+  double r0 = w[warp][lane], r1 = w[warp][lane + 32];
+  for (int j = 0; j < nbw; ++j) {
+    const double wj = __shfl_sync(0xffffffffu, (j < 32) ? r0 : r1, j & 31);
+    const double wpj = tau[j] * wj;
+    if (lane > j) r0 = fma(-G[j * GLD + lane], wpj, r0);
+    if (lane + 32 > j) r1 = fma(-G[j * GLD + lane + 32], wpj, r1);
+    if (lane == (j & 31)) {
+      if (j < 32) r0 = wpj;
+      else r1 = wpj;
+    }
+  }
+  if (lane >= nbw) r0 = 0.0;
+  if (lane + 32 >= nbw) r1 = 0.0;
+  const int f0 = s_f[lane], f1 = s_f[lane + 32];
+  int key = max(fx_key(r0, f0), fx_key(r1, f1));
+  key = __reduce_max_sync(0xffffffffu, key);
+  const bool bad = __any_sync(0xffffffffu, fx_hi(r0) >= 0x7ff00000u || fx_hi(r1) >= 0x7ff00000u);
+  const int g = (key == kFxZero) ? 0 : fx_exp(key);
+  unsigned char *dst = Wimg + (size_t)(c >> 5) * kFxWTile + (c & 31) * 128;
+  const unsigned long long y0 = fx_digits(r0, g - f0), y1 = fx_digits(r1, g - f1);
+  const int sw = (c & 7) << 4;
+#pragma unroll
+  for (int i = 0; i < kFxD; ++i) {
+    const int b = 8 * (6 - i);
+    const uint32_t v = fx_half2((uint32_t)(y0 >> b) & 0xff, (uint32_t)(y1 >> b) & 0xff, 0);
+    *(unsigned short *)(dst + i * 4096 + ((lane * 2) ^ sw)) = (unsigned short)(v & 0xffff);
+    *(unsigned short *)(dst + i * 4096 + ((64 + lane * 2) ^ sw)) = (unsigned short)(v >> 16);
+  }
+  if (lane == 0) ecol[c] = bad ? kFxNonFinite : g;
+}
+
+// --------------------------------------------------------------------------
+// X(i, c) -= sum_a V(i, a) W'(a, c): a CTA keeps the digits of 128 rows of V
+// and goes through `per` tiles of 32 columns, the MMAs of the next tile running
+// behind the reassembly of this one (two sets of eight 32-column accumulators
+// fill tensor memory).  A thread owns one row and 8 columns of a tile: TMEM
+// lane = row, so X is read and written in 256-byte runs.  The new values'
+// column maxima (rows >= 64, those of the next panel) go to cnext.
+// grid: (ceil(M / 128), groups of `per` tiles)
+// --------------------------------------------------------------------------
+__global__ void __launch_bounds__(kFxThreads, 1)
+fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M, int N, int per,
+              const unsigned char *__restrict__ V2, const int *__restrict__ erow,
+              const unsigned char *__restrict__ Wimg, const int *__restrict__ ecol,
+              unsigned *__restrict__ cnext, int *status) {
+  extern __shared__ __align__(1024) unsigned char fx_smem_raw[];
+  unsigned char *base = (unsigned char *)(((uintptr_t)fx_smem_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char *Ws = base + kFxV2Tile;
+  __shared__ uint32_t s_taddr;
+  __shared__ __align__(8) uint64_t s_vfull, s_wfull[2], s_mma[2];
+  __shared__ unsigned s_cm[2][32];
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ntiles = (N + 31) / 32;
+  const int t_begin = blockIdx.y * per, T = min(ntiles, t_begin + per) - t_begin;
+  const int i0 = blockIdx.x * 128;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+                 :: "r"(smem_u32(&s_taddr)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_vfull)));
+    for (int st = 0; st < 2; ++st) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_wfull[st])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_mma[st])));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    s_ok = 1;
+  }
+  if (tid < 64) s_cm[tid >> 5][tid & 31] = 0;
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t taddr = s_taddr;
+
+  int issued = 0;                                        // W' copies (thread 0)
+  auto load_w = [&](int t) {
+    fx_bulk(smem_u32(Ws + (t & 1) * kFxWTile), Wimg + (size_t)(t_begin + t) * kFxWTile, kFxWTile,
+            &s_wfull[t & 1]);
+    ++issued;
+  };
+  auto mma_tile = [&](int t) {                           // thread 0
+    const int st = t & 1;
+    if (!mbar_wait(smem_u32(&s_wfull[st]), (uint32_t)((t >> 1) & 1))) {
+      s_ok = 0;
+      return;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t va = smem_u32(base), wb = smem_u32(Ws + st * kFxWTile);
+    const uint32_t acc0 = taddr + (uint32_t)(st * 256);
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      auto piece = [&](int i, int n0, int n, bool ac) {
+        fx_mma(acc0 + (uint32_t)(i * 32 + n0), sw128_desc(va + i * 16384 + ks * 32),
+               sw128_desc(wb + n0 * 128 + ks * 32), n, ac);
+      };
+      piece(0, 0, 224, ks > 0);
+      piece(1, 0, 192, true); piece(1, 192, 32, ks > 0);
+      piece(2, 0, 192, true);
+      piece(3, 0, 160, true);
+      piece(4, 0, 128, true);
+      piece(5, 0, 96, true);
+      piece(6, 0, 64, true);
+    }
+    fx_commit(&s_mma[st]);
+  };
+  if (tid == 0) {
+    fx_bulk(smem_u32(base), V2 + (size_t)blockIdx.x * kFxV2Tile, kFxV2Tile, &s_vfull);
+    load_w(0);
+    if (T > 1) load_w(1);
+    if (!mbar_wait(smem_u32(&s_vfull), 0)) s_ok = 0;
+    else mma_tile(0);
+  }
+  // this thread's row of the tile and its 8 columns
+  const int q = warp & 3, h = warp >> 2;
+  const int i = i0 + q * 32 + lane;
+  const bool row_ok = i < M;
+  const int er = erow[i];                                // (defined up to the whole tile)
+  double *xrow = X + k0 + i + (i >= nbw ? skip : 0);
+  const bool next_row = row_ok && i >= 64;
+  bool ok = true;
+  for (int t = 0; t < T; ++t) {
+    const int buf = t & 1;
+    const int cb = (t_begin + t) * 32 + h * 8;
+    double x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      x[k] = (row_ok && cb + k < N) ? xrow[(size_t)(cb + k) * ldx] : 0.0;
+    if (tid == 0 && t + 1 < T) mma_tile(t + 1);
+    ok = mbar_wait(smem_u32(&s_mma[buf]), (uint32_t)((t >> 1) & 1));
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (tid == 0 && ok && t + 2 < T) load_w(t + 2);       // this tile's W' has been read
+    if (tid < 32 && t > 0) {                              // maxima of the tile before
+      const unsigned v = s_cm[buf ^ 1][tid];
+      const int c = (t_begin + t - 1) * 32 + tid;
+      if (cnext && v && c < N) atomicMax(cnext + c, v);
+      s_cm[buf ^ 1][tid] = 0;
+    }
+    ok = __all_sync(0xffffffffu, ok);                     // (converged for tcgen05.ld)
+    if (ok) {
+      long long hi[8], lo[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) hi[k] = lo[k] = 0;
+#pragma unroll
+      for (int o = 0; o < kFxOrders; ++o) {
+        uint32_t r[8];
+        FX_LD8(r, taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + o * 32 + h * 8));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        const int w = 1 << (8 * (3 - (o & 3)));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const long long v = (long long)__float2int_rn(__uint_as_float(r[k])) * w;
+          if (o < 4) hi[k] += v;
+          else lo[k] += v;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int c = cb + k;
+        const int g = (c < N) ? ecol[c] : 0;
+        // sum = (hi 2^72 + lo 2^40) 2^(er + g - 110), kept to 2^54 of those
+        // units in 63 bits: |hi| < 2^45 (the leading order sums 64 products)
+        const long long tt = (hi[k] << 18) + ((lo[k] + (1 << 13)) >> 14);
+        const int sh = er + g - 56;
+        double v;
+        if (sh >= -1000 && sh <= 900)
+          v = fma(-__longlong_as_double((long long)(sh + 1023) << 52), (double)tt, x[k]);
+        else
+          v = g == kFxNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                : x[k] - scalbn((double)tt, sh);
+        x[k] = v;
+      }
+      unsigned mine = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (row_ok && cb + k < N) xrow[(size_t)(cb + k) * ldx] = x[k];
+        const unsigned mx = __reduce_max_sync(0xffffffffu, next_row ? fx_hi(x[k]) : 0u);
+        if (lane == k) mine = mx;
+      }
+      if (lane < 8 && mine) atomicMax(&s_cm[buf][h * 8 + lane], mine);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (!__syncthreads_and(ok && s_ok)) { ok = false; break; }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  if (ok && tid < 32 && T > 0) {
+    const unsigned v = s_cm[(T - 1) & 1][tid];
+    const int c = (t_begin + T - 1) * 32 + tid;
+    if (cnext && v && c < N) atomicMax(cnext + c, v);
+  }
+  if (!ok && tid == 0) {
+    mbar_wait(smem_u32(&s_vfull), 0);                     // let the copies in flight land
+    for (int t = max(0, issued - 2); t < issued; ++t)
+      mbar_wait(smem_u32(&s_wfull[t & 1]), (uint32_t)((t >> 1) & 1));
+    atomicCAS(status, 0, SLQR_ETIMEOUT);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(taddr));
+}
+
+// --------------------------------------------------------------------------
+// host side
+// --------------------------------------------------------------------------
+slqr_status init_fx_attrs(slqr_ctx *ctx) {
+  cudaError_t e = cudaFuncSetAttribute(fx_vtx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kFxVtxSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fx_upd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kFxUpdSmem);
+  if (e != cudaSuccess)
+    return fail(ctx, SLQR_ECUDA, "cudaFuncSetAttribute(fp64 tc): %s", cudaGetErrorString(e));
+  return SLQR_OK;
+}
+
+static int fx_slices(int M, int N, int num_sms, int *RS) {
+  // few column tiles: one wave of CTAs (a CTA has an SM to itself); more: about
+  // four, so that the last one is a small part
+  const int tiles = (N + 127) / 128, blocks = (M + 127) / 128;
+  const int want = tiles <= num_sms / 8 ? num_sms / tiles : (4 * num_sms + tiles - 1) / tiles;
+  const int S = std::max(1, std::min(blocks, want));
+  *RS = (blocks + S - 1) / S * 128;
+  return (M + *RS - 1) / *RS;
+}
+
+size_t fx_v_bytes(int m) {
+  const size_t tiles = ((size_t)m + 127) / 128;
+  return tiles * (4 * (size_t)kFxV1Chunk + kFxV2Tile) + align_up(tiles * 128 * sizeof(int), 256);
+}
+
+size_t fx_work_bytes(int m, int n, int num_sms) {
+  // partials: S N' <= (4 num_sms + tiles') 128 over every width N' <= n (fx_slices)
+  (void)m;
+  const size_t part = ((size_t)4 * num_sms + 2) * 128 + (size_t)n;
+  const size_t tiles = ((size_t)n + 31) / 32;
+  return align_up(part * 64 * sizeof(double), 256) + tiles * kFxWTile +
+         align_up(tiles * 32 * sizeof(int), 256);
+}
+
+void fx_split_v(const double *A, int lda, const double *Vtop, int k0, int nbw, int M, int skip,
+                void *vbuf, cudaStream_t stream) {
+  const size_t tiles = ((size_t)M + 127) / 128;
+  unsigned char *V1 = (unsigned char *)vbuf, *V2 = V1 + tiles * 4 * kFxV1Chunk;
+  int *erow = (int *)(V2 + tiles * kFxV2Tile);
+  fx_vsplit_kernel<<<(unsigned)(tiles * 4), 256, 0, stream>>>(A, lda, Vtop, k0, nbw, M, skip, V1,
+                                                              V2, erow);
+}
+
+bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy_panel,
+               const void *vbuf, double *X, int ldx, int N, const unsigned *cmax, unsigned *cnext,
+               void *work, size_t work_bytes, cudaStream_t stream) {
+  int RS = 0;
+  const int S = fx_slices(M, N, ctx->num_sms, &RS);
+  const size_t tiles = ((size_t)M + 127) / 128, wt = ((size_t)N + 31) / 32;
+  const size_t part = align_up((size_t)S * N * 64 * sizeof(double), 256);
+  if (part + wt * kFxWTile + wt * 32 * sizeof(int) > work_bytes) return false;
+  const unsigned char *V1 = (const unsigned char *)vbuf, *V2 = V1 + tiles * 4 * kFxV1Chunk;
+  const int *erow = (const int *)(V2 + tiles * kFxV2Tile);
+  double *Wp = (double *)work;
+  unsigned char *Wimg = (unsigned char *)work + part;
+  int *ecol = (int *)(Wimg + wt * kFxWTile);
+  const double flops = 2.0 * M * nbw * (double)N;
+  int slot = prof_begin(ctx, stream);
+  fx_vtx_kernel<<<dim3((N + 127) / 128, S), kFxThreads, kFxVtxSmem, stream>>>(
+      X, ldx, k0, nbw, skip, M, N, RS, V1, wy_panel, cmax, Wp, ctx->d_status);
+  prof_end(ctx, stream, slot, kVtx, flops);
+  slot = prof_begin(ctx, stream);
+  if (N <= 4 * ctx->num_sms)
+    fx_tw_kernel<1><<<N, 256, 0, stream>>>(Wp, S, N, wy_panel, nbw, Wimg, ecol);
+  else
+    fx_tw_kernel<4><<<(N + 3) / 4, 256, 0, stream>>>(Wp, S, N, wy_panel, nbw, Wimg, ecol);
+  prof_end(ctx, stream, slot, kTw, (double)nbw * nbw * N);
+  slot = prof_begin(ctx, stream);
+  const int rt = (M + 127) / 128;
+  // column tiles per CTA: about four waves of CTAs, at least 4 tiles each (the
+  // V tile is 114 KB, as much as 3.5 tiles of X)
+  const int groups = std::max(1, (4 * ctx->num_sms + rt - 1) / rt);
+  const int per = std::max(rt * (int)wt <= ctx->num_sms ? 1 : 4, ((int)wt + groups - 1) / groups);
+  fx_upd_kernel<<<dim3(rt, ((int)wt + per - 1) / per), kFxThreads, kFxUpdSmem, stream>>>(
+      X, ldx, k0, nbw, skip, M, N, per, V2, erow, Wimg, ecol, cnext, ctx->d_status);
+  prof_end(ctx, stream, slot, kUpd, flops);
+  return true;
+}
+
+void fx_colmax(const double *X, int ldx, int m, int n, int stacked_top, bool upper, unsigned *cmax,
+               int np, int num_sms, cudaStream_t stream) {
+  cudaMemsetAsync(cmax, 0, (size_t)np * n * sizeof(unsigned), stream);
+  const int r0 = stacked_top;                     // dense: 0; stacked: the rows of C
+  if (m > r0) {
+    const int sl = std::max(1, std::min((m - r0 + 1023) / 1024, (8 * num_sms + n - 1) / n));
+    fx_colmax_kernel<<<dim3(n, sl), 256, 0, stream>>>(X, ldx, r0, m, 0, n, cmax);
+  }
+  if (stacked_top > 0)
+    fx_colmax_diag_kernel<<<dim3((n + 7) / 8, np), 256, 0, stream>>>(X, ldx, n, stacked_top, upper,
+                                                                    cmax);
+}
+
+}  // namespace slqr

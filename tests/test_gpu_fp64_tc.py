@@ -1,0 +1,104 @@
+"""The FP64 trailing update and Q^T B on the tensor cores by exact splitting
+(csrc/tc_fp64.cu; panels of 64 reflectors, at least 16 columns) against the
+CPU oracle, at the edges of its tiles (128 rows, 32 and 128 columns, 32-row
+chunks), and against the FP64-pipe kernels, which a context takes whose budget
+does not hold the digit images, also where values are not finite.  Tolerances are those of tests/test_gpu_parity.py.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads
+from test_gpu_parity import U, check_against_oracle, dev, factor_tol, host, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_2506_09463_gb300 import api
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+# (rows, columns, padding of the leading dimension): trailing widths of 16, 17,
+# 31..33 and 127..129 columns, row counts around multiples of 32 and 128, odd
+# leading dimensions (8-byte loads)
+SHAPES = [(337, 336, 0), (384, 273, 0), (385, 287, 1), (513, 289, 0), (449, 449, 3),
+          (640, 320, 0), (641, 383, 1), (1023, 385, 0), (1155, 271, 2)]
+
+
+@pytest.mark.parametrize("m,n,pad", SHAPES)
+def test_factor_at_tile_edges(ctx, m, n, pad):
+    A, b = workloads.gaussian(m, n, seed=m + n)
+    F, up, qtb, x, st = run_gpu(ctx, A, b, lda_pad=pad)
+    assert st == 0
+    check_against_oracle(A, b, F, up, qtb, x)
+
+
+@pytest.mark.parametrize("nrhs", [15, 16, 17, 33, 64, 130])
+@pytest.mark.parametrize("stacked", [False, True])
+def test_apply_qt_blocks(ctx, nrhs, stacked):
+    if stacked:
+        n, m = 300, 450
+        A, _ = workloads.slsqp_stack(n, m - n, seed=nrhs)
+    else:
+        m, n = 461, 300
+        A, _ = workloads.gaussian(m, n, seed=nrhs)
+    B = workloads.gaussian_rhs(m, nrhs, seed=nrhs)
+    Ad, Bd = dev(A), dev(B)
+    up = torch.empty(n, dtype=torch.float64, device="cuda")
+    wy = ctx.wy_buffer(m, n)
+    (ctx.factor_stacked if stacked else ctx.factor)(Ad, up, wy)
+    (ctx.apply_qt_stacked if stacked else ctx.apply_qt)(Ad, up, Bd, wy=wy)
+    assert ctx.sync() == 0
+    Fo, upo, _ = oracle.h12_factor(A)
+    _, kappa = factor_tol(A)
+    out = host(Bd)
+    for j in range(nrhs):
+        want = oracle.apply_qt(Fo, upo, np.ascontiguousarray(B[:, j]))
+        np.testing.assert_allclose(out[:, j], want, rtol=0,
+                                   atol=4.0 * np.sqrt(m) * U * kappa * np.linalg.norm(B[:, j]))
+
+
+def test_columns_of_any_scale(ctx):
+    """Powers of two per column are exact: the factorization of A D is F D."""
+    m, n = 500, 360
+    A, b = workloads.gaussian(m, n, seed=5)
+    e = np.random.default_rng(6).integers(-450, 451, size=n)
+    F, up, _, _, st = run_gpu(ctx, A, b)
+    assert st == 0
+    G, upg, _, _, st = run_gpu(ctx, np.ldexp(A, e[None, :]), b)
+    assert st == 0
+    tol, _ = factor_tol(A)
+    np.testing.assert_allclose(np.ldexp(G, -e[None, :]), F, rtol=0, atol=tol)
+    np.testing.assert_allclose(np.ldexp(upg, -e), up, rtol=0, atol=tol)
+
+
+# a budget that holds the workspace of the FP64-pipe kernels (68 MB) but not the
+# digit images of 20,000 rows (120 MB in all)
+PIPE_BUDGET = 90 << 20
+
+
+@pytest.mark.parametrize("value", [None, np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("row,col", [(3, 130), (19000, 70), (19000, 10)])
+def test_same_as_the_fp64_pipe(ctx, value, row, col):
+    """Over the budget every update stays on the FP64 pipe: the same values to
+    the parity tolerance, and not finite in the same places."""
+    from paper_2506_09463_gb300 import api
+    m, n = 20000, 300
+    A, b = workloads.gaussian(m, n, seed=8)
+    A = np.array(A)
+    if value is not None:
+        A[row, col] = value
+    F, up, _, _, _ = run_gpu(ctx, A, b)
+    with api.Context(0, hbm_budget_bytes=PIPE_BUDGET) as pipe:
+        G, upg, _, _, _ = run_gpu(pipe, A, b)
+    np.testing.assert_array_equal(np.isfinite(up), np.isfinite(upg))
+    np.testing.assert_array_equal(np.isfinite(F), np.isfinite(G))
+    if value is None:
+        tol, _ = factor_tol(A)
+        np.testing.assert_allclose(F, G, rtol=0, atol=tol)
+        assert not np.array_equal(F, G)          # (the two paths round differently)
