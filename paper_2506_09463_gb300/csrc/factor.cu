@@ -1335,6 +1335,22 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       }
       return SLQR_OK;                             // (no grid barrier used)
     }
+    if constexpr (std::is_same<T, double>::value && NB == 64) {
+      int Pg = 0;
+      const int Rg = grid_panel_rows(ctx, M, rmin, &Pg);
+      if (Rg > 0) {
+        GridPanelParams gp;
+        gp.A = A; gp.up = up; gp.wy = wy_store + (size_t)pnl * wy_panel_doubles(NB);
+        gp.rec = rec; gp.srec = srec; gp.gpart = gpart; gp.prow = prow; gp.bar = bar;
+        gp.status = ctx->d_status; gp.m = m; gp.lda = lda; gp.k0 = k0; gp.nbw = nbw;
+        gp.skip = skip; gp.stacked = ntop > 0; gp.bar_base = bar_base; gp.spin = ctx->spin_limit;
+        int slot = prof_begin(ctx, s);
+        slqr_status gst = launch_grid_panel(ctx, gp, Rg, Pg, s);
+        prof_end(ctx, s, slot, kPanel, pflops);
+        bar_base = gp.bar_base;
+        return gst;
+      }
+    }
     const int R = panel_rows_per_cta(M, nbw, Pmax, max_rows_per_cta(NB, sizeof(T)), rmin,
                                      sizeof(T));
     if (R > max_rows_per_cta(NB, sizeof(T)))

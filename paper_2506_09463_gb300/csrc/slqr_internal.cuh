@@ -79,6 +79,8 @@ struct slqr_ctx {
   // 2: BF16 split in hi + lo, with the BF16 shadows of the matrix below)
   int tc_mode = 0;
   void *sh_hi = nullptr, *sh_lo = nullptr;
+  // CTAs the FP64 grid panel may use, in clusters of 8 and as one cluster
+  int grid_panel_ctas = 0, grid_panel_one = 0;
   // limit of the polled exchanges and grid barriers of the cooperative kernels
   unsigned spin_limit = slqr::kSpinLimit;
   std::string last_error;
@@ -291,6 +293,28 @@ slqr_status launch_cluster_panel(slqr_ctx *ctx, bool f32, int nb, const ClusterP
 // Cluster size of the panel for a panel of M rows (0: the cooperative panel)
 // under the setting of slqr_set_panel_cluster.
 int panel_cluster_ctas(slqr_ctx *ctx, bool f32, int nb, int M, int nbw);
+
+// The FP64 panel of 64 columns by thread-block clusters with the panel in
+// registers (panel_grid.cu): P CTAs of R rows each.
+struct GridPanelParams {
+  void *A;             // double *, column-major, leading dimension lda
+  double *up;          // global up array
+  double *wy;          // this panel's compact-WY block (Vtop | G | tau)
+  double *rec;         // 64 * 64 * clusters: per column j and entry c the clusters' dots
+  double *srec;        // P * 64: per-CTA column scales (panel start)
+  double *gpart;       // P * 64 * 63 / 2: per-CTA partial Gram terms
+  double *prow;        // 64 * 64: per column j the pivot row
+  unsigned *bar;       // monotonic arrival counter (two arrivals per CTA and panel)
+  int *status;
+  int m, lda, k0, nbw;
+  int skip, stacked;   // as ClusterPanelParams
+  unsigned bar_base;   // counter value when this panel starts; advanced by the launch
+  unsigned spin;       // polls of a bounded wait before it reports
+};
+slqr_status init_grid_panel_attrs(slqr_ctx *ctx);
+// rows per CTA (0: no grid panel) and CTAs for a panel of M rows; rows_min 0: chosen
+int grid_panel_rows(const slqr_ctx *ctx, int M, int rows_min, int *ctas);
+slqr_status launch_grid_panel(slqr_ctx *ctx, GridPanelParams &p, int R, int P, cudaStream_t stream);
 
 // Look-ahead update of the next panel's columns (at most 64) of an FP32
 // factorization with panels of width 64, in one cooperative launch
