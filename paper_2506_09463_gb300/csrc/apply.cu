@@ -141,9 +141,11 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
   bool fx = NB == 64 && nrhs >= kFxMinCols;
   const size_t fx_v = align_up(fx_v_bytes(m), 256);
   const size_t fx_work = align_up(fx_work_bytes(m, nrhs, ctx->num_sms), 256);
+  const size_t fx_gt = (size_t)np * kFxGt * sizeof(double);
   slqr_status st = SLQR_OK;
   if (fx) {
-    st = ensure_workspace(ctx, head_bytes + fx_v + fx_work + (size_t)np * nrhs * sizeof(unsigned));
+    st = ensure_workspace(ctx, head_bytes + fx_v + fx_work + fx_gt +
+                                   (size_t)np * nrhs * sizeof(unsigned));
     if (st == SLQR_EBUSY || st == SLQR_ENOMEM) fx = false;
     else if (st != SLQR_OK) return st;
   }
@@ -154,7 +156,8 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
   double *Gp = base + wy_doubles;
   char *tail = (char *)base + head_bytes;
   double *work = (double *)tail;
-  unsigned *cmax = (unsigned *)(tail + fx_v + fx_work);
+  double *gt = (double *)(tail + fx_v + fx_work);
+  unsigned *cmax = (unsigned *)(tail + fx_v + fx_work + fx_gt);
   if (!wy) {
     double gflops = 0.0;
     for (int pnl = 0; pnl < np; ++pnl) gflops += 2.0 * (m - pnl * NB) * NB * NB;
@@ -173,6 +176,7 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
   const double *wys = wy ? wy : wy_store;
   if (fx) {
     fx_colmax(B, ldb, m, nrhs, ntop, false, cmax, np, ctx->num_sms, stream);
+    fx_prep(wys, K, NB, gt, stream);
     for (int pnl = 0; pnl < np; ++pnl) {
       const int k0 = pnl * NB, nbw = std::min(NB, K - k0);
       const int skip = ntop > 0 ? ntop - (k0 + nbw) : 0;
@@ -180,7 +184,8 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
       int slot = prof_begin(ctx, stream);
       fx_split_v(A, lda, wyp, k0, nbw, m - k0 - skip, skip, tail, stream);
       prof_end(ctx, stream, slot, kVtx, 0.0);
-      if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip, wyp, tail, B, ldb, nrhs,
+      if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip, wyp, gt + (size_t)pnl * kFxGt,
+                     tail, B, ldb, nrhs,
                      cmax + (size_t)pnl * nrhs,
                      pnl + 1 < np ? cmax + (size_t)(pnl + 1) * nrhs : nullptr, tail + fx_v, fx_work,
                      stream))

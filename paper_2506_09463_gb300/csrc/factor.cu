@@ -1231,10 +1231,26 @@ static size_t panel_smem_bytes(int nb, int R, size_t elem) {
 
 // ntop > 0: A = [L^T; C] with an upper-triangular top block of ntop = n rows
 // (the structure-aware factorization: each panel skips the zero rows between
-// its diagonal block and C).
+// its diagonal block and C).  wy32: compact-WY store in panels of 32 of a
+// factorization in panels of 64 (wy NULL), its blocks on the diagonals of the
+// panels' own.
+__global__ void __launch_bounds__(256)
+wy32_kernel(const double *__restrict__ wy, int K, double *__restrict__ out) {
+  const int p = blockIdx.x, o = (p & 1) * 32;
+  const double *src = wy + (size_t)(p >> 1) * wy_panel_doubles(64);
+  double *dst = out + (size_t)p * wy_panel_doubles(32);
+  for (int idx = threadIdx.x; idx < 32 * 32; idx += 256) {
+    const int c = idx >> 5, r = idx & 31;
+    dst[idx] = src[(o + c) * 64 + o + r];                       // Vtop
+    dst[32 * 32 + idx] = src[64 * 64 + (o + c) * 64 + o + r];   // G
+  }
+  if (threadIdx.x < 32) dst[2 * 32 * 32 + threadIdx.x] = src[2 * 64 * 64 + o + threadIdx.x];
+}
+
 template <typename T, int NB>
 static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, double *up,
-                               double *wy, cudaStream_t stream, int ntop = 0) {
+                               double *wy, cudaStream_t stream, int ntop = 0,
+                               double *wy32 = nullptr) {
   const int K = num_reflectors(m, n);
   auto skip_of = [&](int k0, int nbw) { return ntop > 0 ? ntop - (k0 + nbw) : 0; };
   const int np = num_panels(K, NB);
@@ -1253,21 +1269,24 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
                         (std::is_same<T, float>::value ? (size_t)(m + n) * NB : 0);
   const size_t head_bytes =
       256 + (rec_doubles + srec_doubles + gpart_doubles + prow_doubles + wy_doubles) * 8 + 256;
-  // FP64 updates of at least kFxMinCols columns run on the tensor cores
-  // (tc_fp64.cu) with panels of 64; the digit images of V (of two panels: the
+  // FP64 panels of 64 run on clusters (panel_grid.cu), their Gram terms and
+  // updates of at least kFxMinCols columns on the tensor cores (tc_fp64.cu); the
+  // digit images of V (of two panels: the
   // rest of one update runs beside the next panel), the update's scratch and
   // the column maxima follow the workspace of the FP64-pipe kernels, which
   // narrow updates still use.  Where that does not fit the device or the
   // context's budget, every update stays on the FP64 pipe.
-  bool fx = std::is_same<T, double>::value && NB == 64 && n - NB >= kFxMinCols && np > 1;
+  bool fx = std::is_same<T, double>::value && NB == 64 && np > 0;
   const size_t fx_v = align_up(fx_v_bytes(m), 256);
   const size_t fx_work = align_up(fx_work_bytes(m, n, ctx->num_sms), 256);
   const size_t fx_cm = align_up((size_t)np * n * sizeof(unsigned), 256);
+  const size_t fx_gr = (size_t)np * kFxGramBytes;
+  const size_t fx_gt = 2 * kFxGt * sizeof(double);
   slqr_status st = SLQR_OK;
   if (fx) {
     // (at most m / 64 row slices, see split_count)
     const size_t narrow = ((size_t)std::max(1, m / 64) + 1) * kFxMinCols * NB;
-    const size_t with_fx = head_bytes + align_up(narrow * sizeof(T), 256) + 2 * fx_v + fx_work + fx_cm;
+    const size_t with_fx = head_bytes + align_up(narrow * sizeof(T), 256) + 2 * fx_v + fx_work + fx_cm + fx_gr + fx_gt;
     st = ensure_workspace(ctx, with_fx);
     if (st == SLQR_OK) work_doubles = narrow;
     else if (st == SLQR_EBUSY || st == SLQR_ENOMEM) fx = false;
@@ -1291,6 +1310,8 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   void *vbuf[2] = {fx_base, fx_base + fx_v};
   void *fxw = fx_base + 2 * fx_v;
   unsigned *cmax = (unsigned *)(fx_base + 2 * fx_v + fx_work);   // [panel][column]
+  char *gram_base = fx_base + 2 * fx_v + fx_work + fx_cm;        // per panel
+  double *gt_base = (double *)(gram_base + fx_gr);               // of two panels, as vbuf
 
   cudaError_t e = cudaMemsetAsync(bar, 0, 256, stream);
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
@@ -1336,16 +1357,17 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       return SLQR_OK;                             // (no grid barrier used)
     }
     if constexpr (std::is_same<T, double>::value && NB == 64) {
-      int Pg = 0;
-      const int Rg = grid_panel_rows(ctx, M, rmin, &Pg);
-      if (Rg > 0) {
+      // (the Gram terms of this panel come from the digits of V, so the FP64-pipe
+      // path keeps the panel below)
+      const GridPanelShape shape = fx ? grid_panel_shape(ctx, M, rmin) : GridPanelShape();
+      if (shape.R > 0) {
         GridPanelParams gp;
         gp.A = A; gp.up = up; gp.wy = wy_store + (size_t)pnl * wy_panel_doubles(NB);
-        gp.rec = rec; gp.srec = srec; gp.gpart = gpart; gp.prow = prow; gp.bar = bar;
+        gp.rec = rec; gp.srec = srec; gp.prow = prow; gp.bar = bar;
         gp.status = ctx->d_status; gp.m = m; gp.lda = lda; gp.k0 = k0; gp.nbw = nbw;
         gp.skip = skip; gp.stacked = ntop > 0; gp.bar_base = bar_base; gp.spin = ctx->spin_limit;
         int slot = prof_begin(ctx, s);
-        slqr_status gst = launch_grid_panel(ctx, gp, Rg, Pg, s);
+        slqr_status gst = launch_grid_panel(ctx, gp, shape, s);
         prof_end(ctx, s, slot, kPanel, pflops);
         bar_base = gp.bar_base;
         return gst;
@@ -1381,15 +1403,33 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
     bar_base += 2u * (unsigned)P;                 // two grid barriers per panel
     return SLQR_OK;
   };
-  // digits of the panel's reflectors for its update, right behind the panel
+  // digits of the panel's reflectors for its update, right behind the panel, and
+  // the Gram terms that the grid panel leaves open: in the look-ahead's V^T X
+  // where that runs on the tensor cores, else at once
+  auto on_grid = [&](int pnl) {
+    const int k0 = pnl * NB, nbw = std::min(NB, K - k0);
+    return fx && panel_cluster_ctas(ctx, false, NB, m - k0 - skip_of(k0, nbw), nbw) == 0 &&
+           grid_panel_shape(ctx, m - k0 - skip_of(k0, nbw), rmin).R > 0;
+  };
+  auto gram_in_lookahead = [&](int pnl) {
+    return pnl + 1 < np && std::min(NB, K - (pnl + 1) * NB) >= kFxMinCols;
+  };
+  auto gt_of = [&](int pnl) { return gt_base + (size_t)(pnl & 1) * kFxGt; };
   auto split_v = [&](int pnl, cudaStream_t s) {
     const int k0 = pnl * NB, nbw = std::min(NB, K - k0), skip = skip_of(k0, nbw);
-    if (!fx || n - (k0 + nbw) < kFxMinCols) return;
+    const int trailing = n - (k0 + nbw);
+    const bool gram = on_grid(pnl) && !gram_in_lookahead(pnl) && (wy || wy32 || trailing > 0);
+    if (!fx || (trailing < kFxMinCols && !gram)) return;
     if constexpr (std::is_same<T, double>::value) {
+      double *wyp = wy_store + (size_t)pnl * wy_panel_doubles(NB);
       int slot = prof_begin(ctx, s);
-      fx_split_v(A, lda, wy_store + (size_t)pnl * wy_panel_doubles(NB), k0, nbw, m - k0 - skip, skip,
-                 vbuf[pnl & 1], s);
+      fx_split_v(A, lda, wyp, k0, nbw, m - k0 - skip, skip, vbuf[pnl & 1], s);
       prof_end(ctx, s, slot, kVtx, 0.0);
+      if (gram)
+        fx_gram(ctx, nbw, m - k0 - skip, wyp, vbuf[pnl & 1], gram_base + (size_t)pnl * kFxGramBytes,
+                gt_of(pnl), s);
+      else if (!on_grid(pnl))
+        fx_prep(wyp, nbw, NB, gt_of(pnl), s);
     }
   };
   // the fused look-ahead kernel's grid barriers count on their own counter
@@ -1415,11 +1455,11 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       if (fx && c_end - c_begin >= kFxMinCols) {
         const int skip = skip_of(k0, nbw);
         if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip,
-                       wy_store + (size_t)pnl * wy_panel_doubles(NB), vbuf[pnl & 1],
+                       wy_store + (size_t)pnl * wy_panel_doubles(NB), gt_of(pnl), vbuf[pnl & 1],
                        A + (size_t)c_begin * lda, lda, c_end - c_begin,
                        cmax + (size_t)pnl * n + c_begin,
                        pnl + 1 < np ? cmax + (size_t)(pnl + 1) * n + c_begin : nullptr, fxw, fx_work,
-                       us))
+                       us, lookahead && on_grid(pnl) ? gram_base + (size_t)pnl * kFxGramBytes : nullptr))
           return fail(ctx, SLQR_ENOMEM, "internal: trailing-update workspace too small");
         return check_launch(ctx, "trailing update");
       }
@@ -1434,7 +1474,12 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   if (e == cudaSuccess) e = cudaStreamWaitEvent(aux, ctx->ev_start, 0);
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "event: %s", cudaGetErrorString(e));
   if constexpr (std::is_same<T, double>::value) {
-    if (fx) fx_colmax(A, lda, m, n, ntop, true, cmax, np, ctx->num_sms, stream);
+    if (fx) {
+      fx_colmax(A, lda, m, n, ntop, true, cmax, np, ctx->num_sms, stream);
+      e = cudaMemsetAsync(gram_base, 0, fx_gr, stream);
+      if (e != cudaSuccess)
+        return fail(ctx, SLQR_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    }
   }
   st = launch_panel(0, stream);
   if (st != SLQR_OK) return st;
@@ -1482,6 +1527,7 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       if (st != SLQR_OK) return st;
     }
   }
+  if (wy32) wy32_kernel<<<num_panels(K, 32), 256, 0, stream>>>(wy_store, K, wy32);
   return check_launch(ctx, "factor");
 }
 
@@ -1492,6 +1538,12 @@ slqr_status factor_f32(slqr_ctx *ctx, int m, int n, float *A, int lda, double *u
   return factor_impl<float, 64>(ctx, m, n, A, lda, up, wy, stream, ntop);
 }
 
+
+static slqr_status factor_fp64(slqr_ctx *ctx, int m, int n, double *A, int lda, double *up,
+                               double *wy, cudaStream_t s, int ntop) {
+  if (panel_width(m, n) == 32) return factor_impl<double, 32>(ctx, m, n, A, lda, up, wy, s, ntop);
+  return factor_impl<double, 64>(ctx, m, n, A, lda, up, wy, s, ntop);
+}
 
 }  // namespace slqr
 
@@ -1668,8 +1720,7 @@ extern "C" slqr_status slqr_factor(slqr_ctx *ctx, int m, int n, double *A, int l
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "cudaSetDevice: %s", cudaGetErrorString(e));
   cudaStream_t s = (cudaStream_t)stream;
-  if (panel_width(m, n) == 32) return factor_impl<double, 32>(ctx, m, n, A, lda, up, wy, s);
-  return factor_impl<double, 64>(ctx, m, n, A, lda, up, wy, s);
+  return factor_fp64(ctx, m, n, A, lda, up, wy, s, 0);
 }
 
 extern "C" slqr_status slqr_factor_stacked(slqr_ctx *ctx, int n, int m_eq, double *A, int lda,
@@ -1686,8 +1737,7 @@ extern "C" slqr_status slqr_factor_stacked(slqr_ctx *ctx, int n, int m_eq, doubl
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "cudaSetDevice: %s", cudaGetErrorString(e));
   cudaStream_t s = (cudaStream_t)stream;
-  if (panel_width(m, n) == 32) return factor_impl<double, 32>(ctx, m, n, A, lda, up, wy, s, n);
-  return factor_impl<double, 64>(ctx, m, n, A, lda, up, wy, s, n);
+  return factor_fp64(ctx, m, n, A, lda, up, wy, s, n);
 }
 
 // ==========================================================================

@@ -3,8 +3,9 @@
 //
 // Same arithmetic and outputs as panel_kernel (factor.cu; Alg. 2 of the paper
 // on one panel): the scaled norm, the sign rule and up of Alg. 3, the reflector
-// applied to the later columns; Vtop, the Gram terms of V^T V and tau for the
-// compact-WY update.
+// applied to the later columns; Vtop and tau for the compact-WY update.  The
+// Gram terms of V^T V, a third of the panel's FP64 work there, are formed from
+// the digits of V instead (fx_gram_block in tc_fp64.cu).
 //
 // What bounds a column step: every FP64 warp instruction holds the SM's FP64
 // pipe for 16 clocks, and the step is a chain of two passes over the slice, a
@@ -16,16 +17,13 @@
 //    through shared memory.
 //  * Partial dots go out straight from registers.  Up to 16 CTAs are one
 //    cluster: each warp pushes its columns' partials to every CTA (st.async,
-//    counted on an mbarrier there).  More CTAs are clusters of 8: the partials
-//    of a column go to one CTA of the cluster, which adds the 8 and publishes
-//    the sum in L2, and every warp collects the clusters' sums of its own
-//    columns.  (Without the first level every CTA reads every CTA's record:
+//    counted on an mbarrier there).  More CTAs are clusters of 8 or 4: the
+//    partials of a column go to one CTA of the cluster, which adds them and
+//    publishes the sum in L2, and every warp collects the clusters' sums of its
+//    own columns.  (Without the first level every CTA reads every CTA's record:
 //    128 CTAs spent 3.5 us of a 7.4 us step in those reads.)
 //  * The only CTA barriers of a step are the two that hand over the pivot (from
 //    the warp of column j) and the next column (through shared memory).
-//  * The Gram terms (dots with the finished columns) are formed while the
-//    partials travel: the warps of finished columns start once the others have
-//    published.
 #include "cluster_common.cuh"
 
 #include <algorithm>
@@ -37,7 +35,7 @@ namespace {
 
 constexpr int kGpThreads = 512;
 constexpr int kNB = 64;
-constexpr int kGpCluster = 8;          // CTAs of a cluster where there are several
+constexpr int kGpPolls = 5;            // sums of other clusters a lane collects (40 clusters)
 
 // Published sums are exchanged without a barrier: every slot is written once
 // per panel, and until then it holds a signalling-NaN pattern that no
@@ -63,27 +61,28 @@ __device__ __forceinline__ double gp_sum8(double v) {
   return v;
 }
 
-// s = sqrt(S) and rb = 1 / (up cl) for cl = -+s, up = x0 - cl, for S within
-// [2^-900, 2^900]: one third-order Householder iteration each from the
-// hardware's approximate reciprocal (square root), about 2^-20 relative, then
-// one Newton correction of s.  13 dependent FP64 operations; sqrt() and the
-// division, with their range checks, are the longest part of a column step
-// otherwise (2000 of 9700 clocks at 32 rows per CTA).
+// s = sqrt(S), cl = -+s, up = x0 - cl and rb = 1 / (up cl) = -1 / (S + |x0| s)
+// for S within [2^-900, 2^900]: a third-order Householder iteration each from
+// the hardware's approximate reciprocal (square root), good to 2^-20 or so, and a
+// Newton correction that takes s to half an ulp (its error enters every entry of
+// the reflector).  Ten dependent FP64 operations of 64 clocks; sqrt() and a division with their
+// range checks take 1600 clocks on an idle pipe, the longest part of a column
+// step.
 __device__ __forceinline__ void gp_pivot(double S, double x0, double *cl, double *up, double *rb) {
   double y, z;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(S));
-  const double e = fma(-(S * y), y, 1.0);
-  y = fma(fma(e, 0.375, 0.5) * e, y, y);
-  double s = S * y;
+  const double ax = fabs(x0);
+  const double s0 = S * y;
+  const double b0 = fma(ax, s0, S);                      // approximate -b, for the seed
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(b0));
+  const double e = fma(-s0, y, 1.0);                     // 1 - S y^2 = 1 - s0^2 / S
+  double s = fma(s0 * e, fma(e, 0.375, 0.5), s0);
   s = fma(fma(-s, s, S), 0.5 * y, s);
-  const double c = x0 > 0.0 ? -s : s;
-  const double u = x0 - c;
-  const double b = u * c;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(b));
+  const double b = fma(ax, s, S);
   const double f = fma(-b, z, 1.0);
-  *rb = fma(fma(f, f, f), z, z);
-  *cl = c;
-  *up = u;
+  *rb = -fma(fma(f, f, f), z, z);
+  *cl = x0 > 0.0 ? -s : s;
+  *up = x0 > 0.0 ? x0 + s : x0 - s;
 }
 
 }  // namespace
@@ -93,10 +92,8 @@ template <int RPL, bool ONE>
 __global__ void __launch_bounds__(kGpThreads, 1)
 panel_grid_kernel(GridPanelParams p) {
   constexpr int R = 8 * RPL;
-  constexpr int SRC = ONE ? kClMaxCtas : kGpCluster;       // senders to a receive buffer
-  constexpr int RC = ONE ? kNB : 8;                        // columns of a receive buffer
-  extern __shared__ __align__(16) unsigned char gp_smem[];
-  double *Gl = (double *)gp_smem;             // [NB][NB] at c + j NB: local Gram terms
+  constexpr int SRC = ONE ? kClMaxCtas : 8;                // senders to a receive buffer
+  constexpr int RC = ONE ? kNB : 16;                       // columns of a receive buffer
   __shared__ __align__(16) double xs[2][R];   // column j's tail by j & 1 (zero elsewhere)
   __shared__ __align__(16) double s_recv[2][SRC][RC];
   __shared__ __align__(16) double s_prow[2][ONE ? kNB : 2];
@@ -111,8 +108,8 @@ panel_grid_kernel(GridPanelParams p) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c = warp * 4 + (lane >> 3), l8 = lane & 7;     // this lane's column and rows
   const int cta = blockIdx.x, P = gridDim.x;
-  const int rank = cluster_rank();
-  const int NC = ONE ? 1 : P / kGpCluster, cluster = ONE ? 0 : cta / kGpCluster;
+  const int rank = cluster_rank(), CS = cluster_ctas();
+  const int NC = P / CS, cluster = cta / CS;
   const int row0 = cta * R;
   const int nbw = p.nbw;
   const int RO = min(R, p.m - p.k0 - p.skip - row0);       // rows owned (<= 0: none)
@@ -140,15 +137,16 @@ panel_grid_kernel(GridPanelParams p) {
       for (int idx = tid; idx < nbw * kNB; idx += kGpThreads)
         p.prow[idx] = __longlong_as_double((long long)kGpUnset);
   }
-  for (int idx = tid; idx < kNB * kNB; idx += kGpThreads) Gl[idx] = 0.0;
 
   // Bytes the receive buffer gets for column j.  ONE: every CTA's partials of
   // the active warps and the pivot row; else the cluster's partials of the
-  // active warps among rank and rank + 8 (32 bytes each).
+  // active warps w = rank, rank + CS, ... (32 bytes each).
   auto warp_active = [&](int w, int j) { return 4 * w + 3 >= j && 4 * w < nbw; };
   auto step_bytes = [&](int j) -> unsigned {
     if (ONE) return (unsigned)((P + 1) * ((nbw + 3) / 4 - j / 4) * 32);
-    return (unsigned)(kGpCluster * 32 * (warp_active(rank, j) + warp_active(rank + 8, j)));
+    int act = 0;
+    for (int w = rank; w < kGpThreads / 32; w += CS) act += warp_active(w, j);
+    return (unsigned)(CS * 32 * act);
   };
   if (tid == 0) {
     mbar_init1(&s_mbar[0]);
@@ -195,7 +193,7 @@ panel_grid_kernel(GridPanelParams p) {
   cluster_sync_all();
   if (!ONE) {
     bool all = true;
-    for (int r = 0; r < kGpCluster; ++r) all &= cluster_ld_u32(cluster_addr(&s_ok, r)) != 0;
+    for (int r = 0; r < CS; ++r) all &= cluster_ld_u32(cluster_addr(&s_ok, r)) != 0;
     cluster_sync_all();
     if (!all) {
       if (tid == 0) record_status(p.status, SLQR_ETIMEOUT);
@@ -231,10 +229,16 @@ panel_grid_kernel(GridPanelParams p) {
     // dot of the tail of x_j with this lane's column (c == j: its norm)
     auto dot = [&]() {
       double a0 = 0.0, a1 = 0.0;
+      if (row0 <= j) {                         // rows up to the pivot's take no part
 #pragma unroll
-      for (int i = 0; i < RPL; i += 2) {
-        a0 = fma(x[l8 + 8 * i], v[i], a0);
-        a1 = fma(x[l8 + 8 * (i + 1)], v[i + 1], a1);
+        for (int i = 0; i < RPL; ++i)
+          a0 = fma(x[l8 + 8 * i], row0 + l8 + 8 * i > j ? v[i] : 0.0, a0);
+      } else {
+#pragma unroll
+        for (int i = 0; i < RPL; i += 2) {
+          a0 = fma(x[l8 + 8 * i], v[i], a0);
+          a1 = fma(x[l8 + 8 * (i + 1)], v[i + 1], a1);
+        }
       }
       if (extreme && mine) {
         double n0 = 0.0;
@@ -262,8 +266,8 @@ panel_grid_kernel(GridPanelParams p) {
             st_async16(cluster_addr(&s_recv[buf][rank][warp * 4 + 2 * h], dst), w,
                        cluster_addr(&s_mbar[buf], dst));
         } else if ((lane & 15) == 0) {
-          const int dst = warp & (kGpCluster - 1);
-          st_async16(cluster_addr(&s_recv[buf][rank][(warp >> 3) * 4 + 2 * h], dst), w,
+          const int dst = warp % CS;
+          st_async16(cluster_addr(&s_recv[buf][rank][(warp / CS) * 4 + 2 * h], dst), w,
                      cluster_addr(&s_mbar[buf], dst));
         }
       }
@@ -285,11 +289,9 @@ panel_grid_kernel(GridPanelParams p) {
           gp_publish(p.prow + (size_t)j * kNB + c, w);
         }
       }
-      if (c < j && l8 == 0) Gl[c + j * kNB] = part;
-      asm volatile("bar.arrive 1, %0;" ::"n"(kGpThreads) : "memory");
       const bool want = c >= j && c < nbw;
       // the receive buffer of column j (this CTA's columns of the cluster, or all)
-      const bool collect = ONE || (warp & (kGpCluster - 1)) == rank;
+      const bool collect = ONE || warp % CS == rank;
       if (collect) {
         bool reported = s_reported != 0;
         if (!dead && !mbar_wait_bounded(&s_mbar[buf], (unsigned)(j >> 1) & 1u, p.spin, p.status,
@@ -298,7 +300,8 @@ panel_grid_kernel(GridPanelParams p) {
           dead = true;
         }
         if (reported && lane == 0) s_reported = 1;
-        const bool last = ONE ? mine : (warp >= kGpCluster || !warp_active(warp + kGpCluster, j));
+        // the warp of this buffer that stays active longest announces the next phase
+        const bool last = ONE ? mine : (warp + CS >= kGpThreads / 32 || 4 * (warp + CS) >= nbw);
         if (last && lane == 0 && !dead && j + 2 < nbw && step_bytes(j + 2) > 0)
           mbar_expect(&s_mbar[buf], step_bytes(j + 2));
         __syncwarp();
@@ -310,33 +313,40 @@ panel_grid_kernel(GridPanelParams p) {
           }
           D = gp_sum8(D);
         } else {
-          const double sum = gp_sum8(s_recv[buf][l8][(warp >> 3) * 4 + (lane >> 3)]);
+          const double sum = gp_sum8(l8 < CS ? s_recv[buf][l8][(warp / CS) * 4 + (lane >> 3)] : 0.0);
           if (l8 == 0 && want) gp_publish(p.rec + ((size_t)j * kNB + c) * NC + cluster, sum);
         }
       }
       if (!ONE) {
-        // the clusters' sums of this lane's column, eight clusters at a time
+        // the clusters' sums of this lane's column
         const double *rec = p.rec + ((size_t)j * kNB + c) * NC;
         const double *prow = p.prow + (size_t)j * kNB + c;
         unsigned it = 0;
-        double r[3];
+        double r[kGpPolls];
 #pragma unroll
-        for (int u = 0; u < 3; ++u) {
+        for (int u = 0; u < kGpPolls; ++u) {
           const int q = l8 + 8 * u;
           r[u] = (want && q < NC) ? gp_load(rec + q) : 0.0;
         }
         pc = want ? gp_load(prow) : 0.0;
         while (!dead) {
-          const bool miss = gp_unset(pc) || gp_unset(r[0]) || gp_unset(r[1]) || gp_unset(r[2]);
+          bool miss = gp_unset(pc);
+#pragma unroll
+          for (int u = 0; u < kGpPolls; ++u) miss |= gp_unset(r[u]);
           if (!__any_sync(0xffffffffu, miss)) break;
           if (it == p.spin && lane == 0) record_status(p.status, SLQR_ETIMEOUT);
           if (++it > kSpinLimit) dead = true;
 #pragma unroll
-          for (int u = 0; u < 3; ++u)
+          for (int u = 0; u < kGpPolls; ++u)
             if (gp_unset(r[u])) r[u] = gp_load(rec + l8 + 8 * u);
           if (gp_unset(pc)) pc = gp_load(prow);
         }
-        D = gp_sum8((r[0] + r[1]) + r[2]);
+        // (adds of absent clusters are skipped, uniformly)
+        D = r[0];
+#pragma unroll
+        for (int u = 1; u < kGpPolls; ++u)
+          if (8 * u < NC) D += r[u];
+        D = gp_sum8(D);
       }
       if (mine) {
         // the pivot, in every lane of this warp
@@ -362,13 +372,6 @@ panel_grid_kernel(GridPanelParams p) {
           s_tau[j] = -rb;
         }
       }
-    } else {
-      // finished columns: their Gram terms while the partials travel
-      asm volatile("bar.sync 1, %0;" ::"n"(kGpThreads) : "memory");
-      if (warp * 4 < nbw) {
-        const double part = dot();
-        if (l8 == 0 && c < nbw) Gl[c + j * kNB] = part;
-      }
     }
     __syncthreads();
     const bool defined = s_def[buf] != 0;
@@ -379,7 +382,7 @@ panel_grid_kernel(GridPanelParams p) {
 #pragma unroll
         for (int i = 0; i < RPL; ++i) {
           const int r = l8 + 8 * i;
-          v[i] = fma(sig, row0 + r == j ? up : x[r], v[i]);
+          if (row0 + r >= j) v[i] = fma(sig, row0 + r == j ? up : x[r], v[i]);
         }
       } else {
 #pragma unroll
@@ -417,128 +420,125 @@ panel_grid_kernel(GridPanelParams p) {
     for (int idx = tid; idx < kNB * kNB; idx += kGpThreads)
       if (idx % kNB >= row0 + R) Vtop[idx] = 0.0;
   }
-  double *G = p.wy + (size_t)kNB * kNB, *tau = p.wy + 2 * (size_t)kNB * kNB;
+  double *tau = p.wy + 2 * (size_t)kNB * kNB;
   if (cta == 0 && tid < kNB) {
     tau[tid] = tid < nbw ? s_tau[tid] : 0.0;
     if (tid < nbw) p.up[p.k0 + tid] = s_up[tid];
   }
-  // publish the local Gram terms and reduce them, entry idx by CTA idx % P:
-  // G[c, j] = v_c[j] up_j + the sum of the tails' dots
-  constexpr int NT = kNB * (kNB - 1) / 2;      // strict upper triangle, packed by column
-  {
-    double *dst = p.gpart + (size_t)cta * NT;
-    for (int idx = tid; idx < kNB * kNB; idx += kGpThreads) {
-      const int jj = idx / kNB, cc = idx - jj * kNB;
-      if (cc < jj) dst[jj * (jj - 1) / 2 + cc] = Gl[idx];
-    }
-  }
   cluster_sync_all();                          // (nothing is sent to this CTA any more)
-  if (!ONE && !grid_barrier(p.bar, p.bar_base + 2u * (unsigned)P, p.status, &s_ok, p.spin)) return;
-  // one warp per entry: the CTAs' terms over its lanes
-  for (int idx = cta + warp * P; idx < kNB * kNB; idx += P * (kGpThreads / 32)) {
-    const int jj = idx / kNB, cc = idx - jj * kNB;
-    double g = 0.0;
-    if (cc < jj && jj < nbw) {
-      const int pos = jj * (jj - 1) / 2 + cc;
-      for (int q = lane; q < P; q += 32) g += __ldcg(p.gpart + (size_t)q * NT + pos);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-      if (lane == 0) g = fma(__ldcg(Vtop + cc * kNB + jj), s_up[jj], g);
-    }
-    if (lane == 0) G[idx] = g;
-  }
 }
 
 // --------------------------------------------------------------------------
 // host side
 // --------------------------------------------------------------------------
+constexpr int kGridRows[] = {32, 48, 64, 80, 96, 128, 160, 192, 256};
 static const void *grid_kernel(int R, bool one) {
   switch (R) {
     case 32: return one ? (const void *)panel_grid_kernel<4, true> : (const void *)panel_grid_kernel<4, false>;
     case 64: return one ? (const void *)panel_grid_kernel<8, true> : (const void *)panel_grid_kernel<8, false>;
     case 128: return one ? (const void *)panel_grid_kernel<16, true> : (const void *)panel_grid_kernel<16, false>;
+    case 48: return one ? (const void *)panel_grid_kernel<6, true> : (const void *)panel_grid_kernel<6, false>;
+    case 80: return one ? nullptr : (const void *)panel_grid_kernel<10, false>;
+    case 96: return one ? (const void *)panel_grid_kernel<12, true> : (const void *)panel_grid_kernel<12, false>;
+    case 160: return one ? nullptr : (const void *)panel_grid_kernel<20, false>;
+    case 192: return one ? nullptr : (const void *)panel_grid_kernel<24, false>;
     case 256: return one ? nullptr : (const void *)panel_grid_kernel<32, false>;
     default: return nullptr;
   }
 }
 
-static void grid_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attrs, int P, bool one,
+static void grid_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attrs, int P, int cluster,
                         cudaStream_t stream) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3(P);
   cfg->blockDim = dim3(kGpThreads);
-  cfg->dynamicSmemBytes = kNB * kNB * sizeof(double);
   cfg->stream = stream;
   attrs[0].id = cudaLaunchAttributeClusterDimension;
-  attrs[0].val.clusterDim.x = one ? P : kGpCluster;
+  attrs[0].val.clusterDim.x = cluster;
   attrs[0].val.clusterDim.y = 1;
   attrs[0].val.clusterDim.z = 1;
   attrs[1].id = cudaLaunchAttributeCooperative;
   attrs[1].val.cooperative = 1;
   cfg->attrs = attrs;
-  cfg->numAttrs = one ? 1 : 2;       // (a cluster is resident as a whole by itself)
+  cfg->numAttrs = P == cluster ? 1 : 2;        // (a cluster is resident as a whole by itself)
 }
 
+// CTAs that can be resident at once in clusters of 4, of 8 and as one cluster
 slqr_status init_grid_panel_attrs(slqr_ctx *ctx) {
-  int clusters = 1 << 30;
+  int c4 = 1 << 20, c8 = 1 << 20;
   bool one_fits = true;
-  for (int R : {32, 64, 128, 256})
+  for (int R : kGridRows)
     for (int one = 0; one < 2; ++one) {
       const void *fn = grid_kernel(R, one);
       if (!fn) continue;
-      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kNB * kNB * (int)sizeof(double));
-      if (e == cudaSuccess && one)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess)
-        return fail(ctx, SLQR_ECUDA, "cudaFuncSetAttribute(grid panel): %s", cudaGetErrorString(e));
-      cudaLaunchConfig_t cfg;
-      cudaLaunchAttribute attrs[2];
-      grid_config(&cfg, attrs, one ? kClMaxCtas : kGpCluster, one, nullptr);
-      cfg.numAttrs = 1;
-      int k = 0;
-      if (cudaOccupancyMaxActiveClusters(&k, fn, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        k = 0;
+      if (one) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess)
+          return fail(ctx, SLQR_ECUDA, "cudaFuncSetAttribute(grid panel): %s", cudaGetErrorString(e));
       }
-      if (one) one_fits = one_fits && k >= 1;
-      else clusters = std::min(clusters, k);
+      auto clusters = [&](int size) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attrs[2];
+        grid_config(&cfg, attrs, size, size, nullptr);
+        int k = 0;
+        if (cudaOccupancyMaxActiveClusters(&k, fn, &cfg) != cudaSuccess) {
+          cudaGetLastError();
+          k = 0;
+        }
+        return k;
+      };
+      if (one) {
+        one_fits = one_fits && clusters(kClMaxCtas) >= 1;
+      } else {
+        c4 = std::min(c4, clusters(4));
+        c8 = std::min(c8, clusters(8));
+      }
     }
-  ctx->grid_panel_ctas = clusters * kGpCluster;
-  ctx->grid_panel_one = one_fits ? kClMaxCtas : kGpCluster;
+  ctx->grid_panel_c4 = std::min(4 * c4, 4 * 8 * kGpPolls) / 4 * 4;
+  ctx->grid_panel_c8 = std::min(8 * c8, 8 * 8 * kGpPolls) / 8 * 8;
+  ctx->grid_panel_one = one_fits ? kClMaxCtas : 8;
   return SLQR_OK;
 }
 
-// One cluster up to 16 CTAs of 64 rows, else several.
-int grid_panel_rows(const slqr_ctx *ctx, int M, int rows_min, int *ctas) {
-  for (int R : {32, 64, 128, 256}) {
+// Rows per CTA, smallest first.  One cluster up to 16 CTAs of 64 rows (1024
+// rows: 3.6 us a column; 32 CTAs in clusters of 8: 4.0).  Above that clusters of
+// 8, 64 CTAs at most while 256 rows each are enough: the sums of more clusters
+// take longer to arrive than the shorter slices save (8192 rows: 6.2 us a column
+// on 64 CTAs, 7.6 on 104), and the trailing update runs on the other SMs.
+GridPanelShape grid_panel_shape(const slqr_ctx *ctx, int M, int rows_min) {
+  GridPanelShape s;
+  const int one = ctx->grid_panel_one;
+  for (int R : kGridRows) {
+    const int P = (M + R - 1) / R;
     if (rows_min > 0 && R < rows_min && R < 256) continue;
-    int P = (M + R - 1) / R;
-    if (P <= ctx->grid_panel_one && R <= 128 && (R <= 64 || rows_min > 0)) {
-      *ctas = P;
-      return R;
+    if (P <= one && grid_kernel(R, true) && (R <= 64 || rows_min > 0)) {
+      s.R = R, s.P = P, s.cluster = P;
+      return s;
     }
-    P = (P + kGpCluster - 1) / kGpCluster * kGpCluster;
-    const int most = std::min(ctx->grid_panel_ctas, 24 * kGpCluster);
-    if (P <= (rows_min > 0 || R == 256 ? most : std::min(most, 64))) {
-      if (R < 64 && rows_min == 0 && (M + 63) / 64 <= ctx->grid_panel_one) continue;
-      *ctas = P;
-      return R;
+    if (rows_min == 0 && R < 64 && (M + 63) / 64 <= one) continue;
+    const int P8 = (P + 7) / 8 * 8;
+    if (P8 <= std::min(ctx->grid_panel_c8, rows_min > 0 || R == 256 ? ctx->grid_panel_c8 : 64) &&
+        (P8 > one || !grid_kernel(R, true))) {
+      s.R = R, s.P = P8, s.cluster = 8;
+      return s;
     }
   }
-  return 0;
+  const int P4 = ((M + 255) / 256 + 3) / 4 * 4;
+  if (P4 <= ctx->grid_panel_c4) s.R = 256, s.P = P4, s.cluster = 4;
+  return s;                                    // R = 0: too tall
 }
 
-slqr_status launch_grid_panel(slqr_ctx *ctx, GridPanelParams &p, int R, int P, cudaStream_t stream) {
-  const bool one = P <= ctx->grid_panel_one && R <= 128;
+slqr_status launch_grid_panel(slqr_ctx *ctx, GridPanelParams &p, const GridPanelShape &s,
+                              cudaStream_t stream) {
+  const bool one = s.P == s.cluster && grid_kernel(s.R, true);
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attrs[2];
-  grid_config(&cfg, attrs, P, one, stream);
+  grid_config(&cfg, attrs, s.P, s.cluster, stream);
   void *args[] = {&p};
-  cudaError_t e = cudaLaunchKernelExC(&cfg, grid_kernel(R, one), args);
+  cudaError_t e = cudaLaunchKernelExC(&cfg, grid_kernel(s.R, one), args);
   if (e != cudaSuccess)
-    return fail(ctx, SLQR_ECUDA, "panel launch (P=%d, R=%d): %s", P, R, cudaGetErrorString(e));
-  p.bar_base += one ? 0u : 2u * (unsigned)P;
+    return fail(ctx, SLQR_ECUDA, "panel launch (P=%d, R=%d): %s", s.P, s.R, cudaGetErrorString(e));
+  p.bar_base += one ? 0u : (unsigned)s.P;
   return SLQR_OK;
 }
 

@@ -79,8 +79,8 @@ struct slqr_ctx {
   // 2: BF16 split in hi + lo, with the BF16 shadows of the matrix below)
   int tc_mode = 0;
   void *sh_hi = nullptr, *sh_lo = nullptr;
-  // CTAs the FP64 grid panel may use, in clusters of 8 and as one cluster
-  int grid_panel_ctas = 0, grid_panel_one = 0;
+  // CTAs the FP64 grid panel may use: in clusters of 4, of 8, as one cluster
+  int grid_panel_c4 = 0, grid_panel_c8 = 0, grid_panel_one = 0;
   // limit of the polled exchanges and grid barriers of the cooperative kernels
   unsigned spin_limit = slqr::kSpinLimit;
   std::string last_error;
@@ -166,7 +166,12 @@ int launch_vtx_tc(const float *A, int lda, const double *Vtop, int k0, int M, in
 //   fx_update    X -= V T^T V^T X (rows of the panel at k0, ldx, N columns);
 //                cmax: column maxima of X over those rows; cnext (or NULL)
 //                receives the maxima over the rows of the next panel.  False
-//                (nothing launched) when work_bytes is too small.
+//                (nothing launched) when work_bytes is too small.  gram (or
+//                NULL): scratch of kFxGramBytes, zero before; the panel's G is
+//                formed from V's digits and written to wy_panel and Gt first.
+//                Gt: kFxGt doubles, tau_j G[j, .] by rows and tau
+//   fx_gram      the same G and Gt alone, for a panel without such an update
+//   fx_prep      Gt of every panel of a compact-WY store (panels of nb)
 constexpr int kFxMinCols = 16;       // narrower updates stay on the FP64 pipe
 slqr_status init_fx_attrs(slqr_ctx *ctx);
 size_t fx_v_bytes(int m);
@@ -176,8 +181,14 @@ void fx_colmax(const double *X, int ldx, int m, int n, int stacked_top, bool upp
 void fx_split_v(const double *A, int lda, const double *Vtop, int k0, int nbw, int M, int skip,
                 void *vbuf, cudaStream_t stream);
 bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy_panel,
-               const void *vbuf, double *X, int ldx, int N, const unsigned *cmax, unsigned *cnext,
-               void *work, size_t work_bytes, cudaStream_t stream);
+               const double *Gt, const void *vbuf, double *X, int ldx, int N, const unsigned *cmax,
+               unsigned *cnext, void *work, size_t work_bytes, cudaStream_t stream,
+               void *gram = nullptr);
+constexpr size_t kFxGramBytes = 64 * 64 * 8 + 256;
+constexpr int kFxGt = 64 * 64 + 64;
+void fx_gram(slqr_ctx *ctx, int nbw, int M, double *wy_panel, const void *vbuf, void *gram,
+             double *Gt, cudaStream_t stream);
+void fx_prep(const double *wy, int K, int nb, double *Gt, cudaStream_t stream);
 
 // slqr_batch_factor with a per-problem stacked top block (ntop[i] rows, 0 for a
 // dense problem; ntop may be NULL); takes the context mutex.
@@ -295,16 +306,16 @@ slqr_status launch_cluster_panel(slqr_ctx *ctx, bool f32, int nb, const ClusterP
 int panel_cluster_ctas(slqr_ctx *ctx, bool f32, int nb, int M, int nbw);
 
 // The FP64 panel of 64 columns by thread-block clusters with the panel in
-// registers (panel_grid.cu): P CTAs of R rows each.
+// registers (panel_grid.cu): P CTAs of R rows each.  The Gram terms G of the
+// compact-WY block are left to fx_update / fx_gram.
 struct GridPanelParams {
   void *A;             // double *, column-major, leading dimension lda
   double *up;          // global up array
-  double *wy;          // this panel's compact-WY block (Vtop | G | tau)
+  double *wy;          // this panel's compact-WY block: Vtop and tau are written
   double *rec;         // 64 * 64 * clusters: per column j and entry c the clusters' dots
   double *srec;        // P * 64: per-CTA column scales (panel start)
-  double *gpart;       // P * 64 * 63 / 2: per-CTA partial Gram terms
   double *prow;        // 64 * 64: per column j the pivot row
-  unsigned *bar;       // monotonic arrival counter (two arrivals per CTA and panel)
+  unsigned *bar;       // monotonic arrival counter (one arrival per CTA and panel)
   int *status;
   int m, lda, k0, nbw;
   int skip, stacked;   // as ClusterPanelParams
@@ -312,9 +323,13 @@ struct GridPanelParams {
   unsigned spin;       // polls of a bounded wait before it reports
 };
 slqr_status init_grid_panel_attrs(slqr_ctx *ctx);
-// rows per CTA (0: no grid panel) and CTAs for a panel of M rows; rows_min 0: chosen
-int grid_panel_rows(const slqr_ctx *ctx, int M, int rows_min, int *ctas);
-slqr_status launch_grid_panel(slqr_ctx *ctx, GridPanelParams &p, int R, int P, cudaStream_t stream);
+struct GridPanelShape {
+  int R = 0, P = 0, cluster = 0;       // rows per CTA (0: no grid panel), CTAs, cluster size
+};
+// for a panel of M rows; rows_min 0: chosen
+GridPanelShape grid_panel_shape(const slqr_ctx *ctx, int M, int rows_min);
+slqr_status launch_grid_panel(slqr_ctx *ctx, GridPanelParams &p, const GridPanelShape &s,
+                              cudaStream_t stream);
 
 // Look-ahead update of the next panel's columns (at most 64) of an FP32
 // factorization with panels of width 64, in one cooperative launch

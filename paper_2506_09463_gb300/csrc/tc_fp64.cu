@@ -45,7 +45,8 @@ namespace slqr {
 
 constexpr int kFxD = 7;                       // digits
 constexpr int kFxOrders = 8;                  // accumulated orders i + j
-constexpr int kFxThreads = 512;
+constexpr int kFxWorkers = 16;                // warps that split and reassemble; one more issues MMAs
+constexpr int kFxThreads = 32 * (kFxWorkers + 1);
 constexpr int kFxV1Chunk = kFxD * 64 * 64;            // 28672 B: 32 rows
 constexpr int kFxV2Tile = kFxD * 128 * 128;           // 114688 B: 128 rows
 constexpr int kFxWTile = kFxD * 32 * 128;             // 28672 B: 32 columns
@@ -53,12 +54,23 @@ constexpr int kFxXStage = kFxD * 128 * 64;            // 57344 B: 128 columns x 
 constexpr int kFxStage = kFxXStage + kFxV1Chunk;
 constexpr size_t kFxVtxSmem = 2 * (size_t)kFxStage + 1024;
 constexpr size_t kFxUpdSmem = (size_t)kFxV2Tile + 2 * kFxWTile + 1024;
+constexpr int kFxMaxPer = 32;                // column tiles of a CTA of the update
 constexpr int kFxNonFinite = 1 << 20;         // exponent that stands for Inf / NaN
 
 // D = F32, A = B = F16, both K-major, M = 128; N is added per MMA
 constexpr uint32_t kIdescF16 = (1u << 4) | ((128u >> 4) << 24);
 
 __device__ __forceinline__ uint32_t fx_idesc(int n) { return kIdescF16 | ((uint32_t)(n >> 3) << 17); }
+
+// The Gram terms of a panel beside (or, with no columns, instead of) V^T X
+struct FxGram {
+  unsigned long long *sum;             // [c][a], zero before; NULL: none
+  unsigned *arrived;                   // zero before
+  double *G;                           // the compact-WY store's G (tau follows it)
+  double *Gt;                          // Gt and tau for the substitution (kFxGt doubles)
+  int slices, RS;                      // CTAs, rows of each (a multiple of 128)
+  int vtx_slices;                      // row slices of V^T X
+};
 
 // K-major operand with 64-byte rows, SWIZZLE_64B, 8-row groups 512 bytes apart
 __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
@@ -174,18 +186,38 @@ __device__ __forceinline__ double fx_scale(double t, int k) {
   return scalbn(t, k);
 }
 
-#define FX_LD16(r, addr)                                                                         \
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "                                         \
-               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"                 \
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),         \
-                 "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),       \
-                 "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])                              \
-               : "r"(addr))
-#define FX_LD8(r, addr)                                                                          \
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"          \
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),         \
-                 "=r"(r[6]), "=r"(r[7])                                                          \
-               : "r"(addr))
+// t 2^sh rounded to FP64 for sh in [-1000, 900], in integer arithmetic: a
+// conversion instruction would hold the FP64 pipe for 16 clocks of the SM.
+__device__ __forceinline__ double fx_to_double(long long t, int sh) {
+  const unsigned long long a = (unsigned long long)(t < 0 ? -t : t);
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << (lz & 63);           // leading bit at 63
+  // mantissa rounded half up; its leading bit adds one to the exponent field
+  unsigned long long b = ((unsigned long long)(1085 - lz + sh) << 52) + (m >> 11) + ((m >> 10) & 1);
+  b = a ? b : 0ull;
+  return __longlong_as_double((long long)(b | ((unsigned long long)t & (1ull << 63))));
+}
+
+// Four accumulators of every order for this thread's TMEM lane: order o at
+// addr + o * stride columns.
+__device__ __forceinline__ void fx_ld_orders(uint32_t (&r)[kFxOrders][4], uint32_t addr,
+                                             uint32_t stride) {
+#pragma unroll
+  for (int o = 0; o < kFxOrders; ++o)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[o][0]), "=r"(r[o][1]), "=r"(r[o][2]), "=r"(r[o][3])
+                 : "r"(addr + (uint32_t)o * stride));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// Orders o0 .. o0 + 3 of one output: sum of acc_o 256^(3 - (o - o0))
+__device__ __forceinline__ long long fx_four(const uint32_t (&r)[kFxOrders][4], int o0, int k) {
+  long long v = __float2int_rn(__uint_as_float(r[o0 + 3][k]));
+  v += (long long)__float2int_rn(__uint_as_float(r[o0 + 2][k])) * 256;
+  v += (long long)__float2int_rn(__uint_as_float(r[o0 + 1][k])) * 65536;
+  v += (long long)__float2int_rn(__uint_as_float(r[o0][k])) * 16777216;
+  return v;
+}
 
 // --------------------------------------------------------------------------
 // Column maxima (high words) of the rows each panel sees: cmax[p][c] over the
@@ -309,25 +341,171 @@ fx_vsplit_kernel(const double *__restrict__ A, int lda, const double *__restrict
   }
 }
 
+__device__ __forceinline__ void fx_mbar_init(uint64_t *bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+}
+__device__ __forceinline__ void fx_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// Unit exponent of the totals over slices of RS rows: 56 up to 512 rows, one
+// more for every factor of four.
+__device__ __forceinline__ int fx_unit(int RS) {
+  return 56 + (RS > 512) + (RS > 2048) + (RS > 8192) + (RS > 32768);
+}
+// whole-warp wait (the lanes leave together)
+__device__ __forceinline__ bool fx_wait(uint64_t *bar, int phase) {
+  return __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), (uint32_t)(phase & 1)));
+}
+
+// --------------------------------------------------------------------------
+// Strict upper triangle of G = V^T V of the panel, from the digit images V1 on
+// both sides: gram[c][a] += the sums over this CTA's rows (integers, so the
+// order of the atomic adds does not matter), and the CTA that arrives last
+// writes G to the compact-WY store and tau G for the substitution.  Digits i and i + 1 of V are the two halves
+// of the M side (rows 64 .. 127 of A are digit i + 1, one order up), the stacked
+// digits the N side.  With V's wide leading digits the sums are still exact: by
+// Cauchy-Schwarz a product with them is at most (sqrt(2) 1024)^2 over all rows.
+// G is known to 2^-58 of |up_a up_c|; the panel's own sums in FP64 cost it 0.5
+// us of each column step.
+// Called by every thread of CTAs (gridDim.x - 1, y), y < slices.
+// --------------------------------------------------------------------------
+constexpr int kFxGramChunk = kFxV1Chunk + 4096;       // (a zero digit 7 behind each chunk)
+constexpr int kFxGramShift = 56;                      // units of 2^56 digit products
+
+__device__ __noinline__ void fx_gram_block(const FxGram &gr, int nbw, int M,
+                                           const unsigned char *V1, unsigned char *base,
+                                           uint32_t taddr, uint64_t *s_full, uint64_t *s_acc,
+                                           const int *s_fa, int *status) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int i_begin = blockIdx.y * gr.RS, i_end = min(M, i_begin + gr.RS);
+  const int B = (i_end - i_begin + 127) / 128;
+  for (int idx = tid; idx < 4 * 4096 / 16; idx += kFxThreads)
+    *(uint4 *)(base + (idx >> 8) * kFxGramChunk + kFxV1Chunk + (idx & 255) * 16) =
+        make_uint4(0, 0, 0, 0);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  const int q = warp & 3, h = warp >> 2;               // workers: TMEM lanes, 16 columns
+  const int a = (q * 32 + lane) & 63;
+  const bool upper = q >= 2;                            // lanes of digit i + 1
+  long long tot[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) tot[k] = 0;
+  bool ok = true;
+  for (int b = 0; b < B && ok; ++b) {
+    if (tid == 0) {
+      const uint32_t bar = smem_u32(s_full);
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                   ::"r"(bar), "r"(4 * kFxV1Chunk) : "memory");
+      for (int u = 0; u < 4; ++u)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes"
+                     " [%0], [%1], %2, [%3];"
+                     ::"r"(smem_u32(base + u * kFxGramChunk)),
+                     "l"(V1 + (size_t)(i_begin / 32 + b * 4 + u) * kFxV1Chunk), "r"(kFxV1Chunk),
+                     "r"(bar) : "memory");
+      if (mbar_wait(bar, (uint32_t)(b & 1))) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t v = smem_u32(base + u * kFxGramChunk);
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks) {
+            const bool acc = u > 0 || ks > 0;
+            auto piece = [&](int i, int n0, int n, bool ac) {
+              fx_mma(taddr + (uint32_t)(i * 64 + n0), sw64_desc(v + i * 4096 + ks * 32),
+                     sw64_desc(v + n0 * 64 + ks * 32), n, ac);
+            };
+            piece(0, 0, 256, acc);  piece(0, 256, 192, acc);
+            piece(2, 0, 192, true); piece(2, 192, 128, true); piece(2, 320, 64, acc);
+            piece(4, 0, 256, true);
+            piece(6, 0, 128, true);
+          }
+        }
+        fx_commit(s_acc);
+      }
+    }
+    __syncwarp();
+    ok = fx_wait(s_acc, b);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok && warp < kFxWorkers) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        uint32_t r[kFxOrders][4];
+        fx_ld_orders(r, taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * 16 + u * 4), 64);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          // lower lanes: block t is order t; upper lanes: order t + 1 (8 dropped)
+          if (upper) r[7][k] = 0;
+          const long long x = fx_four(r, 0, k), y = fx_four(r, 4, k);
+          tot[u * 4 + k] += upper ? (x << 8) + ((y + (1 << 23)) >> 24)
+                                  : (x << 16) + ((y + (1 << 15)) >> 16);
+        }
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    ok = __syncthreads_and(ok);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  if (!ok && tid == 0) {
+    mbar_wait(smem_u32(s_full), (uint32_t)((B - 1) & 1));   // let the copies in flight land
+    atomicCAS(status, 0, SLQR_ETIMEOUT);
+  }
+  if (warp < kFxWorkers) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const int c = h * 16 + k;
+      if (a < c) atomicAdd(gr.sum + c * 64 + a, (unsigned long long)tot[k]);
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  __shared__ int s_last;
+  if (tid == 0) s_last = atomicAdd(gr.arrived, 1u) == (unsigned)gr.slices - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int idx = tid; idx < 64 * 64; idx += kFxThreads) {
+    const int c = idx >> 6, aa = idx & 63;
+    double g = 0.0;
+    if (aa < c && c < nbw) {
+      const int fa = s_fa[aa], fc = s_fa[c];
+      const long long t = (long long)__ldcg(gr.sum + idx);
+      g = (fa == kFxNonFinite || fc == kFxNonFinite)
+              ? __longlong_as_double(0x7ff8000000000000ll)
+              : fx_scale((double)t, fa + fc - 110 + kFxGramShift);
+    }
+    gr.G[idx] = g;
+    const double tau = gr.G[64 * 64 + aa];               // (of the panel's own kernel)
+    gr.Gt[aa * 64 + c] = (aa < c && c < nbw) ? tau * g : 0.0;
+    if (c == 0) gr.Gt[64 * 64 + aa] = aa < nbw ? tau : 0.0;
+  }
+}
+
 // --------------------------------------------------------------------------
 // W_part[s][c][a] = sum over the rows i of slice s of X(i, c) V(i, a):
 // 128 columns of X on the M side, the digits of the 64 reflectors stacked on
-// the N side, 32 rows per stage.  X is read as FP64 and split here (a thread
-// owns 8 consecutive rows of a column); V's digits come by bulk copy.  Every
-// 128 rows the eight accumulators are drained into 96-bit integer totals.
-// grid: (ceil(N / 128), S), slices of RS rows (a multiple of 128).
+// the N side, 32 rows per stage, two stages.  The sixteen worker warps read X
+// as FP64 and split it (a thread owns 8 consecutive rows of a column); V's
+// digits come by bulk copy; warp 16 issues the MMAs.  Every 128 rows the eight
+// accumulators (all of tensor memory) are drained into 96-bit integer totals;
+// the workers split the first chunk of the next 128 rows before they wait for
+// that, so the splitting of a chunk runs beside the MMAs of the one before.
+// grid: (ceil(N / 128), S), slices of RS rows (a multiple of 128); with gr.sum
+// one more column of CTAs for the Gram terms (fx_gram_block).
 // --------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFxThreads, 1)
 fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M, int N,
               int RS, const unsigned char *__restrict__ V1, const double *__restrict__ Vtop,
-              const unsigned *__restrict__ cmax, double *__restrict__ Wp, int *status) {
+              const unsigned *__restrict__ cmax, double *__restrict__ Wp, FxGram gr, int *status) {
   extern __shared__ __align__(1024) unsigned char fx_smem_raw[];
   unsigned char *base = (unsigned char *)(((uintptr_t)fx_smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ uint32_t s_taddr;
-  __shared__ __align__(8) uint64_t s_full[2], s_empty[2];
+  // V's copy landed, X's digits written, a stage's MMAs done; accumulators
+  // complete, accumulators drained
+  __shared__ __align__(8) uint64_t s_full[2], s_xfull[2], s_empty[2], s_acc, s_drained;
   __shared__ int s_fa[64];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c0 = blockIdx.x * 128, s = blockIdx.y;
+  const bool gram = gr.sum != nullptr && blockIdx.x == gridDim.x - 1;
+  if ((int)blockIdx.y >= (gram ? gr.slices : gr.vtx_slices)) return;
   const int i_begin = s * RS, i_end = min(M, i_begin + RS);
   const int T = (i_end - i_begin + 31) / 32;
 
@@ -338,89 +516,37 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
   }
   if (tid == 0) {
     for (int st = 0; st < 2; ++st) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_full[st])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_empty[st])));
+      fx_mbar_init(&s_full[st], 1);
+      fx_mbar_init(&s_xfull[st], kFxWorkers);
+      fx_mbar_init(&s_empty[st], 1);
     }
+    fx_mbar_init(&s_acc, 1);
+    fx_mbar_init(&s_drained, kFxWorkers);
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (tid < 64) {
     const double up = Vtop[tid * 65];
     s_fa[tid] = (fx_hi(up) >= 0x7ff00000u) ? kFxNonFinite : fx_exp_of_hi(fx_hi(up)) - 3;
   }
-  // the splitting thread's column and group of 8 rows, and its column's exponent
-  const int sc = tid >> 2, rg = tid & 3;
-  const bool col_ok = c0 + sc < N;
-  const unsigned scm = col_ok ? cmax[c0 + sc] : 0u;
-  const int se = fx_exp_of_hi(scm);
-  const double *xcol = X + (size_t)(c0 + (col_ok ? sc : 0)) * ldx;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t taddr = s_taddr;
 
-  auto load_v = [&](int t) {
-    fx_bulk(smem_u32(base + (t & 1) * kFxStage + kFxXStage),
-            V1 + (size_t)(i_begin / 32 + t) * kFxV1Chunk, kFxV1Chunk, &s_full[t & 1]);
-  };
-  double xv[8];
-  auto load_x = [&](int t) {
-    const int i = i_begin + t * 32 + rg * 8;
-    const double *p = xcol + k0 + i + (i >= nbw ? skip : 0);
-    const bool whole = i + 8 <= i_end && (i >= nbw || i + 8 <= nbw || skip == 0);
-    if (col_ok && whole) {
-      if ((((uintptr_t)p) & 15) == 0) {
-#pragma unroll
-        for (int k = 0; k < 8; k += 2) {
-          const double2 v = *(const double2 *)(p + k);
-          xv[k] = v.x;
-          xv[k + 1] = v.y;
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) xv[k] = p[k];
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int ii = i + k;
-        xv[k] = (col_ok && ii < i_end) ? xcol[k0 + ii + (ii >= nbw ? skip : 0)] : 0.0;
-      }
-    }
-  };
-  int issued = 0;                                       // V copies (thread 0)
-  if (tid == 0)
-    for (; issued < T && issued < 2; ++issued) load_v(issued);
-  load_x(0);
-
-  // drain mapping: TMEM lane = column of X, this thread's 16 reflectors
-  const int dq = warp & 3, dh = warp >> 2;
-  long long hi[16], lo[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) hi[k] = lo[k] = 0;
-  bool ok = true;
-  for (int t = 0; t < T; ++t) {
-    const int st = t & 1;
-    unsigned char *Xs = base + st * kFxStage;
-    if (t >= 2) {                                       // the MMAs of chunk t - 2 are done
-      ok = mbar_wait(smem_u32(&s_empty[st]), (uint32_t)((t / 2 - 1) & 1));
-      if (tid == 0 && ok) { load_v(t); ++issued; }
-    }
-    {
-      unsigned long long y[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) y[k] = fx_digits(xv[k], se);
-      unsigned char *dst = Xs + sc * 64 + ((rg * 16) ^ (((sc >> 1) & 3) << 4));
-#pragma unroll
-      for (int i = 0; i < kFxD; ++i) *(uint4 *)(dst + i * 8192) = fx_pack8(y, i);
-    }
-    if (t + 1 < T) load_x(t + 1);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (!__syncthreads_and(ok)) { ok = false; break; }
-    if (tid == 0) {
-      // (a copy that never lands leaves the wait for these MMAs to run out)
-      if (mbar_wait(smem_u32(&s_full[st]), (uint32_t)((t >> 1) & 1))) {
+  if (gram) {
+    fx_gram_block(gr, nbw, M, V1, base, taddr, &s_full[0], &s_acc, s_fa, status);
+  } else if (warp == kFxWorkers) {                      // ---- the MMAs --------------------
+    if (lane == 0) {
+      bool ok = true;
+      for (int t = 0; t < T; ++t) {
+        const int st = t & 1;
+        ok = mbar_wait(smem_u32(&s_full[st]), (uint32_t)((t >> 1) & 1)) &&
+             mbar_wait(smem_u32(&s_xfull[st]), (uint32_t)((t >> 1) & 1));
+        if (ok && (t & 3) == 0 && t > 0)
+          ok = mbar_wait(smem_u32(&s_drained), (uint32_t)((t / 4 - 1) & 1));
+        if (!ok) break;                                 // (the workers' waits run out too)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t xa = smem_u32(Xs), vb = xa + kFxXStage;
+        const uint32_t xa = smem_u32(base + st * kFxStage), vb = xa + kFxXStage;
         const bool fresh = (t & 3) == 0;
 #pragma unroll
         for (int ks = 0; ks < 2; ++ks) {
@@ -440,50 +566,119 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
           piece(6, 0, 128, true);
         }
         fx_commit(&s_empty[st]);
+        if ((t & 3) == 3 || t == T - 1) fx_commit(&s_acc);
       }
     }
-    if ((t & 3) == 3 || t == T - 1) {                   // drain
-      ok = mbar_wait(smem_u32(&s_empty[st]), (uint32_t)((t >> 1) & 1));
-      ok = __all_sync(0xffffffffu, ok);
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (ok) {
+  } else {                                              // ---- splitting, draining ---------
+    // this thread's column and group of 8 rows, and its column's exponent
+    const int sc = tid >> 2, rg = tid & 3;
+    const bool col_ok = c0 + sc < N;
+    const int se = fx_exp_of_hi(col_ok ? cmax[c0 + sc] : 0u);
+    const double *xcol = X + (size_t)(c0 + (col_ok ? sc : 0)) * ldx;
+    auto load_v = [&](int t) {
+      fx_bulk(smem_u32(base + (t & 1) * kFxStage + kFxXStage),
+              V1 + (size_t)(i_begin / 32 + t) * kFxV1Chunk, kFxV1Chunk, &s_full[t & 1]);
+    };
+    double xv[8];
+    auto load_x = [&](int t) {
+      const int i = i_begin + t * 32 + rg * 8;
+      const double *p = xcol + k0 + i + (i >= nbw ? skip : 0);
+      // the registers hold one chunk ahead; L2 gets three (128 bytes per thread pair)
+      if (col_ok && (rg & 1) == 0 && i + 96 + 16 <= i_end)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(xcol + k0 + i + 96 + (i + 96 >= nbw ? skip : 0)));
+      const bool whole = i + 8 <= i_end && (i >= nbw || i + 8 <= nbw || skip == 0);
+      if (col_ok && whole) {
+        if ((((uintptr_t)p) & 15) == 0) {
 #pragma unroll
-        for (int o = 0; o < kFxOrders; ++o) {
-          uint32_t r[16];
-          FX_LD16(r, taddr + ((uint32_t)(dq * 32) << 16) + (uint32_t)(o * 64 + dh * 16));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          const int w = 1 << (8 * (3 - (o & 3)));
-#pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const long long v = (long long)__float2int_rn(__uint_as_float(r[k])) * w;
-            if (o < 4) hi[k] += v;
-            else lo[k] += v;
+          for (int k = 0; k < 8; k += 2) {
+            const double2 v = *(const double2 *)(p + k);
+            xv[k] = v.x;
+            xv[k + 1] = v.y;
           }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) xv[k] = p[k];
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int ii = i + k;
+          xv[k] = (col_ok && ii < i_end) ? xcol[k0 + ii + (ii >= nbw ? skip : 0)] : 0.0;
         }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      if (!__syncthreads_and(ok)) { ok = false; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    }
-  }
-  if (!ok && tid == 0) {
-    for (int t = max(0, issued - 2); t < issued; ++t)   // let the copies in flight land
-      mbar_wait(smem_u32(&s_full[t & 1]), (uint32_t)((t >> 1) & 1));
-    atomicCAS(status, 0, SLQR_ETIMEOUT);
-  }
-  const int c = c0 + dq * 32 + lane;
-  if (ok && c < N) {
-    const unsigned cm = cmax[c];
-    const int e = fx_exp_of_hi(cm);
-    double *out = Wp + ((size_t)s * N + c) * 64 + dh * 16;
+    };
+    int issued = 0;                                     // V copies (thread 0)
+    if (tid == 0)
+      for (; issued < T && issued < 2; ++issued) load_v(issued);
+    load_x(0);
+    // drain mapping: TMEM lane = column of X, this thread's 16 reflectors
+    const int dq = warp & 3, dh = warp >> 2;
+    // Totals in units of 2^ush digit products, ush from the slice's rows: a total
+    // is at most ||x|| ||v|| < 2^55 sqrt(RS) sqrt(2) 2^58 of those, 62 bits.
+    const int ush = fx_unit(RS);
+    long long tot[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int f = s_fa[dh * 16 + k];
-      // (hi 2^32 + lo) 2^40 in units of 2^(e-55) 2^(f-55)
-      double v = fma((double)hi[k], 4294967296.0, (double)lo[k]);
-      v = (cm >= 0x7ff00000u || f == kFxNonFinite) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                   : fx_scale(v, e + f - 70);
-      out[k] = v;
+    for (int k = 0; k < 16; ++k) tot[k] = 0;
+    auto drain = [&](int b) -> bool {
+      if (!fx_wait(&s_acc, b)) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        uint32_t r[kFxOrders][4];
+        fx_ld_orders(r, taddr + ((uint32_t)(dq * 32) << 16) + (uint32_t)(dh * 16 + u * 4), 64);
+        if (u == 3) {
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          if (lane == 0) fx_arrive(&s_drained);
+        }
+        // orders 0..3 in units of 2^72, 4..7 in units of 2^40
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          tot[u * 4 + k] += (fx_four(r, 0, k) << (72 - ush)) +
+                            ((fx_four(r, 4, k) + (1ll << (ush - 41))) >> (ush - 40));
+      }
+      return true;
+    };
+    bool ok = true;
+    for (int t = 0; t < T && ok; ++t) {
+      const int st = t & 1;
+      if (t >= 2) {                                     // the MMAs of chunk t - 2 are done
+        ok = fx_wait(&s_empty[st], t / 2 - 1);
+        if (!ok) break;
+        if (tid == 0) { load_v(t); ++issued; }
+      }
+      {
+        unsigned long long y[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) y[k] = fx_digits(xv[k], se);
+        unsigned char *dst = base + st * kFxStage + sc * 64 + ((rg * 16) ^ (((sc >> 1) & 3) << 4));
+#pragma unroll
+        for (int i = 0; i < kFxD; ++i) *(uint4 *)(dst + i * 8192) = fx_pack8(y, i);
+      }
+      if (t + 1 < T) load_x(t + 1);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) fx_arrive(&s_xfull[st]);
+      if (t > 0 && (t & 3) == 0) ok = drain(t / 4 - 1);
+    }
+    if (ok) ok = drain((T - 1) / 4);
+    if (!ok && lane == 0) {
+      for (int t = max(0, issued - 2); t < issued; ++t) // let the copies in flight land
+        mbar_wait(smem_u32(&s_full[t & 1]), (uint32_t)((t >> 1) & 1));
+      atomicCAS(status, 0, SLQR_ETIMEOUT);
+    }
+    const int c = c0 + dq * 32 + lane;
+    if (ok && c < N) {
+      const unsigned cm = cmax[c];
+      const int e = fx_exp_of_hi(cm);
+      double *out = Wp + ((size_t)s * N + c) * 64 + dh * 16;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int f = s_fa[dh * 16 + k];
+        // tot 2^ush in units of 2^(e-55) 2^(f-55)
+        out[k] = (cm >= 0x7ff00000u || f == kFxNonFinite)
+                     ? __longlong_as_double(0x7ff8000000000000ll)
+                     : fx_scale((double)tot[k], e + f - 110 + ush);
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -493,105 +688,147 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
 }
 
 // --------------------------------------------------------------------------
-// W' = T^T W from the partials (the substitution of tw_kernel in factor.cu),
-// written as the digit image of X -= V W': column c scaled by the largest
-// |W'(a, c)| 2^(f_a), f_a the exponent of reflector a.  One warp per column.
+// Gt[j][q] = tau_j G[j][q] (q > j, else 0), row-major, then tau: what the
+// substitution of W' = T^T W reads.  One CTA per panel.
 // --------------------------------------------------------------------------
-template <int COLS>
 __global__ void __launch_bounds__(256)
-fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restrict__ wy, int nbw,
-             unsigned char *__restrict__ Wimg, int *__restrict__ ecol) {
-  constexpr int NB = 64, GLD = NB + 1;
-  constexpr int TPE = 256 / (COLS * NB);
-  __shared__ double w[COLS][NB];
-  __shared__ double part[TPE][COLS * NB];
-  __shared__ double G[NB * GLD];
-  __shared__ double tau[NB];
-  __shared__ int s_f[NB];
-  const int tid = threadIdx.x;
+fx_prep_kernel(const double *__restrict__ wy, int K, int nb, double *__restrict__ out) {
+  const int nbw = min(nb, K - (int)blockIdx.x * nb);
+  const double *G = wy + (size_t)blockIdx.x * wy_panel_doubles(nb) + nb * nb, *tau = G + nb * nb;
+  double *o = out + (size_t)blockIdx.x * kFxGt;
+  __shared__ double t[64][65];
+  for (int idx = threadIdx.x; idx < nb * nb; idx += 256) t[idx % nb][idx / nb] = G[idx];
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < 64 * 64; idx += 256) {
+    const int j = idx >> 6, q = idx & 63;
+    o[idx] = (q > j && q < nbw) ? tau[j] * t[j][q] : 0.0;
+  }
+  if (threadIdx.x < 64) o[64 * 64 + threadIdx.x] = threadIdx.x < nbw ? tau[threadIdx.x] : 0.0;
+}
+
+// --------------------------------------------------------------------------
+// W' = T^T W from the partials by substitution,
+//   w'_j = tau_j (w_j - sum_{q<j} G[q,j] w'_q),
+// written as the digit image of X -= V W': column c scaled by the largest
+// |W'(a, c)| 2^(f_a), f_a the exponent of reflector a.  The entries stay
+// unscaled while they are folded in (Gt carries tau), so a step is one shuffle
+// and one FMA per 32 rows still to come.  One warp holds CPW columns (two rows
+// a lane each).  Bound by the FP64 pipe: 96 FMAs a column and the sum of its
+// partials.
+// --------------------------------------------------------------------------
+template <int CPW>
+__global__ void __launch_bounds__(256)
+fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restrict__ wy,
+             const double *__restrict__ Gt, int nbw, unsigned char *__restrict__ Wimg,
+             int *__restrict__ ecol) {
+  constexpr int NB = 64, WARPS = CPW == 1 ? 1 : 8;   // (CPW 1: all threads sum one column)
+  __shared__ double G[NB * NB];
+  __shared__ double part[4][NB];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c0 = (blockIdx.x * WARPS + (CPW == 1 ? 0 : warp)) * CPW;
   {
-    double gv[16];
+    double2 gv[8];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) gv[u] = wy[(size_t)NB * NB + tid + u * 256];
+    for (int u = 0; u < 8; ++u) gv[u] = ((const double2 *)Gt)[tid + u * 256];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int idx = tid + u * 256;
-      G[(idx % NB) * GLD + idx / NB] = gv[u];
+    for (int u = 0; u < 8; ++u) ((double2 *)G)[tid + u * 256] = gv[u];
+  }
+  const double t0 = Gt[NB * NB + lane], t1 = Gt[NB * NB + lane + 32];
+  const double u0 = wy[lane * 65], u1 = wy[(lane + 32) * 65];     // up
+  const size_t stride = (size_t)N * NB;
+  double r0[CPW], r1[CPW];
+  if constexpr (CPW == 1) {
+    const double *src = Wp + (size_t)c0 * NB + (tid & 63);
+    double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+    int s = tid >> 6;
+    for (; s + 12 < S; s += 16) {
+      a0 += src[s * stride];
+      a1 += src[(s + 4) * stride];
+      a2 += src[(s + 8) * stride];
+      a3 += src[(s + 12) * stride];
     }
-  }
-  if (tid < NB) {
-    tau[tid] = wy[2 * (size_t)NB * NB + tid];
-    const double up = wy[tid * 65];
-    s_f[tid] = up == 0.0 ? 0 : fx_exp_of_hi(fx_hi(up));
-  }
-  const int c0 = blockIdx.x * COLS;
-  {
-    const int e = tid % (COLS * NB), h = tid / (COLS * NB);
-    const int c = e / NB, a = e - c * NB;
-    double acc0 = 0, acc1 = 0, acc2 = 0, acc3 = 0;
-    if (c0 + c < N) {
-      const double *src = Wp + (size_t)(c0 + c) * NB + a;
-      const size_t stride = (size_t)N * NB;
-      int s = h;
-      for (; s + 3 * TPE < S; s += 4 * TPE) {
-        acc0 += src[(size_t)s * stride];
-        acc1 += src[(size_t)(s + TPE) * stride];
-        acc2 += src[(size_t)(s + 2 * TPE) * stride];
-        acc3 += src[(size_t)(s + 3 * TPE) * stride];
+    for (; s < S; s += 4) a0 += src[s * stride];
+    part[tid >> 6][tid & 63] = (a0 + a1) + (a2 + a3);
+  } else {
+#pragma unroll
+    for (int k = 0; k < CPW; ++k) {
+      const double *src = Wp + (size_t)min(c0 + k, N - 1) * NB + lane;
+      double a0 = 0, a1 = 0, b0 = 0, b1 = 0;
+      int s = 0;
+      for (; s + 1 < S; s += 2) {
+        a0 += src[s * stride];
+        b0 += src[s * stride + 32];
+        a1 += src[(s + 1) * stride];
+        b1 += src[(s + 1) * stride + 32];
       }
-      for (; s < S; s += TPE) acc0 += src[(size_t)s * stride];
-    }
-    part[h][e] = (acc0 + acc1) + (acc2 + acc3);
-  }
-  __syncthreads();
-  if (tid < COLS * NB) {
-    double v = part[0][tid];
-#pragma unroll
-    for (int h = 1; h < TPE; ++h) v += part[h][tid];
-    w[tid / NB][tid % NB] = v;
-  }
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31;
-  if (warp >= COLS || c0 + warp >= N) return;
-  const int c = c0 + warp;
-  double r0 = w[warp][lane], r1 = w[warp][lane + 32];
-  for (int j = 0; j < nbw; ++j) {
-    const double wj = __shfl_sync(0xffffffffu, (j < 32) ? r0 : r1, j & 31);
-    const double wpj = tau[j] * wj;
-    if (lane > j) r0 = fma(-G[j * GLD + lane], wpj, r0);
-    if (lane + 32 > j) r1 = fma(-G[j * GLD + lane + 32], wpj, r1);
-    if (lane == (j & 31)) {
-      if (j < 32) r0 = wpj;
-      else r1 = wpj;
+      if (s < S) {
+        a0 += src[s * stride];
+        b0 += src[s * stride + 32];
+      }
+      r0[k] = a0 + a1;
+      r1[k] = b0 + b1;
     }
   }
-  if (lane >= nbw) r0 = 0.0;
-  if (lane + 32 >= nbw) r1 = 0.0;
-  const int f0 = s_f[lane], f1 = s_f[lane + 32];
-  int key = max(fx_key(r0, f0), fx_key(r1, f1));
-  key = __reduce_max_sync(0xffffffffu, key);
-  const bool bad = __any_sync(0xffffffffu, fx_hi(r0) >= 0x7ff00000u || fx_hi(r1) >= 0x7ff00000u);
-  const int g = (key == kFxZero) ? 0 : fx_exp(key);
-  unsigned char *dst = Wimg + (size_t)(c >> 5) * kFxWTile + (c & 31) * 128;
-  const unsigned long long y0 = fx_digits(r0, g - f0), y1 = fx_digits(r1, g - f1);
-  const int sw = (c & 7) << 4;
-#pragma unroll
-  for (int i = 0; i < kFxD; ++i) {
-    const int b = 8 * (6 - i);
-    const uint32_t v = fx_half2((uint32_t)(y0 >> b) & 0xff, (uint32_t)(y1 >> b) & 0xff, 0);
-    *(unsigned short *)(dst + i * 4096 + ((lane * 2) ^ sw)) = (unsigned short)(v & 0xffff);
-    *(unsigned short *)(dst + i * 4096 + ((64 + lane * 2) ^ sw)) = (unsigned short)(v >> 16);
+  __syncthreads();
+  if (warp >= WARPS || c0 >= N) return;
+  if constexpr (CPW == 1) {
+    r0[0] = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
+    r1[0] = (part[0][lane + 32] + part[1][lane + 32]) + (part[2][lane + 32] + part[3][lane + 32]);
   }
-  if (lane == 0) ecol[c] = bad ? kFxNonFinite : g;
+  // (on and below the diagonal Gt is zero, but a product with an entry that is
+  // not finite would not be)
+  for (int j = 0; j < min(nbw, 32); ++j) {
+    const double g0 = -G[j * NB + lane], g1 = -G[j * NB + lane + 32];
+#pragma unroll
+    for (int k = 0; k < CPW; ++k) {
+      const double wj = __shfl_sync(0xffffffffu, r0[k], j);
+      if (lane > j) r0[k] = fma(g0, wj, r0[k]);
+      r1[k] = fma(g1, wj, r1[k]);
+    }
+  }
+  for (int j = 32; j < nbw; ++j) {
+    const double g1 = -G[j * NB + lane + 32];
+#pragma unroll
+    for (int k = 0; k < CPW; ++k) {
+      const double wj = __shfl_sync(0xffffffffu, r1[k], j - 32);
+      if (lane + 32 > j) r1[k] = fma(g1, wj, r1[k]);
+    }
+  }
+  const int f0 = u0 == 0.0 ? 0 : fx_exp_of_hi(fx_hi(u0));
+  const int f1 = u1 == 0.0 ? 0 : fx_exp_of_hi(fx_hi(u1));
+#pragma unroll
+  for (int k = 0; k < CPW; ++k) {
+    const int c = c0 + k;
+    if (c >= N) break;
+    const double w0 = lane < nbw ? r0[k] * t0 : 0.0, w1 = lane + 32 < nbw ? r1[k] * t1 : 0.0;
+    int key = max(fx_key(w0, f0), fx_key(w1, f1));
+    key = __reduce_max_sync(0xffffffffu, key);
+    const bool bad =
+        __any_sync(0xffffffffu, fx_hi(w0) >= 0x7ff00000u || fx_hi(w1) >= 0x7ff00000u);
+    const int g = (key == kFxZero) ? 0 : fx_exp(key);
+    unsigned char *dst = Wimg + (size_t)(c >> 5) * kFxWTile + (c & 31) * 128;
+    const unsigned long long y0 = fx_digits(w0, g - f0), y1 = fx_digits(w1, g - f1);
+    const int sw = (c & 7) << 4;
+#pragma unroll
+    for (int i = 0; i < kFxD; ++i) {
+      const int b = 8 * (6 - i);
+      const uint32_t v = fx_half2((uint32_t)(y0 >> b) & 0xff, (uint32_t)(y1 >> b) & 0xff, 0);
+      *(unsigned short *)(dst + i * 4096 + ((lane * 2) ^ sw)) = (unsigned short)(v & 0xffff);
+      *(unsigned short *)(dst + i * 4096 + ((64 + lane * 2) ^ sw)) = (unsigned short)(v >> 16);
+    }
+    if (lane == 0) ecol[c] = bad ? kFxNonFinite : g;
+  }
 }
 
 // --------------------------------------------------------------------------
 // X(i, c) -= sum_a V(i, a) W'(a, c): a CTA keeps the digits of 128 rows of V
-// and goes through `per` tiles of 32 columns, the MMAs of the next tile running
-// behind the reassembly of this one (two sets of eight 32-column accumulators
-// fill tensor memory).  A thread owns one row and 8 columns of a tile: TMEM
-// lane = row, so X is read and written in 256-byte runs.  The new values'
-// column maxima (rows >= 64, those of the next panel) go to cnext.
+// and goes through `per` tiles of 32 columns.  Warp 16 fetches W' and issues
+// the MMAs, a tile ahead of the reassembly (two sets of eight 32-column
+// accumulators fill tensor memory); the sixteen worker warps are coupled to it
+// by mbarriers only and read X of the next tile before they reassemble this
+// one.  A thread owns one row and 8 columns of a tile: TMEM lane = row, so X is
+// read and written in 256-byte runs.  The new values' column maxima (rows >= 64,
+// those of the next panel) go to cnext.
 // grid: (ceil(M / 128), groups of `per` tiles)
 // --------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFxThreads, 1)
@@ -603,154 +840,143 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
   unsigned char *base = (unsigned char *)(((uintptr_t)fx_smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char *Ws = base + kFxV2Tile;
   __shared__ uint32_t s_taddr;
-  __shared__ __align__(8) uint64_t s_vfull, s_wfull[2], s_mma[2];
-  __shared__ unsigned s_cm[2][32];
-  __shared__ int s_ok;
+  // copies landed; a tile's MMAs done, its accumulators read
+  __shared__ __align__(8) uint64_t s_vfull, s_wfull[2], s_mma[2], s_free[2];
+  __shared__ int s_ecol[32 * kFxMaxPer];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ntiles = (N + 31) / 32;
   const int t_begin = blockIdx.y * per, T = min(ntiles, t_begin + per) - t_begin;
   const int i0 = blockIdx.x * 128;
 
+  for (int idx = tid; idx < 32 * T; idx += kFxThreads)
+    s_ecol[idx] = t_begin * 32 + idx < N ? ecol[t_begin * 32 + idx] : 0;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
                  :: "r"(smem_u32(&s_taddr)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_vfull)));
+    fx_mbar_init(&s_vfull, 1);
     for (int st = 0; st < 2; ++st) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_wfull[st])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&s_mma[st])));
+      fx_mbar_init(&s_wfull[st], 1);
+      fx_mbar_init(&s_mma[st], 1);
+      fx_mbar_init(&s_free[st], kFxWorkers);
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
-    s_ok = 1;
   }
-  if (tid < 64) s_cm[tid >> 5][tid & 31] = 0;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t taddr = s_taddr;
 
-  int issued = 0;                                        // W' copies (thread 0)
-  auto load_w = [&](int t) {
-    fx_bulk(smem_u32(Ws + (t & 1) * kFxWTile), Wimg + (size_t)(t_begin + t) * kFxWTile, kFxWTile,
-            &s_wfull[t & 1]);
-    ++issued;
-  };
-  auto mma_tile = [&](int t) {                           // thread 0
-    const int st = t & 1;
-    if (!mbar_wait(smem_u32(&s_wfull[st]), (uint32_t)((t >> 1) & 1))) {
-      s_ok = 0;
-      return;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t va = smem_u32(base), wb = smem_u32(Ws + st * kFxWTile);
-    const uint32_t acc0 = taddr + (uint32_t)(st * 256);
-#pragma unroll
-    for (int ks = 0; ks < 4; ++ks) {
-      auto piece = [&](int i, int n0, int n, bool ac) {
-        fx_mma(acc0 + (uint32_t)(i * 32 + n0), sw128_desc(va + i * 16384 + ks * 32),
-               sw128_desc(wb + n0 * 128 + ks * 32), n, ac);
+  if (warp == kFxWorkers) {                              // ---- copies and MMAs -------------
+    if (lane == 0) {
+      int issued = 0;
+      auto load_w = [&](int t) {
+        fx_bulk(smem_u32(Ws + (t & 1) * kFxWTile), Wimg + (size_t)(t_begin + t) * kFxWTile,
+                kFxWTile, &s_wfull[t & 1]);
+        ++issued;
       };
-      piece(0, 0, 224, ks > 0);
-      piece(1, 0, 192, true); piece(1, 192, 32, ks > 0);
-      piece(2, 0, 192, true);
-      piece(3, 0, 160, true);
-      piece(4, 0, 128, true);
-      piece(5, 0, 96, true);
-      piece(6, 0, 64, true);
-    }
-    fx_commit(&s_mma[st]);
-  };
-  if (tid == 0) {
-    fx_bulk(smem_u32(base), V2 + (size_t)blockIdx.x * kFxV2Tile, kFxV2Tile, &s_vfull);
-    load_w(0);
-    if (T > 1) load_w(1);
-    if (!mbar_wait(smem_u32(&s_vfull), 0)) s_ok = 0;
-    else mma_tile(0);
-  }
-  // this thread's row of the tile and its 8 columns
-  const int q = warp & 3, h = warp >> 2;
-  const int i = i0 + q * 32 + lane;
-  const bool row_ok = i < M;
-  const int er = erow[i];                                // (defined up to the whole tile)
-  double *xrow = X + k0 + i + (i >= nbw ? skip : 0);
-  const bool next_row = row_ok && i >= 64;
-  bool ok = true;
-  for (int t = 0; t < T; ++t) {
-    const int buf = t & 1;
-    const int cb = (t_begin + t) * 32 + h * 8;
-    double x[8];
+      fx_bulk(smem_u32(base), V2 + (size_t)blockIdx.x * kFxV2Tile, kFxV2Tile, &s_vfull);
+      load_w(0);
+      if (T > 1) load_w(1);
+      bool ok = mbar_wait(smem_u32(&s_vfull), 0);
+      for (int t = 0; t < T && ok; ++t) {
+        const int st = t & 1;
+        ok = mbar_wait(smem_u32(&s_wfull[st]), (uint32_t)((t >> 1) & 1));
+        if (ok && t >= 2) ok = mbar_wait(smem_u32(&s_free[st]), (uint32_t)((t / 2 - 1) & 1));
+        if (!ok) break;                                  // (the workers' waits run out too)
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t va = smem_u32(base), wb = smem_u32(Ws + st * kFxWTile);
+        const uint32_t acc0 = taddr + (uint32_t)(st * 256);
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      x[k] = (row_ok && cb + k < N) ? xrow[(size_t)(cb + k) * ldx] : 0.0;
-    if (tid == 0 && t + 1 < T) mma_tile(t + 1);
-    ok = mbar_wait(smem_u32(&s_mma[buf]), (uint32_t)((t >> 1) & 1));
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (tid == 0 && ok && t + 2 < T) load_w(t + 2);       // this tile's W' has been read
-    if (tid < 32 && t > 0) {                              // maxima of the tile before
-      const unsigned v = s_cm[buf ^ 1][tid];
-      const int c = (t_begin + t - 1) * 32 + tid;
-      if (cnext && v && c < N) atomicMax(cnext + c, v);
-      s_cm[buf ^ 1][tid] = 0;
-    }
-    ok = __all_sync(0xffffffffu, ok);                     // (converged for tcgen05.ld)
-    if (ok) {
-      long long hi[8], lo[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) hi[k] = lo[k] = 0;
-#pragma unroll
-      for (int o = 0; o < kFxOrders; ++o) {
-        uint32_t r[8];
-        FX_LD8(r, taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + o * 32 + h * 8));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int w = 1 << (8 * (3 - (o & 3)));
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const long long v = (long long)__float2int_rn(__uint_as_float(r[k])) * w;
-          if (o < 4) hi[k] += v;
-          else lo[k] += v;
+        for (int ks = 0; ks < 4; ++ks) {
+          auto piece = [&](int i, int n0, int n, bool ac) {
+            fx_mma(acc0 + (uint32_t)(i * 32 + n0), sw128_desc(va + i * 16384 + ks * 32),
+                   sw128_desc(wb + n0 * 128 + ks * 32), n, ac);
+          };
+          piece(0, 0, 224, ks > 0);
+          piece(1, 0, 192, true); piece(1, 192, 32, ks > 0);
+          piece(2, 0, 192, true);
+          piece(3, 0, 160, true);
+          piece(4, 0, 128, true);
+          piece(5, 0, 96, true);
+          piece(6, 0, 64, true);
+        }
+        fx_commit(&s_mma[st]);
+        if (t >= 1 && t + 1 < T) {                       // the stage of tile t - 1 is free
+          ok = mbar_wait(smem_u32(&s_mma[st ^ 1]), (uint32_t)(((t - 1) >> 1) & 1));
+          if (ok) load_w(t + 1);
         }
       }
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int c = cb + k;
-        const int g = (c < N) ? ecol[c] : 0;
-        // sum = (hi 2^72 + lo 2^40) 2^(er + g - 110), kept to 2^54 of those
-        // units in 63 bits: |hi| < 2^45 (the leading order sums 64 products)
-        const long long tt = (hi[k] << 18) + ((lo[k] + (1 << 13)) >> 14);
-        const int sh = er + g - 56;
-        double v;
-        if (sh >= -1000 && sh <= 900)
-          v = fma(-__longlong_as_double((long long)(sh + 1023) << 52), (double)tt, x[k]);
-        else
-          v = g == kFxNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
-                                : x[k] - scalbn((double)tt, sh);
-        x[k] = v;
+      if (!ok) {
+        mbar_wait(smem_u32(&s_vfull), 0);                // let the copies in flight land
+        for (int t = max(0, issued - 2); t < issued; ++t)
+          mbar_wait(smem_u32(&s_wfull[t & 1]), (uint32_t)((t >> 1) & 1));
+        atomicCAS(status, 0, SLQR_ETIMEOUT);
       }
+    }
+  } else {                                               // ---- reassembly ------------------
+    // this thread's row of the tile and its 8 columns
+    const int q = warp & 3, h = warp >> 2;
+    const int i = i0 + q * 32 + lane;
+    const bool row_ok = i < M;
+    const int er = erow[i] - 56;                         // (defined up to the whole tile)
+    double *xrow = X + k0 + i + (i >= nbw ? skip : 0) + (size_t)(t_begin * 32 + h * 8) * ldx;
+    const bool next_row = row_ok && i >= 64;
+    int c = t_begin * 32 + h * 8;
+    double xn[8];
+    auto load_x = [&]() {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) xn[k] = (row_ok && c + k < N) ? xrow[(size_t)k * ldx] : 0.0;
+    };
+    load_x();
+    for (int t = 0; t < T; ++t) {
+      const int buf = t & 1;
+      double x[8];
+      double *xw = xrow;
+      const int cw = c;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = xn[k];
+      xrow += (size_t)32 * ldx;
+      c += 32;
+      if (t + 1 < T) load_x();
+      const int *g = s_ecol + t * 32 + h * 8;
+      if (!fx_wait(&s_mma[buf], t >> 1)) {
+        if (lane == 0) atomicCAS(status, 0, SLQR_ETIMEOUT);
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ta = taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + h * 8);
       unsigned mine = 0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (row_ok && cb + k < N) xrow[(size_t)(cb + k) * ldx] = x[k];
-        const unsigned mx = __reduce_max_sync(0xffffffffu, next_row ? fx_hi(x[k]) : 0u);
-        if (lane == k) mine = mx;
+      for (int u = 0; u < 2; ++u) {
+        uint32_t r[kFxOrders][4];
+        fx_ld_orders(r, ta + (uint32_t)(u * 4), 32);
+        if (u == 1) {
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          if (lane == 0) fx_arrive(&s_free[buf]);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const int k = u * 4 + kk;
+          // orders 0..3 in units of 2^72, 4..7 in units of 2^40, of 2^(erow + g -
+          // 110); kept to 2^54 of those units in 63 bits: the first are below 2^45
+          // (the leading order sums 64 products)
+          const long long tt = (fx_four(r, 0, kk) << 18) + ((fx_four(r, 4, kk) + (1 << 13)) >> 14);
+          const int gk = g[k], sh = er + gk;
+          if (sh >= -1000 && sh <= 900)
+            x[k] -= fx_to_double(tt, sh);
+          else
+            x[k] = gk == kFxNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                      : x[k] - scalbn((double)tt, sh);
+          if (row_ok && cw + k < N) xw[(size_t)k * ldx] = x[k];
+          const unsigned mx = __reduce_max_sync(0xffffffffu, next_row ? fx_hi(x[k]) : 0u);
+          if (lane == k) mine = mx;
+        }
       }
-      if (lane < 8 && mine) atomicMax(&s_cm[buf][h * 8 + lane], mine);
+      if (cnext && lane < 8 && cw + lane < N && mine) atomicMax(cnext + cw + lane, mine);
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    if (!__syncthreads_and(ok && s_ok)) { ok = false; break; }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  }
-  if (ok && tid < 32 && T > 0) {
-    const unsigned v = s_cm[(T - 1) & 1][tid];
-    const int c = (t_begin + T - 1) * 32 + tid;
-    if (cnext && v && c < N) atomicMax(cnext + c, v);
-  }
-  if (!ok && tid == 0) {
-    mbar_wait(smem_u32(&s_vfull), 0);                     // let the copies in flight land
-    for (int t = max(0, issued - 2); t < issued; ++t)
-      mbar_wait(smem_u32(&s_wfull[t & 1]), (uint32_t)((t >> 1) & 1));
-    atomicCAS(status, 0, SLQR_ETIMEOUT);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -788,9 +1014,10 @@ size_t fx_v_bytes(int m) {
 }
 
 size_t fx_work_bytes(int m, int n, int num_sms) {
-  // partials: S N' <= (4 num_sms + tiles') 128 over every width N' <= n (fx_slices)
-  (void)m;
-  const size_t part = ((size_t)4 * num_sms + 2) * 128 + (size_t)n;
+  // partials: S N' <= (4 num_sms + tiles') 128 over every width N' <= n, and at
+  // most a slice per 128 rows (fx_slices)
+  const size_t part = std::min(((size_t)4 * num_sms + 2) * 128 + (size_t)n,
+                               ((size_t)m + 127) / 128 * (size_t)n);
   const size_t tiles = ((size_t)n + 31) / 32;
   return align_up(part * 64 * sizeof(double), 256) + tiles * kFxWTile +
          align_up(tiles * 32 * sizeof(int), 256);
@@ -805,9 +1032,36 @@ void fx_split_v(const double *A, int lda, const double *Vtop, int k0, int nbw, i
                                                               V2, erow);
 }
 
+static FxGram fx_gram_args(double *wy_panel, void *gram, double *Gt, int M, int ctas) {
+  FxGram gr;
+  gr.sum = (unsigned long long *)gram;
+  gr.arrived = (unsigned *)(gr.sum + 64 * 64);
+  gr.G = wy_panel + 64 * 64;
+  gr.Gt = Gt;
+  const int blocks = (M + 127) / 128;
+  gr.RS = (blocks + ctas - 1) / ctas * 128;
+  gr.slices = (M + gr.RS - 1) / gr.RS;
+  gr.vtx_slices = 0;
+  return gr;
+}
+
+void fx_gram(slqr_ctx *ctx, int nbw, int M, double *wy_panel, const void *vbuf, void *gram,
+             double *Gt, cudaStream_t stream) {
+  const FxGram gr = fx_gram_args(wy_panel, gram, Gt, M, ctx->num_sms);
+  int slot = prof_begin(ctx, stream);
+  fx_vtx_kernel<<<dim3(1, gr.slices), kFxThreads, kFxVtxSmem, stream>>>(
+      nullptr, 0, 0, nbw, 0, M, 0, 128, (const unsigned char *)vbuf, wy_panel, nullptr, nullptr, gr,
+      ctx->d_status);
+  prof_end(ctx, stream, slot, kVtx, 0.0);
+}
+
+void fx_prep(const double *wy, int K, int nb, double *Gt, cudaStream_t stream) {
+  fx_prep_kernel<<<num_panels(K, nb), 256, 0, stream>>>(wy, K, nb, Gt);
+}
+
 bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy_panel,
-               const void *vbuf, double *X, int ldx, int N, const unsigned *cmax, unsigned *cnext,
-               void *work, size_t work_bytes, cudaStream_t stream) {
+               const double *Gt, const void *vbuf, double *X, int ldx, int N, const unsigned *cmax,
+               unsigned *cnext, void *work, size_t work_bytes, cudaStream_t stream, void *gram) {
   int RS = 0;
   const int S = fx_slices(M, N, ctx->num_sms, &RS);
   const size_t tiles = ((size_t)M + 127) / 128, wt = ((size_t)N + 31) / 32;
@@ -820,21 +1074,28 @@ bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy
   int *ecol = (int *)(Wimg + wt * kFxWTile);
   const double flops = 2.0 * M * nbw * (double)N;
   int slot = prof_begin(ctx, stream);
-  fx_vtx_kernel<<<dim3((N + 127) / 128, S), kFxThreads, kFxVtxSmem, stream>>>(
-      X, ldx, k0, nbw, skip, M, N, RS, V1, wy_panel, cmax, Wp, ctx->d_status);
+  // the panel's Gram terms beside it, on the SMs the products leave (a quarter at least)
+  const int vt = (N + 127) / 128;
+  FxGram gr = fx_gram_args((double *)wy_panel, gram, (double *)Gt, M,
+                           std::max(ctx->num_sms / 4, ctx->num_sms - vt * S));
+  gr.vtx_slices = S;
+  fx_vtx_kernel<<<dim3(vt + (gram ? 1 : 0), std::max(S, gram ? gr.slices : 0)), kFxThreads,
+                  kFxVtxSmem, stream>>>(X, ldx, k0, nbw, skip, M, N, RS, V1, wy_panel, cmax, Wp, gr,
+                                        ctx->d_status);
   prof_end(ctx, stream, slot, kVtx, flops);
   slot = prof_begin(ctx, stream);
   if (N <= 4 * ctx->num_sms)
-    fx_tw_kernel<1><<<N, 256, 0, stream>>>(Wp, S, N, wy_panel, nbw, Wimg, ecol);
+    fx_tw_kernel<1><<<N, 256, 0, stream>>>(Wp, S, N, wy_panel, Gt, nbw, Wimg, ecol);
   else
-    fx_tw_kernel<4><<<(N + 3) / 4, 256, 0, stream>>>(Wp, S, N, wy_panel, nbw, Wimg, ecol);
+    fx_tw_kernel<2><<<(N + 15) / 16, 256, 0, stream>>>(Wp, S, N, wy_panel, Gt, nbw, Wimg, ecol);
   prof_end(ctx, stream, slot, kTw, (double)nbw * nbw * N);
   slot = prof_begin(ctx, stream);
   const int rt = (M + 127) / 128;
   // column tiles per CTA: about four waves of CTAs, at least 4 tiles each (the
   // V tile is 114 KB, as much as 3.5 tiles of X)
   const int groups = std::max(1, (4 * ctx->num_sms + rt - 1) / rt);
-  const int per = std::max(rt * (int)wt <= ctx->num_sms ? 1 : 4, ((int)wt + groups - 1) / groups);
+  const int per = std::min(
+      kFxMaxPer, std::max(rt * (int)wt <= ctx->num_sms ? 1 : 4, ((int)wt + groups - 1) / groups));
   fx_upd_kernel<<<dim3(rt, ((int)wt + per - 1) / per), kFxThreads, kFxUpdSmem, stream>>>(
       X, ldx, k0, nbw, skip, M, N, per, V2, erow, Wimg, ecol, cnext, ctx->d_status);
   prof_end(ctx, stream, slot, kUpd, flops);

@@ -102,3 +102,4 @@ def test_same_as_the_fp64_pipe(ctx, value, row, col):
         tol, _ = factor_tol(A)
         np.testing.assert_allclose(F, G, rtol=0, atol=tol)
         assert not np.array_equal(F, G)          # (the two paths round differently)
+
