@@ -136,20 +136,27 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
   const size_t gp_doubles = wy ? 0 : (size_t)np * Sg * NB * NB;
   const size_t work_doubles = panel_update_work_doubles(m, nrhs, NB, ctx->num_sms);
   const size_t head_bytes = align_up((wy_doubles + gp_doubles) * 8, 256);
-  // kFxMinCols right-hand sides and up: the products on the tensor cores
-  // (tc_fp64.cu), unless the scratch does not fit
+  // few right-hand sides: all panels in one launch (qt_vec.cu); kFxMinCols and
+  // up: the products on the tensor cores (tc_fp64.cu); unless the scratch of
+  // either does not fit
+  bool vec = nrhs < kFxMinCols && qt_vec_bytes(ctx, m, K, NB) > 0;
   bool fx = NB == 64 && nrhs >= kFxMinCols;
   const size_t fx_v = align_up(fx_v_bytes(m), 256);
   const size_t fx_work = align_up(fx_work_bytes(m, nrhs, ctx->num_sms), 256);
   const size_t fx_gt = (size_t)np * kFxGt * sizeof(double);
   slqr_status st = SLQR_OK;
+  if (vec) {
+    st = ensure_workspace(ctx, head_bytes + qt_vec_bytes(ctx, m, K, NB));
+    if (st == SLQR_EBUSY || st == SLQR_ENOMEM) vec = false;
+    else if (st != SLQR_OK) return st;
+  }
   if (fx) {
     st = ensure_workspace(ctx, head_bytes + fx_v + fx_work + fx_gt +
                                    (size_t)np * nrhs * sizeof(unsigned));
     if (st == SLQR_EBUSY || st == SLQR_ENOMEM) fx = false;
     else if (st != SLQR_OK) return st;
   }
-  if (!fx) st = ensure_workspace(ctx, head_bytes + work_doubles * 8 + 256);
+  if (!fx && !vec) st = ensure_workspace(ctx, head_bytes + work_doubles * 8 + 256);
   if (st != SLQR_OK) return st;
   double *base = (double *)ctx->ws.ptr;
   double *wy_store = base;
@@ -174,6 +181,10 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
     if (st != SLQR_OK) return st;
   }
   const double *wys = wy ? wy : wy_store;
+  if (vec) {
+    st = qt_vec(ctx, m, K, NB, A, lda, up, wys, nrhs, B, ldb, ntop, tail, stream);
+    return st != SLQR_OK ? st : check_launch(ctx, "Q^T b");
+  }
   if (fx) {
     fx_colmax(B, ldb, m, nrhs, ntop, false, cmax, np, ctx->num_sms, stream);
     fx_prep(wys, K, NB, gt, stream);

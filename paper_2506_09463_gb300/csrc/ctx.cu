@@ -241,7 +241,8 @@ extern "C" slqr_status slqr_create(slqr_ctx **out, int device, size_t hbm_budget
   if (init_kernel_attrs(ctx) != SLQR_OK || init_batch_attrs(ctx) != SLQR_OK ||
       init_tc_attrs(ctx) != SLQR_OK || init_bf16_attrs(ctx) != SLQR_OK ||
       init_cluster_attrs(ctx) != SLQR_OK || init_lookahead_attrs(ctx) != SLQR_OK ||
-      init_fx_attrs(ctx) != SLQR_OK || init_grid_panel_attrs(ctx) != SLQR_OK) {
+      init_fx_attrs(ctx) != SLQR_OK || init_grid_panel_attrs(ctx) != SLQR_OK ||
+      init_qt_vec_attrs(ctx) != SLQR_OK) {
     cudaEventDestroy(ctx->ev_start);
     cudaEventDestroy(ctx->ev_ready);
     cudaEventDestroy(ctx->ev_panel);

@@ -190,6 +190,15 @@ void fx_gram(slqr_ctx *ctx, int nbw, int M, double *wy_panel, const void *vbuf, 
              double *Gt, cudaStream_t stream);
 void fx_prep(const double *wy, int K, int nb, double *Gt, cudaStream_t stream);
 
+// B <- Q^T B for fewer than kFxMinCols right-hand sides in one launch for all
+// panels (qt_vec.cu), panels of nb reflectors (64 or 32) with their compact-WY
+// store; work: qt_vec_bytes (0: m is too tall for it).
+slqr_status init_qt_vec_attrs(slqr_ctx *ctx);
+size_t qt_vec_bytes(const slqr_ctx *ctx, int m, int K, int nb);
+slqr_status qt_vec(slqr_ctx *ctx, int m, int K, int nb, const double *A, int lda, const double *up,
+                   const double *wy, int nrhs, double *B, int ldb, int ntop, void *work,
+                   cudaStream_t stream);
+
 // slqr_batch_factor with a per-problem stacked top block (ntop[i] rows, 0 for a
 // dense problem; ntop may be NULL); takes the context mutex.
 slqr_status batch_factor_locked(slqr_ctx *ctx, int count, const int *m, const int *n,

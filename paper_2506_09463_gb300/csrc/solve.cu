@@ -21,7 +21,6 @@
 namespace slqr {
 
 constexpr int kTB = 64;    // rows per block of R
-constexpr int kRC = 16;    // right-hand sides per CTA
 
 // Rinv[b] = inverse of the upper-triangular diagonal block b (kTB x kTB,
 // column-major, zero-padded).  Thread j computes column j by back-substitution
@@ -63,81 +62,86 @@ trsm_inv_kernel(const double *__restrict__ A, int lda, int n, double *__restrict
   if (zero) atomicCAS(status, 0, SLQR_ERANK);
 }
 
-// grid: (blocks, ceil(nrhs / kRC)), row block t = t_first + blockIdx.x.
+// grid: (blocks, ceil(nrhs / RC)), row block t = t_first + blockIdx.x.
 // CTA t updates row block t with the x of block b_src (when b_src >= 0), and
 // CTA t == b_diag then replaces its right-hand sides by Rinv[t] times them.
+// A step is a chain of loads and of FP64 instructions (16 clocks of the SM's
+// FP64 pipe each), so a CTA takes few right-hand sides: RC = 4, a thread for
+// each row and right-hand side, or RC = 1, a thread for each row and quarter of
+// the columns (16 right-hand sides a CTA: 47 us a step whatever their number).
+template <int RC>
 __global__ void __launch_bounds__(kThreads)
 trsm_step_kernel(const double *__restrict__ A, int lda, int n, int nrhs, double *__restrict__ B,
                  int ldb, int t_first, int b_src, int b_diag, const double *__restrict__ Rinv) {
-  __shared__ double Rs[kTB][kTB + 1];   // R tile (or the block inverse) [row][col]
-  __shared__ double Xs[kRC][kTB + 1];   // x of block b_src, or the rhs being solved
+  constexpr int CQ = kThreads / kTB / RC;      // column splits
+  constexpr int CW = kTB / CQ;                 // columns of a split
+  constexpr int PER = kTB * kTB / kThreads;
+  __shared__ double Rs[kTB][kTB + 1];   // R tile (or the block inverse) [col][row]
+  __shared__ double Xs[RC][kTB];        // x of block b_src, or the rhs being solved
+  __shared__ double part[CQ][kTB];
   const int t = t_first + blockIdx.x;
-  const int r0 = blockIdx.y * kRC;
-  const int nr = min(kRC, nrhs - r0);
+  const int r0 = blockIdx.y * RC;
   const int tid = threadIdx.x;
   const int row_begin = t * kTB;
   const int rows = min(kTB, n - row_begin);
-  // thread -> (row r, rhs group g): 64 rows x 4 groups of 4 rhs
-  const int r = tid & (kTB - 1);
-  const int g = tid >> 6;
-
+  const int r = tid & (kTB - 1), g = tid >> 6;
+  const int q = RC > 1 ? g : 0, cs = RC > 1 ? 0 : g;
+  const bool rhs_ok = r0 + q < nrhs;
+  const bool diag = t == b_diag;
+  // everything this step reads of R, its inverse and B, in flight at once
+  double tile[PER], inv[PER];
+  double rhs = 0.0, xsrc = 0.0;
+  const int col_begin = b_src * kTB;
+  const int cols = b_src >= 0 ? min(kTB, n - col_begin) : 0;
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int c = g + u * (kThreads / kTB);
+    tile[u] = (r < rows && c < cols) ? A[SLQR_IDX(row_begin + r, col_begin + c, lda)] : 0.0;
+  }
+  if (diag) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+      inv[u] = Rinv[(size_t)t * kTB * kTB + tid + u * kThreads];
+  }
+  if (rhs_ok && cs == 0) {
+    if (r < rows) rhs = B[SLQR_IDX(row_begin + r, r0 + q, ldb)];
+    if (r < cols) xsrc = B[SLQR_IDX(col_begin + r, r0 + q, ldb)];
+  }
+  // this thread's part of row r of the tile times the vectors in Xs
+  auto product = [&]() {
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+    for (int c = 0; c < CW; c += 2) {
+      a0 = fma(Rs[cs * CW + c][r], Xs[q][cs * CW + c], a0);
+      a1 = fma(Rs[cs * CW + c + 1][r], Xs[q][cs * CW + c + 1], a1);
+    }
+    a0 += a1;
+    if (CQ > 1) {
+      part[cs][r] = a0;
+      __syncthreads();
+      a0 = part[0][r];
+#pragma unroll
+      for (int s = 1; s < CQ; ++s) a0 += part[s][r];
+    }
+    return a0;
+  };
   if (b_src >= 0) {
-    const int col_begin = b_src * kTB;
-    const int cols = min(kTB, n - col_begin);
-    for (int idx = tid; idx < kTB * kTB; idx += kThreads) {
-      int c = idx / kTB, rr = idx - c * kTB;
-      Rs[rr][c] = (rr < rows && c < cols) ? A[SLQR_IDX(row_begin + rr, col_begin + c, lda)] : 0.0;
-    }
-    for (int idx = tid; idx < kRC * kTB; idx += kThreads) {
-      int q = idx / kTB, c = idx - q * kTB;
-      Xs[q][c] = (q < nr && c < cols) ? B[SLQR_IDX(col_begin + c, r0 + q, ldb)] : 0.0;
-    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u) Rs[g + u * (kThreads / kTB)][r] = tile[u];
+    if (cs == 0) Xs[q][r] = xsrc;
     __syncthreads();
-    if (r < rows) {
-      double acc[kRC / 4];
-#pragma unroll
-      for (int q = 0; q < kRC / 4; ++q) acc[q] = 0.0;
-      for (int c = 0; c < cols; ++c) {
-        double rv = Rs[r][c];
-#pragma unroll
-        for (int q = 0; q < kRC / 4; ++q) acc[q] = fma(rv, Xs[g * (kRC / 4) + q][c], acc[q]);
-      }
-#pragma unroll
-      for (int q = 0; q < kRC / 4; ++q) {
-        int rr = g * (kRC / 4) + q;
-        if (rr < nr) B[SLQR_IDX(row_begin + r, r0 + rr, ldb)] -= acc[q];
-      }
-    }
+    rhs -= product();
+    if (!diag && rhs_ok && cs == 0 && r < rows) B[SLQR_IDX(row_begin + r, r0 + q, ldb)] = rhs;
     __syncthreads();
   }
-  if (t != b_diag) return;
-
+  if (!diag) return;
   // x of the diagonal block = Rinv[t] * (its updated right-hand sides)
-  const double *Ri = Rinv + (size_t)t * kTB * kTB;
-  for (int idx = tid; idx < kTB * kTB; idx += kThreads) {
-    int c = idx / kTB, rr = idx - c * kTB;
-    Rs[rr][c] = Ri[idx];
-  }
-  for (int idx = tid; idx < kRC * kTB; idx += kThreads) {
-    int q = idx / kTB, rr = idx - q * kTB;
-    Xs[q][rr] = (q < nr && rr < rows) ? B[SLQR_IDX(row_begin + rr, r0 + q, ldb)] : 0.0;
-  }
+#pragma unroll
+  for (int u = 0; u < PER; ++u) Rs[g + u * (kThreads / kTB)][r] = inv[u];
+  if (cs == 0) Xs[q][r] = (rhs_ok && r < rows) ? rhs : 0.0;
   __syncthreads();
-  if (r < rows) {
-    double acc[kRC / 4];
-#pragma unroll
-    for (int q = 0; q < kRC / 4; ++q) acc[q] = 0.0;
-    for (int c = r; c < rows; ++c) {                 // the inverse is upper triangular
-      double rv = Rs[r][c];
-#pragma unroll
-      for (int q = 0; q < kRC / 4; ++q) acc[q] = fma(rv, Xs[g * (kRC / 4) + q][c], acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < kRC / 4; ++q) {
-      int rr = g * (kRC / 4) + q;
-      if (rr < nr) B[SLQR_IDX(row_begin + r, r0 + rr, ldb)] = acc[q];
-    }
-  }
+  const double x = product();
+  if (rhs_ok && cs == 0 && r < rows) B[SLQR_IDX(row_begin + r, r0 + q, ldb)] = x;
 }
 
 }  // namespace slqr
@@ -158,7 +162,19 @@ extern "C" slqr_status slqr_solve_r(slqr_ctx *ctx, int n, const double *A, int l
   if (e != cudaSuccess) return fail(ctx, SLQR_ECUDA, "cudaSetDevice: %s", cudaGetErrorString(e));
   cudaStream_t s = (cudaStream_t)stream;
   const int nblk = (n + kTB - 1) / kTB;
-  const int gy = (nrhs + kRC - 1) / kRC;
+  const int RC = nrhs <= 2 ? 1 : 4;
+  const int gy = (nrhs + RC - 1) / RC;
+  auto step = [&](int blocks, int b_src, int b_diag, double fl) {
+    int slot = prof_begin(ctx, s);
+    const int first = b_src < 0 ? b_diag : 0;
+    if (RC == 1)
+      trsm_step_kernel<1><<<dim3(blocks, gy), kThreads, 0, s>>>(
+          A, lda, n, nrhs, B, ldb, first, b_src, b_diag, (const double *)ctx->ws.ptr);
+    else
+      trsm_step_kernel<4><<<dim3(blocks, gy), kThreads, 0, s>>>(
+          A, lda, n, nrhs, B, ldb, first, b_src, b_diag, (const double *)ctx->ws.ptr);
+    prof_end(ctx, s, slot, kTrsm, fl);
+  };
   slqr_status st = ensure_workspace(ctx, (size_t)nblk * kTB * kTB * sizeof(double));
   if (st != SLQR_OK) return st;
   double *Rinv = (double *)ctx->ws.ptr;
@@ -167,17 +183,9 @@ extern "C" slqr_status slqr_solve_r(slqr_ctx *ctx, int n, const double *A, int l
   trsm_inv_kernel<<<nblk, kTB, 0, s>>>(A, lda, n, Rinv, ctx->d_status);
   prof_end(ctx, s, slot, kTrsm, 0.0);
   // first launch: only the last diagonal block
-  double fl = (double)rows_of(nblk - 1) * rows_of(nblk - 1) * nrhs;
-  slot = prof_begin(ctx, s);
-  trsm_step_kernel<<<dim3(1, gy), kThreads, 0, s>>>(A, lda, n, nrhs, B, ldb, nblk - 1, -1,
-                                                     nblk - 1, Rinv);
-  prof_end(ctx, s, slot, kTrsm, fl);
-  for (int b = nblk - 1; b >= 1; --b) {
-    // update of rows [0, b*kTB) by block b, then the diagonal block b-1
-    fl = 2.0 * b * kTB * rows_of(b) * nrhs + (double)kTB * kTB * nrhs;
-    slot = prof_begin(ctx, s);
-    trsm_step_kernel<<<dim3(b, gy), kThreads, 0, s>>>(A, lda, n, nrhs, B, ldb, 0, b, b - 1, Rinv);
-    prof_end(ctx, s, slot, kTrsm, fl);
-  }
+  step(1, -1, nblk - 1, (double)rows_of(nblk - 1) * rows_of(nblk - 1) * nrhs);
+  // update of rows [0, b*kTB) by block b, then the diagonal block b-1
+  for (int b = nblk - 1; b >= 1; --b)
+    step(b, b, b - 1, 2.0 * b * kTB * rows_of(b) * nrhs + (double)kTB * kTB * nrhs);
   return check_launch(ctx, "solve_r");
 }

@@ -103,3 +103,32 @@ def test_same_as_the_fp64_pipe(ctx, value, row, col):
         np.testing.assert_allclose(F, G, rtol=0, atol=tol)
         assert not np.array_equal(F, G)          # (the two paths round differently)
 
+
+# right-hand sides of one launch (1, 2, 4) and remainders; rows per CTA 32, 64,
+# 128 with one cluster and several; panels of 32 and 64, a ragged last one
+@pytest.mark.parametrize("m,n", [(200, 150), (700, 321), (2200, 130), (4300, 260), (8300, 70)])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 5, 15])
+@pytest.mark.parametrize("use_wy", [True, False])
+def test_apply_qt_few_right_hand_sides(ctx, m, n, nrhs, use_wy):
+    A, _ = workloads.gaussian(m, n, seed=m + nrhs)
+    B = workloads.gaussian_rhs(m, nrhs, seed=nrhs)
+    Ad, Bd = dev(A), dev(B)
+    up = torch.empty(n, dtype=torch.float64, device="cuda")
+    wy = ctx.wy_buffer(m, n) if use_wy else None
+    ctx.factor(Ad, up, wy)
+    ctx.apply_qt(Ad, up, Bd, wy=wy)
+    ctx.solve_r(Ad, Bd)
+    assert ctx.sync() == 0
+    F, upf, out = host(Ad), host(up), host(Bd)
+    for j in range(nrhs):
+        b = np.ascontiguousarray(B[:, j])
+        qtb = oracle.apply_qt(F, upf, b)
+        x, _ = oracle.solve_r(F, qtb)
+        # the same factorization applied: Q^T b to the summation's rounding, x by
+        # the condition of R
+        np.testing.assert_allclose(out[n:, j], qtb[n:], rtol=0,
+                                   atol=4.0 * np.sqrt(m) * U * np.linalg.norm(b) * np.sqrt(n))
+        kappa = np.linalg.cond(np.triu(F[:n]))
+        assert np.linalg.norm(out[:n, j] - x) <= 64.0 * kappa * U * np.sqrt(n) * \
+            np.linalg.norm(b) / np.linalg.norm(A, 2) + 64.0 * kappa * U * np.linalg.norm(x)
+
