@@ -1539,10 +1539,21 @@ slqr_status factor_f32(slqr_ctx *ctx, int m, int n, float *A, int lda, double *u
 }
 
 
+// The FP64 factorization.  Few columns (n <= 256) have a compact-WY store in
+// panels of 32; unless that width was set (slqr_set_tuning, slqr_autotune) they
+// are factored in panels of 64 all the same, whose panel and update kernels are
+// the faster ones (256 x 128: 0.42 against 0.92 ms), and the store is taken from
+// theirs.
 static slqr_status factor_fp64(slqr_ctx *ctx, int m, int n, double *A, int lda, double *up,
                                double *wy, cudaStream_t s, int ntop) {
-  if (panel_width(m, n) == 32) return factor_impl<double, 32>(ctx, m, n, A, lda, up, wy, s, ntop);
-  return factor_impl<double, 64>(ctx, m, n, A, lda, up, wy, s, ntop);
+  TuneEntry tuned;
+  if (panel_width(m, n) == 64) return factor_impl<double, 64>(ctx, m, n, A, lda, up, wy, s, ntop);
+  if (g_tune_nb != 32 && !tune_lookup(m, n, &tuned)) {
+    const slqr_status st = factor_impl<double, 64>(ctx, m, n, A, lda, up, nullptr, s, ntop, wy);
+    // (a workspace that does not fit: nothing was enqueued)
+    if (st != SLQR_EBUSY && st != SLQR_ENOMEM) return st;
+  }
+  return factor_impl<double, 32>(ctx, m, n, A, lda, up, wy, s, ntop);
 }
 
 }  // namespace slqr

@@ -132,3 +132,31 @@ def test_apply_qt_few_right_hand_sides(ctx, m, n, nrhs, use_wy):
         assert np.linalg.norm(out[:n, j] - x) <= 64.0 * kappa * U * np.sqrt(n) * \
             np.linalg.norm(b) / np.linalg.norm(A, 2) + 64.0 * kappa * U * np.linalg.norm(x)
 
+
+@pytest.mark.parametrize("m,n", [(64, 32), (70, 69), (256, 128), (300, 200), (257, 256)])
+def test_compact_wy_of_few_columns(ctx, m, n):
+    """Panels of 32 in the store, factored in panels of 64: the store's blocks against
+    V of the factorization (G = striu(V^T V), tau = -1 / (up R_kk))."""
+    A, _ = workloads.gaussian(m, n, seed=m)
+    Ad = dev(A)
+    up = torch.empty(n, dtype=torch.float64, device="cuda")
+    wy = ctx.wy_buffer(m, n)
+    wy.fill_(float("nan"))
+    ctx.factor(Ad, up, wy)
+    assert ctx.sync() == 0
+    F, u, store = host(Ad), host(up), host(wy)
+    K = min(m - 1, n)
+    V = np.tril(F, -1)[:, :K] + np.vstack([np.diag(u[:K]), np.zeros((m - K, K))])
+    size = 2 * 32 * 32 + 32
+    for p in range((K + 31) // 32):
+        k0, w = 32 * p, min(32, K - 32 * p)
+        blk = store[p * size:(p + 1) * size]
+        Vp = V[k0:, k0:k0 + w]
+        vtop = blk[:1024].reshape(32, 32).T
+        np.testing.assert_array_equal(vtop[:min(w, m - k0), :w], Vp[:w][:, :w])
+        G = blk[1024:2048].reshape(32, 32).T[:w, :w]
+        want = np.triu(Vp.T @ Vp, 1)
+        nrm = np.linalg.norm(Vp, axis=0)
+        assert np.all(np.abs(np.triu(G, 1) - want) <= 4.0 * np.sqrt(m) * U * np.outer(nrm, nrm))
+        tau = -1.0 / (u[k0:k0 + w] * np.diag(F)[k0:k0 + w])
+        np.testing.assert_allclose(blk[2048:2048 + w], tau, rtol=16 * U)
