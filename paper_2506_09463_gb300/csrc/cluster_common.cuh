@@ -160,13 +160,19 @@ __device__ __forceinline__ void mbar_expect(unsigned long long *mbar, unsigned b
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                ::"r"((unsigned)__cvta_generic_to_shared(mbar)), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(unsigned long long *mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];"
+               ::"r"((unsigned)__cvta_generic_to_shared(mbar)) : "memory");
+}
 // Bounded wait for the phase of the given parity.  Past `report` polls (the
 // context's spin limit) it records SLQR_ETIMEOUT once but goes on waiting, up
 // to kSpinLimit polls, so that normally no store of the column is still in
 // flight when the kernel moves on (the stores come from CTAs of the same
-// cluster, all resident); false only when even that limit ran out.
+// cluster, all resident); false only when even that limit ran out.  It polls
+// without a pause `awake` times.
 __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *mbar, unsigned parity,
-                                                  unsigned report, int *status, bool *reported) {
+                                                  unsigned report, int *status, bool *reported,
+                                                  unsigned awake = 64) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(mbar);
   for (unsigned it = 0;; ++it) {
     unsigned done;
@@ -179,7 +185,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *mbar, unsi
       *reported = true;
     }
     if (it >= kSpinLimit) return false;
-    if (it > 64) __nanosleep(32);
+    if (it > awake) __nanosleep(32);
   }
 }
 

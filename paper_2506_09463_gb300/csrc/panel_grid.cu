@@ -7,9 +7,10 @@
 // Gram terms of V^T V, a third of the panel's FP64 work there, are formed from
 // the digits of V instead (fx_gram_block in tc_fp64.cu).
 //
-// What bounds a column step: every FP64 warp instruction holds the SM's FP64
-// pipe for 16 clocks, and the step is a chain of two passes over the slice, a
-// sum over all CTAs and the pivot's square root and division.  So:
+// What bounds a column step: every FP64 warp instruction takes the SM's FP64
+// pipe for 16 clocks, the next one of the same warp starts 64 clocks later, and
+// the step is a chain of two passes over the slice, a sum over all CTAs and the
+// pivot's square root and division.  So:
 //  * The slice is spread over many CTAs (R = 32 .. 256 rows each) and lives in
 //    registers: warp w holds columns 4 w .. 4 w + 3, eight lanes to a column,
 //    lane l of them rows l, l + 8, ...  A column's dot needs three butterfly
@@ -18,13 +19,24 @@
 //  * Partial dots go out straight from registers.  Up to 16 CTAs are one
 //    cluster: each warp pushes its columns' partials to every CTA (st.async,
 //    counted on an mbarrier there).  More CTAs are clusters of 8 or 4: the
-//    partials of a column go to one CTA of the cluster, which adds them and
-//    publishes the sum in L2, and every warp collects the clusters' sums of its
-//    own columns.  (Without the first level every CTA reads every CTA's record:
-//    128 CTAs spent 3.5 us of a 7.4 us step in those reads.)
-//  * The only CTA barriers of a step are the two that hand over the pivot (from
-//    the warp of column j) and the next column (through shared memory).
+//    partials of a column go to one CTA of the cluster, whose collecting warp
+//    adds them and publishes the sum in L2; every CTA polls the clusters' sums.
+//    (Without the first level every CTA reads every CTA's record: 128 CTAs spent
+//    3.5 us of a 7.4 us step in those reads; norms alone sent that way, around
+//    the first level, cost 0.8 us a step on 64 CTAs.)
+//  * The sums over all CTAs are taken by four warps, 16 columns each, so that at
+//    most five warps share the pipe with the pivot's chain.  (On all sixteen,
+//    four columns each, the sums took 1200 clocks of a step and the chain 1700:
+//    3.0 us a column at 512 rows against 2.5, 4.4 against 3.6 at 2048.)
+//  * A reflector is applied and the next column's dots are taken in one go: the
+//    next column's warp hands it over through shared memory and goes on, and one
+//    CTA barrier a step, after the multipliers, is left.  In one cluster its
+//    partials are counted apart from the others', so that the pivot starts while
+//    the other columns' sums are still coming.
+// Microseconds a column (with 64 columns): 2.5 at 512 rows, 3.4 at 1100, 3.6 at
+// 2048, 4.2 at 4096; panel_kernel took 9.8 at 8192.
 #include "cluster_common.cuh"
+#include "pivot_fp64.cuh"
 
 #include <algorithm>
 
@@ -35,7 +47,9 @@ namespace {
 
 constexpr int kGpThreads = 512;
 constexpr int kNB = 64;
-constexpr int kGpPolls = 5;            // sums of other clusters a lane collects (40 clusters)
+constexpr int kGpPolls = 5;            // clusters' sums a lane collects (40 clusters at most)
+constexpr int kGpPivot = 3;            // the warp of the pivot
+constexpr int kGpCollector = 5;        // the warp that adds up a cluster's partials
 
 // Published sums are exchanged without a barrier: every slot is written once
 // per panel, and until then it holds a signalling-NaN pattern that no
@@ -61,30 +75,6 @@ __device__ __forceinline__ double gp_sum8(double v) {
   return v;
 }
 
-// s = sqrt(S), cl = -+s, up = x0 - cl and rb = 1 / (up cl) = -1 / (S + |x0| s)
-// for S within [2^-900, 2^900]: a third-order Householder iteration each from
-// the hardware's approximate reciprocal (square root), good to 2^-20 or so, and a
-// Newton correction that takes s to half an ulp (its error enters every entry of
-// the reflector).  Ten dependent FP64 operations of 64 clocks; sqrt() and a division with their
-// range checks take 1600 clocks on an idle pipe, the longest part of a column
-// step.
-__device__ __forceinline__ void gp_pivot(double S, double x0, double *cl, double *up, double *rb) {
-  double y, z;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(S));
-  const double ax = fabs(x0);
-  const double s0 = S * y;
-  const double b0 = fma(ax, s0, S);                      // approximate -b, for the seed
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(b0));
-  const double e = fma(-s0, y, 1.0);                     // 1 - S y^2 = 1 - s0^2 / S
-  double s = fma(s0 * e, fma(e, 0.375, 0.5), s0);
-  s = fma(fma(-s, s, S), 0.5 * y, s);
-  const double b = fma(ax, s, S);
-  const double f = fma(-b, z, 1.0);
-  *rb = -fma(fma(f, f, f), z, z);
-  *cl = x0 > 0.0 ? -s : s;
-  *up = x0 > 0.0 ? x0 + s : x0 - s;
-}
-
 }  // namespace
 
 // RPL rows per lane, R = 8 RPL rows per CTA; ONE: the grid is one cluster.
@@ -100,9 +90,9 @@ panel_grid_kernel(GridPanelParams p) {
   __shared__ unsigned s_mx[kNB];
   __shared__ int s_E[kNB];
   __shared__ double s_up[kNB], s_tau[kNB];
-  __shared__ double s_piv[2][3];              // cl, up, 1/b by j & 1
+  __shared__ double s_piv[2][3], s_sig[2][kNB];   // cl, up, 1/b; the columns' multipliers, by j & 1
   __shared__ int s_def[2];
-  __shared__ __align__(8) unsigned long long s_mbar[2];
+  __shared__ __align__(8) unsigned long long s_mbar[2], s_nbar[2];   // sums, column j's warp's
   __shared__ int s_ok, s_reported;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -139,11 +129,12 @@ panel_grid_kernel(GridPanelParams p) {
   }
 
   // Bytes the receive buffer gets for column j.  ONE: every CTA's partials of
-  // the active warps and the pivot row; else the cluster's partials of the
-  // active warps w = rank, rank + CS, ... (32 bytes each).
+  // the active warps and the pivot row, less those of column j's warp, which
+  // are counted on s_nbar; else the cluster's partials of the active warps
+  // w = rank, rank + CS, ... (32 bytes each).
   auto warp_active = [&](int w, int j) { return 4 * w + 3 >= j && 4 * w < nbw; };
   auto step_bytes = [&](int j) -> unsigned {
-    if (ONE) return (unsigned)((P + 1) * ((nbw + 3) / 4 - j / 4) * 32);
+    if (ONE) return (unsigned)((P + 1) * ((nbw + 3) / 4 - j / 4 - 1) * 32);
     int act = 0;
     for (int w = rank; w < kGpThreads / 32; w += CS) act += warp_active(w, j);
     return (unsigned)(CS * 32 * act);
@@ -151,11 +142,15 @@ panel_grid_kernel(GridPanelParams p) {
   if (tid == 0) {
     mbar_init1(&s_mbar[0]);
     mbar_init1(&s_mbar[1]);
+    mbar_init1(&s_nbar[0]);
+    mbar_init1(&s_nbar[1]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // columns 0 and 1; column j + 2's phase is announced once column j's has
     // completed, before this CTA sends anything for column j + 1
     for (int j = 0; j < 2; ++j)
       if (j < nbw && step_bytes(j) > 0) mbar_expect(&s_mbar[j], step_bytes(j));
+    if (ONE)
+      for (int j = 0; j < 2 && j < nbw; ++j) mbar_expect(&s_nbar[j], (unsigned)(P + 1) * 32);
     s_ok = 1;
     s_reported = 0;
   }
@@ -206,10 +201,6 @@ panel_grid_kernel(GridPanelParams p) {
       mx = max(mx, (unsigned)__ldcg(p.srec + (size_t)q * kNB + (tid & (kNB - 1))));
     atomicMax(&s_mx[tid & (kNB - 1)], mx);
   }
-  if (c == 0) {                               // column 0's tail
-#pragma unroll
-    for (int i = 0; i < RPL; ++i) xs[0][l8 + 8 * i] = (row0 + l8 + 8 * i > 0) ? v[i] : 0.0;
-  }
   __syncthreads();
   if (tid < kNB) {
     const int E = (int)((s_mx[tid] >> 20) & 0x7ff) - 1023;
@@ -217,45 +208,119 @@ panel_grid_kernel(GridPanelParams p) {
   }
   __syncthreads();
 
+  // Who takes the sums over all CTAs: four warps, 16 columns cs and two lanes to
+  // a column; the warps whose own columns end first take those that end last.
+  // More clusters than two lanes can poll: every warp its own columns.
+  const int cshift = ONE || NC <= 2 * kGpPolls ? 4 : 2;
+  const int sw = cshift == 2 ? warp : (warp < 3 ? 3 - warp : warp == 7 ? 0 : 16);
+  const int cs = (sw << cshift) + (lane & ((1 << cshift) - 1)), sub = lane >> cshift;
+  auto wait = [&](unsigned long long *bar, unsigned parity) {
+    bool reported = s_reported != 0;
+    if (!dead && !mbar_wait_bounded(bar, parity & 1u, p.spin, p.status, &reported, 1u << 16)) {
+      record_status(p.status, SLQR_ETIMEOUT);
+      dead = true;
+    }
+    if (reported && lane == 0) s_reported = 1;
+    __syncwarp();
+  };
+  // Named barriers between column j's warp (which does not wait) and the active
+  // warps of a quarter of the SM, w = g mod 4
+  auto quarter_threads = [&](int g, int j) {
+    const int n = (((nbw - 1) >> 2) - g >> 2) - ((j >> 2) - 1 - g >> 2);
+    return 32 * (n + (((j >> 2) & 3) != g));
+  };
+  auto quarter_arrive = [&](int g, int j) {
+    const int n = quarter_threads(g, j);
+    if (n > 32) asm volatile("bar.arrive %0, %1;" ::"r"(2 + g), "r"(n) : "memory");
+  };
+  auto quarter_sync = [&](int g, int j) {
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + g), "r"(quarter_threads(g, j)) : "memory");
+  };
+  // reflector k to this lane's column (the multipliers of step k)
+  auto apply = [&](int k) {
+    const int b = k & 1;
+    const double *x = xs[b];
+    if (s_def[b] && c > k && c < nbw) {
+      const double sig = s_sig[b][c], up = s_piv[b][1];
+      if (row0 <= k) {                         // the CTA with the pivot row (or above it)
+#pragma unroll
+        for (int i = 0; i < RPL; ++i) {
+          const int r = l8 + 8 * i;
+          if (row0 + r >= k) v[i] = fma(sig, row0 + r == k ? up : x[r], v[i]);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < RPL; ++i) v[i] = fma(sig, x[l8 + 8 * i], v[i]);
+      }
+    }
+  };
+  // the diagonal entry to column k
+  auto diagonal = [&](int k) {
+    if (s_def[k & 1] && c == k && row0 <= k && k < row0 + R) {
+      const double cl = s_piv[k & 1][0];
+#pragma unroll
+      for (int i = 0; i < RPL; ++i) v[i] = (row0 + l8 + 8 * i == k) ? cl : v[i];
+    }
+  };
+
   for (int j = 0; j < nbw; ++j) {
     const int buf = j & 1;
+    const unsigned phase = (unsigned)(j >> 1) & 1u;
     const double *x = xs[buf];
     const bool mine = (j >> 2) == warp;        // this warp holds column j
     // a column of extreme scale squares its scaled entries (uniform)
     const bool extreme = abs(s_E[j]) > 400;
-    const double sc = exp2i(-s_E[j]);
-    double D = 0.0, pc = 0.0;
 
-    // dot of the tail of x_j with this lane's column (c == j: its norm)
-    auto dot = [&]() {
-      double a0 = 0.0, a1 = 0.0;
+    // Reflector j - 1, then the dots with column j.  Its warp does not wait for
+    // the others, and those of its quarter let it go first where its norm makes
+    // its own way to the pivot.
+    if (warp_active(warp, j)) {
+      const int quarter = (j >> 2) & 3;
+      if (ONE && !mine && (warp & 3) == quarter) quarter_sync(warp & 3, j);
+      if (j > 0) apply(j - 1);
+      if (mine) {
+        if (c == j) {                          // its tail to the other warps
+#pragma unroll
+          for (int i = 0; i < RPL; ++i)
+            xs[buf][l8 + 8 * i] = (row0 + l8 + 8 * i > j) ? v[i] : 0.0;
+        }
+        __syncwarp();
+        for (int g = 0; g < 4; ++g)
+          if (!ONE || g != quarter) quarter_arrive(g, j);
+      } else if (!ONE || (warp & 3) != quarter) {
+        quarter_sync(warp & 3, j);
+      }
+      // dot of the tail of x_j with this lane's column (c == j: its norm); one
+      // chain up to 8 terms: an FP64 operation's latency is the time the pipe
+      // takes to issue it
+      double part = 0.0, part1 = 0.0;
       if (row0 <= j) {                         // rows up to the pivot's take no part
 #pragma unroll
         for (int i = 0; i < RPL; ++i)
-          a0 = fma(x[l8 + 8 * i], row0 + l8 + 8 * i > j ? v[i] : 0.0, a0);
+          part = fma(x[l8 + 8 * i], row0 + l8 + 8 * i > j ? v[i] : 0.0, part);
       } else {
 #pragma unroll
-        for (int i = 0; i < RPL; i += 2) {
-          a0 = fma(x[l8 + 8 * i], v[i], a0);
-          a1 = fma(x[l8 + 8 * (i + 1)], v[i + 1], a1);
+        for (int i = 0; i < RPL; ++i) {
+          if (RPL > 8 && (i & 1)) part1 = fma(x[l8 + 8 * i], v[i], part1);
+          else part = fma(x[l8 + 8 * i], v[i], part);
         }
       }
       if (extreme && mine) {
-        double n0 = 0.0;
+        const double sc = exp2i(-s_E[j]);
+        double n = 0.0;
 #pragma unroll
         for (int i = 0; i < RPL; ++i) {
           const double t = x[l8 + 8 * i] * sc;
-          n0 = fma(t, t, n0);
+          n = fma(t, t, n);
         }
-        if (c == j) a0 = n0, a1 = 0.0;
+        if (c == j) part = n, part1 = 0.0;
       }
-      return gp_sum8(a0 + a1);
-    };
-
-    if (warp_active(warp, j)) {
-      const double part = dot();
+      if (RPL > 8) part += part1;
+      part = gp_sum8(part);
+      if (ONE && mine) quarter_arrive(quarter, j);
       // two columns' partials per lane half, 16 bytes to a receiver
       const int h = lane >> 4;
+      unsigned long long *bar = mine && ONE ? &s_nbar[buf] : &s_mbar[buf];
       {
         double w[2];
         w[0] = __shfl_sync(0xffffffffu, part, 16 * h);
@@ -264,11 +329,11 @@ panel_grid_kernel(GridPanelParams p) {
           const int dst = lane & 15;
           if (dst < P)
             st_async16(cluster_addr(&s_recv[buf][rank][warp * 4 + 2 * h], dst), w,
-                       cluster_addr(&s_mbar[buf], dst));
+                       cluster_addr(bar, dst));
         } else if ((lane & 15) == 0) {
           const int dst = warp % CS;
           st_async16(cluster_addr(&s_recv[buf][rank][(warp / CS) * 4 + 2 * h], dst), w,
-                     cluster_addr(&s_mbar[buf], dst));
+                     cluster_addr(bar, dst));
         }
       }
       // the pivot row, by the CTA that holds it
@@ -284,50 +349,79 @@ panel_grid_kernel(GridPanelParams p) {
           const int dst = lane & 15;
           if (dst < P)
             st_async16(cluster_addr(&s_prow[buf][warp * 4 + 2 * h], dst), ww,
-                       cluster_addr(&s_mbar[buf], dst));
+                       cluster_addr(bar, dst));
         } else if (l8 == l && c >= j && c < nbw) {
           gp_publish(p.prow + (size_t)j * kNB + c, w);
         }
       }
-      const bool want = c >= j && c < nbw;
-      // the receive buffer of column j (this CTA's columns of the cluster, or all)
-      const bool collect = ONE || warp % CS == rank;
-      if (collect) {
-        bool reported = s_reported != 0;
-        if (!dead && !mbar_wait_bounded(&s_mbar[buf], (unsigned)(j >> 1) & 1u, p.spin, p.status,
-                                        &reported)) {
-          record_status(p.status, SLQR_ETIMEOUT);
-          dead = true;
-        }
-        if (reported && lane == 0) s_reported = 1;
-        // the warp of this buffer that stays active longest announces the next phase
-        const bool last = ONE ? mine : (warp + CS >= kGpThreads / 32 || 4 * (warp + CS) >= nbw);
-        if (last && lane == 0 && !dead && j + 2 < nbw && step_bytes(j + 2) > 0)
+    }
+    if (j > 0 && (j - 1) >> 2 == warp) diagonal(j - 1);
+    // the cluster's sums of this CTA's columns: one warp, CS / 2 lanes a column
+    if (!ONE && warp == kGpCollector && step_bytes(j) > 0) {
+      wait(&s_mbar[buf], phase);
+      if (lane == 0 && !dead && j + 2 < nbw && step_bytes(j + 2) > 0)
+        mbar_expect(&s_mbar[buf], step_bytes(j + 2));
+      __syncwarp();
+      const int half = CS / 2, q = CS == 8 ? lane >> 2 : lane >> 1, l = lane & (half - 1);
+      double sum = s_recv[buf][l][q] + s_recv[buf][l + half][q];
+      for (int o = 1; o < half; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      const int cc = ((q >> 2) * CS + rank) * 4 + (q & 3);
+      if (l == 0 && cc >= j && cc < nbw)
+        gp_publish(p.rec + ((size_t)j * NC + cluster) * kNB + cc, sum);
+    }
+    // the pivot, in every lane of a warp
+    auto pivot = [&](double x0, double tail) {
+      const PivotFp64 f = pivot_fp64(x0, tail, extreme, s_E[j]);
+      if (lane == 0) {
+        s_piv[buf][0] = f.cl;
+        s_piv[buf][1] = f.up;
+        s_piv[buf][2] = f.rb;
+        s_def[buf] = f.defined;
+        s_up[j] = f.up;
+        s_tau[j] = -f.rb;
+      }
+    };
+    if (ONE && warp == kGpPivot) {
+      wait(&s_nbar[buf], phase);
+      if (lane == 0 && !dead && j + 2 < nbw) mbar_expect(&s_nbar[buf], (unsigned)(P + 1) * 32);
+      __syncwarp();
+      double tail = lane < P ? s_recv[buf][lane][j] : 0.0;
+      if (P > 8) tail += __shfl_xor_sync(0xffffffffu, tail, 8);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) tail += __shfl_xor_sync(0xffffffffu, tail, o);
+      pivot(s_prow[buf][j], __shfl_sync(0xffffffffu, tail, 0));
+    }
+    // the columns' sums and their multipliers (of the columns after j; in a
+    // cluster panel column j's sum is among them, and its warp takes the pivot)
+    const int c0 = ONE ? j + 1 : j;
+    const int first = c0 >> cshift, last = (nbw - 1) >> cshift;
+    const bool summing = c0 < nbw && sw >= first && sw <= last;
+    double D = 0.0, pc = 0.0;
+    if (summing) {
+      if (ONE) {
+        wait(&s_nbar[buf], phase);
+        if (step_bytes(j) > 0) wait(&s_mbar[buf], phase);
+        if (sw == last && lane == 0 && !dead && j + 2 < nbw && step_bytes(j + 2) > 0)
           mbar_expect(&s_mbar[buf], step_bytes(j + 2));
         __syncwarp();
-        if (ONE) {
-          if (want) {
-            D = l8 < P ? s_recv[buf][l8][c] : 0.0;
-            if (l8 + 8 < P) D += s_recv[buf][l8 + 8][c];
-            pc = s_prow[buf][c];
-          }
-          D = gp_sum8(D);
-        } else {
-          const double sum = gp_sum8(l8 < CS ? s_recv[buf][l8][(warp / CS) * 4 + (lane >> 3)] : 0.0);
-          if (l8 == 0 && want) gp_publish(p.rec + ((size_t)j * kNB + c) * NC + cluster, sum);
+        D = sub < P ? s_recv[buf][sub][cs] : 0.0;
+#pragma unroll
+        for (int q = 2; q < kClMaxCtas; q += 2) {
+          if (q >= P) break;
+          D += q + sub < P ? s_recv[buf][q + sub][cs] : 0.0;
         }
-      }
-      if (!ONE) {
-        // the clusters' sums of this lane's column
-        const double *rec = p.rec + ((size_t)j * kNB + c) * NC;
-        const double *prow = p.prow + (size_t)j * kNB + c;
+        D += __shfl_xor_sync(0xffffffffu, D, 16);
+        pc = s_prow[buf][cs];
+      } else {
+        const bool want = cs >= j && cs < nbw;
+        const double *rec = p.rec + ((size_t)j * NC + sub) * kNB + cs;
+        const double *prow = p.prow + (size_t)j * kNB + cs;
+        const int subs = 32 >> cshift;
         unsigned it = 0;
         double r[kGpPolls];
 #pragma unroll
-        for (int u = 0; u < kGpPolls; ++u) {
-          const int q = l8 + 8 * u;
-          r[u] = (want && q < NC) ? gp_load(rec + q) : 0.0;
-        }
+        for (int u = 0; u < kGpPolls; ++u)
+          r[u] = (want && sub + u * subs < NC) ? gp_load(rec + (size_t)u * subs * kNB) : 0.0;
         pc = want ? gp_load(prow) : 0.0;
         while (!dead) {
           bool miss = gp_unset(pc);
@@ -338,67 +432,31 @@ panel_grid_kernel(GridPanelParams p) {
           if (++it > kSpinLimit) dead = true;
 #pragma unroll
           for (int u = 0; u < kGpPolls; ++u)
-            if (gp_unset(r[u])) r[u] = gp_load(rec + l8 + 8 * u);
+            if (gp_unset(r[u])) r[u] = gp_load(rec + (size_t)u * subs * kNB);
           if (gp_unset(pc)) pc = gp_load(prow);
         }
         // (adds of absent clusters are skipped, uniformly)
         D = r[0];
 #pragma unroll
         for (int u = 1; u < kGpPolls; ++u)
-          if (8 * u < NC) D += r[u];
-        D = gp_sum8(D);
-      }
-      if (mine) {
-        // the pivot, in every lane of this warp
-        const double tail = __shfl_sync(0xffffffffu, D, (j & 3) * 8);
-        const double x0 = __shfl_sync(0xffffffffu, pc, (j & 3) * 8);
-        const double t0 = extreme ? x0 * sc : x0;
-        const double S = fma(t0, t0, tail);
-        double cl = 0.0, up = 0.0, rb = 0.0;
-        if (!extreme && S > exp2i(-900) && S < exp2i(900)) {
-          gp_pivot(S, x0, &cl, &up, &rb);
-        } else if (S != 0.0) {
-          const double s = extreme ? sqrt(S) * exp2i(s_E[j]) : sqrt(S);
-          cl = (x0 > 0.0) ? -s : s;
-          up = x0 - cl;
-          rb = 1.0 / (up * cl);
-        }
-        if (lane == 0) {
-          s_piv[buf][0] = cl;
-          s_piv[buf][1] = up;
-          s_piv[buf][2] = rb;
-          s_def[buf] = S != 0.0;
-          s_up[j] = up;
-          s_tau[j] = -rb;
+          if (u * subs < NC) D += r[u];
+        for (int o = 16; o >= 1 << cshift; o >>= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
+        if (sw == first) {
+          const int l = j & ((1 << cshift) - 1);
+          const double x0 = __shfl_sync(0xffffffffu, pc, l);
+          pivot(x0, __shfl_sync(0xffffffffu, D, l));
         }
       }
     }
-    __syncthreads();
-    const bool defined = s_def[buf] != 0;
-    const double cl = s_piv[buf][0], up = s_piv[buf][1], rb = s_piv[buf][2];
-    if (defined && c > j && c < nbw) {
-      const double sig = fma(up, pc, D) * rb;
-      if (row0 <= j) {                         // the CTA with the pivot row (or above it)
-#pragma unroll
-        for (int i = 0; i < RPL; ++i) {
-          const int r = l8 + 8 * i;
-          if (row0 + r >= j) v[i] = fma(sig, row0 + r == j ? up : x[r], v[i]);
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < RPL; ++i) v[i] = fma(sig, x[l8 + 8 * i], v[i]);
-      }
-    }
-    if (c == j + 1) {                          // the next column's tail
-#pragma unroll
-      for (int i = 0; i < RPL; ++i) xs[buf ^ 1][l8 + 8 * i] = (row0 + l8 + 8 * i > j + 1) ? v[i] : 0.0;
-    }
-    if (defined && c == j && row0 <= j && j < row0 + R) {
-#pragma unroll
-      for (int i = 0; i < RPL; ++i) v[i] = (row0 + l8 + 8 * i == j) ? cl : v[i];
+    // the pivot to the summing warps
+    if (summing || (ONE && warp == kGpPivot)) {
+      const int n = (c0 < nbw ? last - first + 1 : 0) + (ONE ? 1 : 0);
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * n) : "memory");
+      if (summing && sub == 0) s_sig[buf][cs] = fma(s_piv[buf][1], pc, D) * s_piv[buf][2];
     }
     __syncthreads();
   }
+  if (warp == (nbw - 1) >> 2) diagonal(nbw - 1);
 
   // the slice back to the matrix, Vtop (ld NB: zero above the diagonal, up on
   // it, tails below) from the CTAs of the top rows
@@ -438,7 +496,7 @@ static const void *grid_kernel(int R, bool one) {
     case 64: return one ? (const void *)panel_grid_kernel<8, true> : (const void *)panel_grid_kernel<8, false>;
     case 128: return one ? (const void *)panel_grid_kernel<16, true> : (const void *)panel_grid_kernel<16, false>;
     case 48: return one ? (const void *)panel_grid_kernel<6, true> : (const void *)panel_grid_kernel<6, false>;
-    case 80: return one ? nullptr : (const void *)panel_grid_kernel<10, false>;
+    case 80: return one ? (const void *)panel_grid_kernel<10, true> : (const void *)panel_grid_kernel<10, false>;
     case 96: return one ? (const void *)panel_grid_kernel<12, true> : (const void *)panel_grid_kernel<12, false>;
     case 160: return one ? nullptr : (const void *)panel_grid_kernel<20, false>;
     case 192: return one ? nullptr : (const void *)panel_grid_kernel<24, false>;
@@ -500,22 +558,23 @@ slqr_status init_grid_panel_attrs(slqr_ctx *ctx) {
   return SLQR_OK;
 }
 
-// Rows per CTA, smallest first.  One cluster up to 16 CTAs of 64 rows (1024
-// rows: 3.6 us a column; 32 CTAs in clusters of 8: 4.0).  Above that clusters of
-// 8, 64 CTAs at most while 256 rows each are enough: the sums of more clusters
-// take longer to arrive than the shorter slices save (8192 rows: 6.2 us a column
-// on 64 CTAs, 7.6 on 104), and the trailing update runs on the other SMs.
+// Rows per CTA, smallest first.  One cluster up to 16 CTAs of 80 rows (1100 rows:
+// 3.4 us a column, 35 CTAs of 32 rows in clusters of 8 3.5; 1300 rows on CTAs of
+// 96: 3.7 against 3.6).  Above that clusters of 8, 64 CTAs at most while 256 rows
+// each are enough: the sums of more clusters take longer to arrive than the
+// shorter slices save (8192 rows: 6.2 us a column on 64 CTAs, 7.6 on 104), and the
+// trailing update runs on the other SMs.
 GridPanelShape grid_panel_shape(const slqr_ctx *ctx, int M, int rows_min) {
   GridPanelShape s;
   const int one = ctx->grid_panel_one;
   for (int R : kGridRows) {
     const int P = (M + R - 1) / R;
     if (rows_min > 0 && R < rows_min && R < 256) continue;
-    if (P <= one && grid_kernel(R, true) && (R <= 64 || rows_min > 0)) {
+    if (P <= one && grid_kernel(R, true) && (R <= 80 || rows_min > 0)) {
       s.R = R, s.P = P, s.cluster = P;
       return s;
     }
-    if (rows_min == 0 && R < 64 && (M + 63) / 64 <= one) continue;
+    if (rows_min == 0 && R < 80 && (M + 79) / 80 <= one) continue;
     const int P8 = (P + 7) / 8 * 8;
     if (P8 <= std::min(ctx->grid_panel_c8, rows_min > 0 || R == 256 ? ctx->grid_panel_c8 : 64) &&
         (P8 > one || !grid_kernel(R, true))) {

@@ -160,3 +160,14 @@ def test_compact_wy_of_few_columns(ctx, m, n):
         assert np.all(np.abs(np.triu(G, 1) - want) <= 4.0 * np.sqrt(m) * U * np.outer(nrm, nrm))
         tau = -1.0 / (u[k0:k0 + w] * np.diag(F)[k0:k0 + w])
         np.testing.assert_allclose(blk[2048:2048 + w], tau, rtol=16 * U)
+
+
+# the last rows of one cluster of 16 CTAs of 32 and of 80 rows, clusters of 8 with
+# up to 10 and with more sums to collect, clusters of 4; a last panel of 1..6 columns
+@pytest.mark.parametrize("m,n", [(33, 33), (512, 70), (513, 65), (1280, 130), (1281, 67),
+                                 (2049, 66), (16385, 69), (21000, 70), (29000, 68)])
+def test_panel_shapes(ctx, m, n):
+    A, b = workloads.gaussian(m, n, seed=m - n)
+    F, up, qtb, x, st = run_gpu(ctx, A, b)
+    assert st == 0
+    check_against_oracle(A, b, F, up, qtb, x)
