@@ -36,6 +36,7 @@
 // The digit matrices of one operand are stacked, so A_i times all B_j with
 // j <= 7 - i is one MMA (N = 64 or 32 per digit) whose result columns are the
 // accumulators of the orders i, i + 1, ...
+#include "fx_digits.cuh"
 #include "tc_common.cuh"
 
 #include <cuda_fp16.h>
@@ -43,8 +44,6 @@
 
 namespace slqr {
 
-constexpr int kFxD = 7;                       // digits
-constexpr int kFxOrders = 8;                  // accumulated orders i + j
 constexpr int kFxWorkers = 16;                // warps that split and reassemble; one more issues MMAs
 constexpr int kFxThreads = 32 * (kFxWorkers + 1);
 constexpr int kFxV1Chunk = kFxD * 64 * 64;            // 28672 B: 32 rows
@@ -55,7 +54,6 @@ constexpr int kFxStage = kFxXStage + kFxV1Chunk;
 constexpr size_t kFxVtxSmem = 2 * (size_t)kFxStage + 1024;
 constexpr size_t kFxUpdSmem = (size_t)kFxV2Tile + 2 * kFxWTile + 1024;
 constexpr int kFxMaxPer = 32;                // column tiles of a CTA of the update
-constexpr int kFxNonFinite = 1 << 20;         // exponent that stands for Inf / NaN
 
 // D = F32, A = B = F16, both K-major, M = 128; N is added per MMA
 constexpr uint32_t kIdescF16 = (1u << 4) | ((128u >> 4) << 24);
@@ -94,6 +92,11 @@ __device__ __forceinline__ void fx_commit(uint64_t *bar) {
                :: "r"(smem_u32(bar)) : "memory");
 }
 
+// Row (of 32) of slot 8 rg + k along K in V1 and in the digits of X: a thread of
+// V^T X reads 8 rows of a column, two at a time, and its four neighbours' pairs
+// are adjacent, so that a load covers whole sectors.
+__device__ __forceinline__ int fx_row(int rg, int k) { return (k >> 1) * 8 + rg * 2 + (k & 1); }
+
 // 1-D bulk copy (16-byte aligned, a multiple of 16 bytes) counted on an mbarrier
 __device__ __forceinline__ void fx_bulk(uint32_t dst, const void *src, uint32_t bytes,
                                         uint64_t *bar) {
@@ -102,100 +105,6 @@ __device__ __forceinline__ void fx_bulk(uint32_t dst, const void *src, uint32_t 
                : "memory");
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes"
                " [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(b) : "memory");
-}
-
-// High word of |x| (sign cleared): ordered as |x|.
-__device__ __forceinline__ uint32_t fx_hi(double x) {
-  return (uint32_t)__double2hiint(x) & 0x7fffffffu;
-}
-
-// Key of a vector maximum: the high word of |x| with the exponent unbiased (a
-// denormal counts as its binade), plus a power of two as `shift` exponents;
-// kFxZero for a zero.
-constexpr int kFxZero = -0x7fffffff;
-__device__ __forceinline__ int fx_key_of_hi(uint32_t hi) {
-  return (int)(hi < 0x00100000u ? (hi | 0x00100000u) : hi) - (1023 << 20);
-}
-__device__ __forceinline__ int fx_key(double x, int shift) {
-  return x != 0.0 ? fx_key_of_hi(fx_hi(x)) + shift * (1 << 20) : kFxZero;
-}
-
-// Exponent e of a vector whose largest entry has this key: every entry is at
-// most 1.9883 * 2^(e-1), so that |x| 2^(55-e) stays within the balanced digits
-// (127 (256^7 - 1) / 255 = 1.9921 * 2^54).
-__device__ __forceinline__ int fx_exp(int key) {
-  return (key >> 20) + 1 + ((key & 0xfffff) >= 0xFD000 ? 1 : 0);   // (shift: floor)
-}
-
-__device__ __forceinline__ int fx_exp_of_hi(uint32_t hi) { return fx_exp(fx_key_of_hi(hi)); }
-
-// round(x 2^(55-e)) as seven balanced digits, each biased by 128: byte 6 - i
-// of the result is d_i + 128.
-__device__ __forceinline__ unsigned long long fx_digits(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int Ef = (int)(b >> 52) & 0x7ff;
-  unsigned long long m = b & 0xfffffffffffffull;
-  m |= Ef ? (1ull << 52) : 0ull;
-  const int rsh = min(max(1022 + e - max(Ef, 1), 0), 62);
-  m = (((m << 3) >> rsh) + 1) >> 1;                       // (m << 2) >> rsh, rounded
-  const unsigned long long bias = 0x80808080808080ull;
-  return (long long)b < 0 ? bias - m : bias + m;
-}
-
-// The same with three bits more for the leading digit (|x| up to 2^3 times
-// the bound above): bytes 5 .. 0 biased, the rest the signed leading digit,
-// at most 1024 in magnitude (exact in FP16).
-__device__ __forceinline__ long long fx_digits_wide(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int Ef = (int)(b >> 52) & 0x7ff;
-  unsigned long long m = b & 0xfffffffffffffull;
-  m |= Ef ? (1ull << 52) : 0ull;
-  const int rsh = min(max(1022 + e + 3 - max(Ef, 1), 0), 62);
-  m = (((m << 6) >> rsh) + 1) >> 1;                       // (m << 5) >> rsh, rounded
-  const long long bias = 0x808080808080ll;
-  return (long long)b < 0 ? bias - (long long)m : bias + (long long)m;
-}
-
-// The digits at byte `byte` of two biased words as two FP16 values (low, high).
-__device__ __forceinline__ uint32_t fx_half2(uint32_t w0, uint32_t w1, int byte) {
-  // bytes w0[byte], 0x64, w1[byte], 0x64: 1024 + u in each half (exact in FP16)
-  const uint32_t r =
-      (__byte_perm(w0, w1, byte | ((4 + byte) << 8)) & 0x00ff00ffu) | 0x64006400u;
-  uint32_t o;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(o) : "r"(r), "r"(0x64806480u));   // minus 1152
-  return o;
-}
-
-// Eight values' digits i as 16 bytes (value k in half k).
-__device__ __forceinline__ uint4 fx_pack8(const unsigned long long (&y)[8], int i) {
-  const int byte = 6 - i;
-  uint32_t o[4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const uint32_t w0 = byte < 4 ? (uint32_t)y[2 * p] : (uint32_t)(y[2 * p] >> 32);
-    const uint32_t w1 = byte < 4 ? (uint32_t)y[2 * p + 1] : (uint32_t)(y[2 * p + 1] >> 32);
-    o[p] = fx_half2(w0, w1, byte & 3);
-  }
-  return make_uint4(o[0], o[1], o[2], o[3]);
-}
-
-// t 2^k for any k (the exact power of two in one or two steps)
-__device__ __forceinline__ double fx_scale(double t, int k) {
-  if (k >= -960 && k <= 1000)
-    return t * __longlong_as_double((long long)(k + 1023) << 52);
-  return scalbn(t, k);
-}
-
-// t 2^sh rounded to FP64 for sh in [-1000, 900], in integer arithmetic: a
-// conversion instruction would hold the FP64 pipe for 16 clocks of the SM.
-__device__ __forceinline__ double fx_to_double(long long t, int sh) {
-  const unsigned long long a = (unsigned long long)(t < 0 ? -t : t);
-  const int lz = __clzll((long long)a);
-  const unsigned long long m = a << (lz & 63);           // leading bit at 63
-  // mantissa rounded half up; its leading bit adds one to the exponent field
-  unsigned long long b = ((unsigned long long)(1085 - lz + sh) << 52) + (m >> 11) + ((m >> 10) & 1);
-  b = a ? b : 0ull;
-  return __longlong_as_double((long long)(b | ((unsigned long long)t & (1ull << 63))));
 }
 
 // Four accumulators of every order for this thread's TMEM lane: order o at
@@ -208,15 +117,6 @@ __device__ __forceinline__ void fx_ld_orders(uint32_t (&r)[kFxOrders][4], uint32
                  : "=r"(r[o][0]), "=r"(r[o][1]), "=r"(r[o][2]), "=r"(r[o][3])
                  : "r"(addr + (uint32_t)o * stride));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Orders o0 .. o0 + 3 of one output: sum of acc_o 256^(3 - (o - o0))
-__device__ __forceinline__ long long fx_four(const uint32_t (&r)[kFxOrders][4], int o0, int k) {
-  long long v = __float2int_rn(__uint_as_float(r[o0 + 3][k]));
-  v += (long long)__float2int_rn(__uint_as_float(r[o0 + 2][k])) * 256;
-  v += (long long)__float2int_rn(__uint_as_float(r[o0 + 1][k])) * 65536;
-  v += (long long)__float2int_rn(__uint_as_float(r[o0][k])) * 16777216;
-  return v;
 }
 
 // --------------------------------------------------------------------------
@@ -302,9 +202,9 @@ fx_vsplit_kernel(const double *__restrict__ A, int lda, const double *__restrict
     __align__(16) __half lead[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const long long v = fx_digits_wide(f == kFxNonFinite ? 0.0 : t[a][rg * 8 + k], f - 3);
-      y[k] = (unsigned long long)v;
-      lead[k] = __int2half_rn((int)(v >> 48));
+      int d0;
+      y[k] = fx_digits_wide(f == kFxNonFinite ? 0.0 : t[a][fx_row(rg, k)], f - 3, &d0);
+      lead[k] = __int2half_rn(d0);
     }
     unsigned char *dst = V1 + (size_t)blockIdx.x * kFxV1Chunk + a * 64 +
                          ((rg * 16) ^ (((a >> 1) & 3) << 4));
@@ -346,11 +246,6 @@ __device__ __forceinline__ void fx_mbar_init(uint64_t *bar, int count) {
 }
 __device__ __forceinline__ void fx_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// Unit exponent of the totals over slices of RS rows: 56 up to 512 rows, one
-// more for every factor of four.
-__device__ __forceinline__ int fx_unit(int RS) {
-  return 56 + (RS > 512) + (RS > 2048) + (RS > 8192) + (RS > 32768);
 }
 // whole-warp wait (the lanes leave together)
 __device__ __forceinline__ bool fx_wait(uint64_t *bar, int phase) {
@@ -580,29 +475,29 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
               V1 + (size_t)(i_begin / 32 + t) * kFxV1Chunk, kFxV1Chunk, &s_full[t & 1]);
     };
     double xv[8];
+    const bool even_col = (((uintptr_t)xcol) & 15) == 0;
     auto load_x = [&](int t) {
-      const int i = i_begin + t * 32 + rg * 8;
-      const double *p = xcol + k0 + i + (i >= nbw ? skip : 0);
+      const int ib = i_begin + t * 32, i = ib + rg * 2;
       // the registers hold one chunk ahead; L2 gets three (128 bytes per thread pair)
-      if (col_ok && (rg & 1) == 0 && i + 96 + 16 <= i_end)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(xcol + k0 + i + 96 + (i + 96 >= nbw ? skip : 0)));
-      const bool whole = i + 8 <= i_end && (i >= nbw || i + 8 <= nbw || skip == 0);
-      if (col_ok && whole) {
-        if ((((uintptr_t)p) & 15) == 0) {
+      if (col_ok && (rg & 1) == 0 && ib + 128 <= i_end)
+        asm volatile("prefetch.global.L2 [%0];"
+                     ::"l"(xcol + k0 + ib + 96 + rg * 8 + (ib + 96 >= nbw ? skip : 0)));
+      const bool whole = ib + 32 <= i_end && (ib >= nbw || ib + 32 <= nbw || skip == 0);
+      const int off = k0 + i + (ib >= nbw ? skip : 0);
+      if (col_ok && whole && even_col && (off & 1) == 0) {
 #pragma unroll
-          for (int k = 0; k < 8; k += 2) {
-            const double2 v = *(const double2 *)(p + k);
-            xv[k] = v.x;
-            xv[k + 1] = v.y;
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) xv[k] = p[k];
+        for (int k = 0; k < 8; k += 2) {
+          const double2 v = *(const double2 *)(xcol + off + k * 4);
+          xv[k] = v.x;
+          xv[k + 1] = v.y;
         }
+      } else if (col_ok && whole) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) xv[k] = xcol[off + (k >> 1) * 8 + (k & 1)];
       } else {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          const int ii = i + k;
+          const int ii = ib + fx_row(rg, k);
           xv[k] = (col_ok && ii < i_end) ? xcol[k0 + ii + (ii >= nbw ? skip : 0)] : 0.0;
         }
       }
@@ -630,11 +525,19 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           if (lane == 0) fx_arrive(&s_drained);
         }
-        // orders 0..3 in units of 2^72, 4..7 in units of 2^40
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          tot[u * 4 + k] += (fx_four(r, 0, k) << (72 - ush)) +
-                            ((fx_four(r, 4, k) + (1ll << (ush - 41))) >> (ush - 40));
+        for (int k = 0; k < 4; ++k) {
+          // 128 terms: orders 0 and 1 are at most 2^22; of 6 and 7 two units are
+          // lost, 2^-63 of the bound; the others are converted
+          auto f = [&](int o) { return __uint_as_float(r[o][k]); };
+          const long long hi = ((long long)(fx_small(f(0)) * 256 + fx_small(f(1))) << 16) +
+                               (long long)__float2int_rn(f(2)) * 256 + __float2int_rn(f(3));
+          const long long lo = (long long)__float2int_rn(f(4)) * 65536 +
+                               (long long)__float2int_rn(f(5)) * 256 + fx_small_quarter(f(6)) * 4 +
+                               (fx_small_quarter(f(7)) >> 6);
+          // hi in units of 2^72, lo of 2^48
+          tot[u * 4 + k] += (hi << (72 - ush)) + ((lo + (1ll << (ush - 49))) >> (ush - 48));
+        }
       }
       return true;
     };
@@ -654,10 +557,10 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
 #pragma unroll
         for (int i = 0; i < kFxD; ++i) *(uint4 *)(dst + i * 8192) = fx_pack8(y, i);
       }
-      if (t + 1 < T) load_x(t + 1);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) fx_arrive(&s_xfull[st]);
+      if (t + 1 < T) load_x(t + 1);                     // (behind the fence, which waits for loads)
       if (t > 0 && (t & 3) == 0) ok = drain(t / 4 - 1);
     }
     if (ok) ok = drain((T - 1) / 4);
@@ -811,7 +714,7 @@ fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restri
     const int sw = (c & 7) << 4;
 #pragma unroll
     for (int i = 0; i < kFxD; ++i) {
-      const int b = 8 * (6 - i);
+      const int b = 8 * (7 - i);
       const uint32_t v = fx_half2((uint32_t)(y0 >> b) & 0xff, (uint32_t)(y1 >> b) & 0xff, 0);
       *(unsigned short *)(dst + i * 4096 + ((lane * 2) ^ sw)) = (unsigned short)(v & 0xffff);
       *(unsigned short *)(dst + i * 4096 + ((64 + lane * 2) ^ sw)) = (unsigned short)(v >> 16);
@@ -960,16 +863,22 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const int k = u * 4 + kk;
-          // orders 0..3 in units of 2^72, 4..7 in units of 2^40, of 2^(erow + g -
-          // 110); kept to 2^54 of those units in 63 bits: the first are below 2^45
-          // (the leading order sums 64 products)
-          const long long tt = (fx_four(r, 0, kk) << 18) + ((fx_four(r, 4, kk) + (1 << 13)) >> 14);
+          // Orders in units of 2^(erow + g - 110), kept to 2^54 of those in 63 bits
+          // (the leading order sums 64 products).  Orders 0..3 are at most 2^22,
+          // 4 and 5 above; of 6 and 7 half a unit is lost, 2^-62 of the bound.
+          auto f = [&](int o) { return __uint_as_float(r[o][kk]); };
+          const long long tt =
+              fx_join(fx_small(f(0)) * 256 + fx_small(f(1)), fx_small(f(2)) * 256 + fx_small(f(3)),
+                      __float2int_rn(f(4)) * 256 + __float2int_rn(f(5)),
+                      (fx_small_half(f(6)) * 256 + fx_small_half(f(7))) * 2, 20);
           const int gk = g[k], sh = er + gk;
-          if (sh >= -1000 && sh <= 900)
+          // (uniform: exponents out of the quick form's range are rare)
+          if (__all_sync(0xffffffffu, sh >= -1000 && sh <= 900))
             x[k] -= fx_to_double(tt, sh);
+          else if (gk == kFxNonFinite)
+            x[k] = __longlong_as_double(0x7ff8000000000000ll);
           else
-            x[k] = gk == kFxNonFinite ? __longlong_as_double(0x7ff8000000000000ll)
-                                      : x[k] - scalbn((double)tt, sh);
+            x[k] -= fx_scale_slow((double)tt, sh);
           if (row_ok && cw + k < N) xw[(size_t)k * ldx] = x[k];
           const unsigned mx = __reduce_max_sync(0xffffffffu, next_row ? fx_hi(x[k]) : 0u);
           if (lane == k) mine = mx;
