@@ -39,21 +39,30 @@ BatchKernels batch_kernels_nb16(int tc) {
   }
 }
 
-// kernels of a setting (null pointers when not valid); rm > 0: the
-// shared-memory-resident FP64 kernel for problems of at most rm rows
-static BatchKernels batch_kernels(int nb, int tc, int rm = 0) {
+// kernels of a setting (null pointers when not valid) for problems of at most
+// `rows` rows; rm > 0: the shared-memory-resident FP64 kernel for problems of at
+// most rm rows
+static BatchKernels batch_kernels(int nb, int tc, int rm = 0, int rows = kBMaxRows) {
   if (rm > 0) {
     if (nb != 16 || tc != 32) return BatchKernels{};
     if (rm == 64) return batch_resident_kernels_of<16, 32, 64>();
     if (rm == 128) return batch_resident_kernels_of<16, 32, 128>();
     return BatchKernels{};
   }
+  BatchKernels k;
   switch (nb) {
-    case 8: return batch_kernels_nb8(tc);
-    case 16: return batch_kernels_nb16(tc);
-    case 32: return batch_kernels_nb32(tc);
-    default: return BatchKernels{};
+    case 8: k = batch_kernels_nb8(tc); break;
+    case 16: k = batch_kernels_nb16(tc); break;
+    case 32: k = batch_kernels_nb32(tc); break;
+    default: return k;
   }
+  if (nb == kBNBDefault && tc == kBTCDefault) {
+    const BatchKernels f = batch_fx_kernels(rows);
+    k.fp64 = f.fp64;
+    k.smem_fp64 = f.smem_fp64;
+    k.threads_fp64 = f.threads_fp64;
+  }
+  return k;
 }
 
 // size classes of the problems by their row count
@@ -100,6 +109,10 @@ slqr_status init_batch_attrs(slqr_ctx *ctx) {
       e = cudaFuncSetAttribute(k.mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)k.smem_mixed);
   }
+  for (int c = 0; c < kBClasses && e == cudaSuccess; ++c) {
+    BatchKernels k = batch_fx_kernels(kBClassHi[c]);
+    e = cudaFuncSetAttribute(k.fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_fp64);
+  }
   for (int c = 0; c < 2 && e == cudaSuccess; ++c) {
     const BatchSetting r = resident_setting(c);
     BatchKernels k = batch_kernels(r.nb, r.tc, r.rm);
@@ -124,6 +137,7 @@ namespace slqr {
 struct BatchGroup {
   BatchSetting set;
   int begin = 0, count = 0, grid = 0;
+  int rows = 0;                 // most rows of a problem
   double cost = 0.0;
 };
 
@@ -206,13 +220,15 @@ static slqr_status batch_build(slqr_ctx *ctx, int count, const int *m, const int
     grp.begin = (int)bs.order.size();
     grp.count = (int)members[g].size();
     bs.order.insert(bs.order.end(), members[g].begin(), members[g].end());
-    BatchKernels k = batch_kernels(grp.set.nb, grp.set.tc, grp.set.rm);
+    for (int i : members[g]) grp.rows = std::max(grp.rows, m[i]);
+    BatchKernels k = batch_kernels(grp.set.nb, grp.set.tc, grp.set.rm, grp.rows);
     if (bs.mixed ? !k.mixed : !k.fp64)
       return fail(ctx, SLQR_EINVAL, "batch setting (%d, %d, resident %d) has no kernel here",
                   grp.set.nb, grp.set.tc, grp.set.rm);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, bs.mixed ? k.mixed : k.fp64, kThreads, bs.mixed ? k.smem_mixed : k.smem_fp64);
+        &per_sm, bs.mixed ? k.mixed : k.fp64, bs.mixed ? kThreads : k.threads_fp64,
+        bs.mixed ? k.smem_mixed : k.smem_fp64);
     if (e != cudaSuccess || per_sm < 1)
       return fail(ctx, SLQR_ECUDA, "batch occupancy: %s", cudaGetErrorString(e));
     grp.grid = std::min(grp.count, per_sm * ctx->num_sms);
@@ -237,11 +253,11 @@ static void batch_kernel_launch(const BatchSetup &bs, char *base, int *status, d
   int *d_order = (int *)(base + 256 + bs.table_bytes);
   for (size_t gi = 0; gi < bs.groups.size(); ++gi) {
     const BatchGroup &g = bs.groups[gi];
-    BatchKernels k = batch_kernels(g.set.nb, g.set.tc, g.set.rm);
+    BatchKernels k = batch_kernels(g.set.nb, g.set.tc, g.set.rm, g.rows);
     if (!bs.mixed) {
       BatchParams bp{d_probs, d_order + g.begin, g.count, counters + gi, status};
       void *args[] = {&bp};
-      cudaLaunchKernel(k.fp64, dim3(g.grid), dim3(kThreads), args, k.smem_fp64, s);
+      cudaLaunchKernel(k.fp64, dim3(g.grid), dim3(k.threads_fp64), args, k.smem_fp64, s);
     } else {
       BatchMixedParams mp{d_probs, d_order + g.begin, g.count, counters + gi, status, err,
                           (float *)(base + bs.head), (double *)(base + bs.head + bs.af_bytes),

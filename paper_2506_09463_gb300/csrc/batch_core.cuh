@@ -893,14 +893,17 @@ constexpr size_t batch_mixed_smem_bytes() {
 struct BatchKernels {
   const void *fp64 = nullptr, *mixed = nullptr;
   size_t smem_fp64 = 0, smem_mixed = 0;
+  int threads_fp64 = kThreads;
 };
 
 template <int NB, int TC>
 BatchKernels batch_kernels_of() {
   BatchKernels k;
-  k.fp64 = (const void *)batch_factor_fp64_kernel<NB, TC>;
+  if constexpr (NB != kBNBDefault || TC != kBTCDefault) {   // (the default: batch_fx.cu)
+    k.fp64 = (const void *)batch_factor_fp64_kernel<NB, TC>;
+    k.smem_fp64 = BatchSmem<double, NB, TC>::kBytes;
+  }
   k.mixed = (const void *)batch_factor_mixed_kernel<NB, TC>;
-  k.smem_fp64 = BatchSmem<double, NB, TC>::kBytes;
   k.smem_mixed = batch_mixed_smem_bytes<NB, TC>();
   return k;
 }
@@ -919,5 +922,8 @@ BatchKernels batch_resident_kernels_of() {
 BatchKernels batch_kernels_nb8(int tc);
 BatchKernels batch_kernels_nb16(int tc);
 BatchKernels batch_kernels_nb32(int tc);
+// the FP64 kernel of the default setting for problems of at most `rows` rows
+// (batch_fx.cu)
+BatchKernels batch_fx_kernels(int rows);
 
 }  // namespace slqr
