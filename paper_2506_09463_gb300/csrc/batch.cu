@@ -155,6 +155,20 @@ struct BatchSetup {
 
 constexpr int kBMaxGroups = 64;   // work counters in the first 256 bytes of the layout
 
+// Bytes of the device layout, with at most `cap` CTAs a group: each CTA of a mixed
+// launch has its own scratch, and where that of every resident CTA (three to an SM)
+// does not fit, two to an SM do with less.
+static size_t batch_bytes(BatchSetup &bs, int cap = 1 << 30) {
+  bs.max_grid = 0;
+  for (BatchGroup &g : bs.groups) {
+    g.grid = std::min(g.grid, cap);
+    bs.max_grid = std::max(bs.max_grid, g.grid);
+  }
+  bs.af_bytes = bs.mixed ? (size_t)bs.max_grid * kBMaxRows * kBMaxRows * sizeof(float) : 0;
+  bs.gt_bytes = bs.mixed ? (size_t)bs.max_grid * kBGtDoubles * sizeof(double) : 0;
+  return bs.head + bs.af_bytes + bs.gt_bytes;
+}
+
 // Validate the arguments and build the setup (no device work).
 static slqr_status batch_build(slqr_ctx *ctx, int count, const int *m, const int *n,
                                const int *ntop, double *const *A, const int *lda,
@@ -232,15 +246,12 @@ static slqr_status batch_build(slqr_ctx *ctx, int count, const int *m, const int
     if (e != cudaSuccess || per_sm < 1)
       return fail(ctx, SLQR_ECUDA, "batch occupancy: %s", cudaGetErrorString(e));
     grp.grid = std::min(grp.count, per_sm * ctx->num_sms);
-    bs.max_grid = std::max(bs.max_grid, grp.grid);
     groups.push_back(grp);
   }
   bs.groups = groups;
   // device layout: [work counters 256 B][problem table][order][per-CTA scratch (mixed)]
   bs.table_bytes = align_up(sizeof(BatchProblem) * count, 256);
   bs.head = align_up(256 + bs.table_bytes + sizeof(int) * count, 256);
-  bs.af_bytes = bs.mixed ? (size_t)bs.max_grid * kBMaxRows * kBMaxRows * sizeof(float) : 0;
-  bs.gt_bytes = bs.mixed ? (size_t)bs.max_grid * kBGtDoubles * sizeof(double) : 0;
   return SLQR_OK;
 }
 
@@ -281,7 +292,8 @@ slqr_status batch_launch(slqr_ctx *ctx, int count, const int *m, const int *n, c
   BatchSetup bs;
   slqr_status st = batch_build(ctx, count, m, n, ntop, A, lda, up, b, prec, bs);
   if (st != SLQR_OK) return st;
-  st = ensure_workspace(ctx, bs.head + bs.af_bytes + bs.gt_bytes);
+  st = ensure_workspace(ctx, batch_bytes(bs));
+  if (st != SLQR_OK && bs.mixed) st = ensure_workspace(ctx, batch_bytes(bs, 2 * ctx->num_sms));
   if (st != SLQR_OK) return st;
   char *base = (char *)ctx->ws.ptr;
   cudaStream_t s = (cudaStream_t)stream;
@@ -605,12 +617,17 @@ extern "C" slqr_status slqr_batch_plan_create(slqr_ctx *ctx, int count, const in
     delete plan;
     return st;
   }
-  const size_t bytes = plan->bs.head + plan->bs.af_bytes + plan->bs.gt_bytes;
+  size_t bytes = batch_bytes(plan->bs);
+  if (ctx->hbm_budget && bytes > ctx->hbm_budget) bytes = batch_bytes(plan->bs, 2 * ctx->num_sms);
   if (ctx->hbm_budget && bytes > ctx->hbm_budget) {
     delete plan;
     return fail(ctx, SLQR_EBUSY, "batch plan of %zu bytes exceeds the HBM budget", bytes);
   }
   e = cudaMalloc(&plan->dev, bytes);
+  if (e == cudaErrorMemoryAllocation && plan->bs.mixed) {
+    cudaGetLastError();
+    e = cudaMalloc(&plan->dev, batch_bytes(plan->bs, 2 * ctx->num_sms));
+  }
   if (e == cudaSuccess)
     e = cudaMemcpy(plan->dev + 256, plan->bs.probs.data(), sizeof(BatchProblem) * count,
                    cudaMemcpyHostToDevice);

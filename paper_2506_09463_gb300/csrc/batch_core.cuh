@@ -152,7 +152,7 @@ struct BatchSmem {
 // factor a shared-memory copy of the problem); PR is the panel's row capacity.
 template <typename T, int NB, int TC, int PR = kBMaxRows>
 __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, double *Bcol,
-                                  double *G_out, double *tau_out, char *smraw, int ntop) {
+                                  T *G_out, T *tau_out, char *smraw, int ntop) {
   using SM = BatchSmem<T, NB, TC, PR>;
   using TL = BTile<NB, TC>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -161,15 +161,18 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
   T *Wt = Ps + SM::kPanel;
   T *Gt = Wt + SM::kW;              // G and tau of the panel in T (phase B)
   T *taut = Gt + SM::kG;
-  double *Gs = (double *)(smraw + align_up_c(SM::kBytesT, 16));
-  double *dots = Gs + SM::kG;
-  double *sig = dots + NB;
-  double *tau = sig + NB;
-  double *ups = tau + NB;
-  double *scl = ups + NB;           // per-column scale 2^-E of the panel
-  double *sinv = scl + NB;          // and its inverse 2^E
-  double *fst = sinv + NB;          // 1: FP32 pivot for this column (T == float, |E| <= 60)
-  double *misc = fst + NB;          // [0] = norm
+  // the panel's small quantities, in T: on an FP32 panel every conversion from or
+  // to FP64 would take the FP64 pipe for 16 clocks a warp
+  T *Gs = (T *)(smraw + align_up_c(SM::kBytesT, 16));
+  T *dots = Gs + SM::kG;
+  T *sig = dots + NB;
+  T *tau = sig + NB;
+  T *ups = tau + NB;
+  T *scl = ups + NB;                // per-column scale 2^-E of the panel
+  T *sinv = scl + NB;               // and its inverse 2^E
+  T *fst = sinv + NB;               // 1: FP32 pivot for this column (T == float, |E| <= 60)
+  T *norm = fst + NB;
+  double *norm64 = (double *)(smraw + align_up_c(SM::kBytesT, 16) + (SM::kG + 7 * NB + 4) * sizeof(double));
   // An FP32 factorization (T == float) forms the norm, the pivot and the
   // multipliers in FP32 (its per-column chain then stays off the FP64 pipe);
   // a column whose power-of-two scale is extreme for FP32 forms its pivot in
@@ -206,9 +209,9 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
           int E = (int)((mx >> 20) & 0x7ff) - 1023;
           // (FP32: 2^-E and 2^E both normal floats)
           E = kF32 ? min(max(E, -126), 126) : min(max(E, -1000), 1022);
-          scl[c] = b_pow2(-E);
-          sinv[c] = b_pow2(E);
-          fst[c] = (kF32 && E >= -60 && E <= 60) ? 1.0 : 0.0;
+          scl[c] = (T)b_pow2(-E);
+          sinv[c] = (T)b_pow2(E);
+          fst[c] = (kF32 && E >= -60 && E <= 60) ? T(1) : T(0);
         }
       }
     }
@@ -221,7 +224,7 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
         const int c = warp + kBWarps * t;
         if (c >= nbw) continue;
         if (c == j) {
-          const T sc = (T)scl[j];
+          const T sc = scl[j];
           T S = T(0), S1 = T(0);                       // two chains
           int r = j + lane;
           for (; r + 32 < M; r += 64) {
@@ -235,9 +238,12 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
           }
           S = b_warp_sum(S + S1);
           if (lane == 0) {                             // exact rescale by 2^E
-            if (S == T(0)) misc[0] = 0.0;
-            else if (kF32 && fst[j] != 0.0) misc[0] = (double)(sqrt(S) * (T)sinv[j]);
-            else misc[0] = sqrt((double)S) * sinv[j];
+            if (S == T(0) || (kF32 && fst[j] != T(0))) {
+              *norm = S == T(0) ? T(0) : sqrt(S) * sinv[j];
+              if (fst[j] == T(0)) *norm64 = 0.0;
+            } else {
+              *norm64 = sqrt((double)S) * (double)sinv[j];
+            }
           }
         } else {
           const T *col = Ps + c * PR;
@@ -251,16 +257,15 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
           acc += acc1;
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-          if (lane == 0) dots[c] = (double)acc;
+          if (lane == 0) dots[c] = acc;
         }
       }
       __syncthreads();
-      const double s = misc[0];
-      const bool defined = (s != 0.0);
-      double cl = 0.0, upk = 0.0, tk = 0.0;
-      if (kF32 && fst[j] != 0.0) {                     // FP32 pivot and multipliers
-        const T sT = (T)s, x0 = x[j];
-        T clT = T(0), upT = T(0), tkT = T(0);
+      bool defined;
+      T clT = T(0), upT = T(0), tkT = T(0);
+      if (kF32 && fst[j] != T(0)) {                    // FP32 pivot and multipliers
+        const T sT = *norm, x0 = x[j];
+        defined = sT != T(0);
         if (defined) {
           clT = (x0 > T(0)) ? -sT : sT;
           upT = x0 - clT;
@@ -269,14 +274,13 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
         if (tid < nbw) {
           const int c = tid;
           const T pr_c = Ps[c * PR + j];
-          if (c > j) sig[c] = defined ? (double)(-(upT * pr_c + (T)dots[c]) * tkT) : 0.0;
-          else if (c < j) Gs[c + j * NB] = (double)(pr_c * upT + (T)dots[c]);
+          if (c > j) sig[c] = defined ? -(upT * pr_c + dots[c]) * tkT : T(0);
+          else if (c < j) Gs[c + j * NB] = pr_c * upT + dots[c];
         }
-        cl = clT;
-        upk = upT;
-        tk = tkT;
       } else {
-        const double x0 = (double)x[j];
+        const double s = *norm64, x0 = (double)x[j];
+        double cl = 0.0, upk = 0.0, tk = 0.0;
+        defined = (s != 0.0);
         if (defined) {
           cl = (x0 > 0.0) ? -s : s;
           upk = x0 - cl;
@@ -286,19 +290,21 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
           const int c = tid;
           const double pr_c = (double)Ps[c * PR + j];
           // sigma_c = (up p_c + D_c) / b = -(up p_c + D_c) tau
-          if (c > j) sig[c] = defined ? -(upk * pr_c + dots[c]) * tk : 0.0;
-          else if (c < j) Gs[c + j * NB] = pr_c * upk + dots[c];
+          if (c > j) sig[c] = defined ? (T)(-(upk * pr_c + (double)dots[c]) * tk) : T(0);
+          else if (c < j) Gs[c + j * NB] = (T)(pr_c * upk + (double)dots[c]);
         }
+        clT = (T)cl;
+        upT = (T)upk;
+        tkT = (T)tk;
       }
       __syncthreads();
       if (defined) {
-        const T upT = (T)upk;
 #pragma unroll
         for (int t = 0; t < TL::NBW8; ++t) {
           const int c = warp + kBWarps * t;
           if (c > j && c < nbw) {
             T *col = Ps + c * PR;
-            const T sg = (T)sig[c];
+            const T sg = sig[c];
             for (int r = j + 1 + lane; r < M; r += 32) col[r] = fma(sg, x[r], col[r]);
             if (lane == 0) col[j] = fma(sg, upT, col[j]);
           }
@@ -306,9 +312,9 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
       }
       __syncthreads();
       if (tid == 0) {
-        if (defined) Ps[j * PR + j] = (T)cl;
-        tau[j] = tk;
-        ups[j] = upk;
+        if (defined) Ps[j * PR + j] = clT;
+        tau[j] = tkT;
+        ups[j] = upT;
       }
       __syncthreads();
     }
@@ -318,22 +324,22 @@ __device__ void batch_factor_core(T *A, int lda, int m, int n, double *up_out, d
       int c = idx / M, r = idx - c * M;
       if (!(ntop > 0 && r < nbw && r > c)) A[SLQR_IDX(k0 + prow(r), k0 + c, lda)] = Ps[c * PR + r];
     }
-    if (tid < nbw) up_out[k0 + tid] = ups[tid];
+    if (tid < nbw) up_out[k0 + tid] = (double)ups[tid];
     if (G_out) {
-      double *Gp = G_out + (size_t)(k0 / NB) * NB * NB;
+      T *Gp = G_out + (size_t)(k0 / NB) * NB * NB;
       for (int idx = tid; idx < NB * NB; idx += kThreads) {
         int jj = idx / NB, q = idx - jj * NB;
-        Gp[idx] = (q < jj && jj < nbw) ? Gs[idx] : 0.0;
+        Gp[idx] = (q < jj && jj < nbw) ? Gs[idx] : T(0);
       }
-      if (tid < NB) tau_out[k0 + tid] = (tid < nbw) ? tau[tid] : 0.0;
+      if (tid < NB) tau_out[k0 + tid] = (tid < nbw) ? tau[tid] : T(0);
     }
     __syncthreads();
     for (int idx = tid; idx < NB * NB; idx += kThreads) {
       int c = idx / NB, r = idx - c * NB;
-      if (r <= c && r < M) Ps[c * PR + r] = (r == c && c < nbw) ? (T)ups[c] : T(0);
-      Gt[idx] = (T)Gs[idx];
+      if (r <= c && r < M) Ps[c * PR + r] = (r == c && c < nbw) ? ups[c] : T(0);
+      Gt[idx] = Gs[idx];
     }
-    if (tid < NB) taut[tid] = (T)tau[tid];
+    if (tid < NB) taut[tid] = tau[tid];
     __syncthreads();
 
     // trailing columns [k0 + nbw, n), plus Bcol as one more column
@@ -576,7 +582,7 @@ constexpr int kBRowsPerThread = kBMaxRows / kThreads;
 static_assert(kBRowsPerThread * kThreads == kBMaxRows, "rows per thread");
 
 template <int NB>
-__device__ void mixed_apply_q(const float *Af, int m, int n, const double *G, const double *tau,
+__device__ void mixed_apply_q(const float *Af, int m, int n, const float *G, const float *tau,
                               const double *up, float *y, float *red, bool forward) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = num_reflectors(m, n);
@@ -597,11 +603,14 @@ __device__ void mixed_apply_q(const float *Af, int m, int n, const double *G, co
     for (int t = 0; t < kBRowsPerThread; ++t) {
       const int i = tid + t * kThreads;
       const bool in = i < M;
+      // (one conversion of up a thread: in the loop over a it took the FP64 pipe
+      // 16 times)
+      const float upi = t == 0 && i < nbw ? (float)up[k0 + i] : 0.f;
 #pragma unroll
       for (int a = 0; a < NB; ++a) {
         float v = 0.f;
-        if (in && a < nbw && i >= a)
-          v = (i == a) ? (float)up[k0 + a] : Af[SLQR_IDX(k0 + i, k0 + a, m)];
+        if (in && a < nbw && i > a) v = Af[SLQR_IDX(k0 + i, k0 + a, m)];
+        if (t == 0 && i == a) v = upi;
         vr[t][a] = v;
       }
       yv[t] = in ? y[k0 + i] : 0.f;
@@ -630,7 +639,7 @@ __device__ void mixed_apply_q(const float *Af, int m, int n, const double *G, co
     // w_j and its column (forward) or row of G; at step q lane q's value is
     // final and the lanes still open subtract its contribution
     if (warp == 0) {
-      const double *Gp = G + (size_t)pnl * NB * NB;
+      const float *Gp = G + (size_t)pnl * NB * NB;
       const int j = lane;
       const bool act = j < nbw;
       float t = 0.f;
@@ -638,11 +647,11 @@ __device__ void mixed_apply_q(const float *Af, int m, int n, const double *G, co
 #pragma unroll
         for (int w8 = 0; w8 < kBWarps; ++w8) t += red[w8 * NB + j];
       }
-      const float tj = act ? (float)tau[k0 + j] : 0.f;
+      const float tj = act ? tau[k0 + j] : 0.f;
       float gl[NB];
 #pragma unroll
       for (int q = 0; q < NB; ++q)
-        gl[q] = (act && q < nbw) ? (float)(forward ? Gp[q + j * NB] : Gp[j + q * NB]) : 0.f;
+        gl[q] = (act && q < nbw) ? (forward ? Gp[q + j * NB] : Gp[j + q * NB]) : 0.f;
       float wf = 0.f;
 #pragma unroll
       for (int s2 = 0; s2 < NB; ++s2) {
@@ -740,16 +749,37 @@ static __device__ double block_max_abs(double v, double *red) {
   return r;
 }
 
+// 2^-e for a column with an entry that is not a normal number (a warp)
+static __device__ __noinline__ double mixed_column_scale(const double *Aj, int m) {
+  double mx = 0.0;
+  for (int i = threadIdx.x & 31; i < m; i += 32) mx = fmax(mx, fabs(Aj[i]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  int ex = 0;
+  if (mx > 0.0 && isfinite(mx)) {
+    frexp(mx, &ex);
+    ex = max(-1000, min(1000, ex));
+  }
+  return ldexp(1.0, -ex);
+}
+
+// CTAs of the mixed kernel on an SM: three with panels of 16 (80 registers a
+// thread), since its phases wait on each other more than they compute (2000
+// problems of up to 512 rows: two CTAs 17.7 ms, three 14.4, four, which spill,
+// 16.6).
+template <int NB>
+constexpr int batch_min_ctas_mixed() { return NB == 16 ? 3 : batch_min_ctas<NB>(); }
+
 template <int NB, int TC>
-__global__ void __launch_bounds__(kThreads, batch_min_ctas<NB>())
+__global__ void __launch_bounds__(kThreads, batch_min_ctas_mixed<NB>())
 batch_factor_mixed_kernel(BatchMixedParams bp) {
   extern __shared__ __align__(16) char smraw[];
   __shared__ int s_item;
   __shared__ double red[kBWarps];
   float *Af = bp.af + (size_t)blockIdx.x * kBMaxRows * kBMaxRows;
-  double *G = bp.gt + (size_t)blockIdx.x * kBGtDoubles;
-  double *tau = G + kBGDoubles;
-  double *up = tau + kBMaxRows;
+  float *G = (float *)(bp.gt + (size_t)blockIdx.x * kBGtDoubles);
+  float *tau = (float *)(bp.gt + (size_t)blockIdx.x * kBGtDoubles + kBGDoubles);
+  double *up = bp.gt + (size_t)blockIdx.x * kBGtDoubles + kBGDoubles + kBMaxRows;
   double *dcol = up + kBMaxRows;       // d_j = 2^-e_j: the FP32 copy is of A D
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (;;) {
@@ -772,24 +802,30 @@ batch_factor_mixed_kernel(BatchMixedParams bp) {
     // column of A D in [1/2, 1): no FP32 overflow or underflow of products for
     // any column scale), the FP32 working copy of A D (ld = m), then its FP32
     // factorization; the refinement solves for y with x = D y
+    // (the column's largest magnitude from the bits of its finite entries, then
+    // the same warp's copy of it: no division, no comparison in FP64)
     for (int j = warp; j < n; j += kBWarps) {
-      double mx = 0.0;
-      for (int i = lane; i < m; i += 32) mx = fmax(mx, fabs(pr.A[SLQR_IDX(i, j, pr.lda)]));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (lane == 0) {
-        int ex = 0;
-        if (mx > 0.0 && isfinite(mx)) {
-          frexp(mx, &ex);
-          ex = max(-1000, min(1000, ex));
-        }
-        dcol[j] = ldexp(1.0, -ex);
+      const double *Aj = pr.A + (size_t)j * pr.lda;
+      unsigned mh = 0;
+      bool odd = false;
+#pragma unroll 4
+      for (int i = lane; i < m; i += 32) {
+        const unsigned h = (unsigned)__double2hiint(Aj[i]) & 0x7fffffffu;
+        odd |= h >= 0x7ff00000u || (h < 0x00100000u && h != 0);
+        mh = max(mh, h);
       }
-    }
-    __syncthreads();
-    for (int idx = tid; idx < m * n; idx += kThreads) {
-      int c = idx / m, r = idx - c * m;
-      Af[idx] = (float)(pr.A[SLQR_IDX(r, c, pr.lda)] * dcol[c]);
+      mh = __reduce_max_sync(0xffffffffu, mh);
+      double d;
+      if (__any_sync(0xffffffffu, odd) || mh < 0x00100000u) {
+        d = mixed_column_scale(Aj, m);
+      } else {
+        const int ex = max(-1000, min(1000, (int)(mh >> 20) - 1022));
+        d = b_pow2(-ex);
+      }
+      if (lane == 0) dcol[j] = d;
+      float *Fj = Af + (size_t)j * m;
+#pragma unroll 4
+      for (int i = lane; i < m; i += 32) Fj[i] = (float)(Aj[i] * d);
     }
     __syncthreads();
     batch_factor_core<float, NB, TC>(Af, m, m, n, up, nullptr, G, tau, smraw, pr.ntop);
@@ -810,8 +846,12 @@ batch_factor_mixed_kernel(BatchMixedParams bp) {
     double err = 1.0, prev = 1e300;
     for (int it = 0; it < bp.max_it; ++it) {
       // f = b - r - A x (FP64), one thread per row
-      // (four partial sums: the dependent FP64 chain is a quarter as long)
-      for (int i = tid; i < m; i += kThreads) {
+      // (four partial sums: the dependent FP64 chain is a quarter as long).  The
+      // first sweep has r = 0 and x = 0: f = b, g = 0, h = 0.
+      if (it == 0) {
+        for (int i = tid; i < m; i += kThreads) f[i] = (float)pr.b[i];
+        for (int i = tid; i < n; i += kThreads) g[i] = 0.f;
+      } else for (int i = tid; i < m; i += kThreads) {
         double a0 = pr.b[i] - r[i], a1 = 0.0, a2 = 0.0, a3 = 0.0;
         int j = 0;
         for (; j + 3 < n; j += 4) {
@@ -824,7 +864,7 @@ batch_factor_mixed_kernel(BatchMixedParams bp) {
         f[i] = (float)((a0 + a1) + (a2 + a3));
       }
       // g = -D A^T r (FP64), one warp per column
-      for (int j = warp; j < n; j += kBWarps) {
+      for (int j = it == 0 ? n : warp; j < n; j += kBWarps) {
         double acc = 0.0;
         for (int i = lane; i < m; i += 32) acc = fma(pr.A[SLQR_IDX(i, j, pr.lda)], r[i], acc);
 #pragma unroll
@@ -832,7 +872,7 @@ batch_factor_mixed_kernel(BatchMixedParams bp) {
         if (lane == 0) g[j] = (float)(-acc * dcol[j]);
       }
       __syncthreads();
-      bool zero = mixed_trsv(Af, m, n, g, false);            // h = R^-T g (in g)
+      bool zero = it > 0 && mixed_trsv(Af, m, n, g, false);  // h = R^-T g (in g)
       mixed_apply_q<NB>(Af, m, n, G, tau, up, f, w, true);    // d = Q^T f (in f)
       for (int i = tid; i < m; i += kThreads) e[i] = (i < n) ? f[i] - g[i] : f[i];
       __syncthreads();
