@@ -171,3 +171,43 @@ def test_panel_shapes(ctx, m, n):
     F, up, qtb, x, st = run_gpu(ctx, A, b)
     assert st == 0
     check_against_oracle(A, b, F, up, qtb, x)
+
+
+# back-substitution of few right-hand sides in one launch: one row block, a ragged
+# last one, several, and more than are resident at once; zero and not finite
+# diagonal entries
+@pytest.mark.parametrize("n", [64, 65, 127, 129, 640, 2049, 9800])
+@pytest.mark.parametrize("nrhs", [1, 3, 4, 5])
+@pytest.mark.parametrize("kind", ["plain", "zero", "nan"])
+def test_solve_r_few_right_hand_sides(ctx, n, nrhs, kind):
+    g = torch.Generator(device="cuda").manual_seed(n + nrhs)
+    R = torch.randn(n, n, generator=g, dtype=torch.float64, device="cuda") / n ** 0.5   # R^T
+    R.diagonal().copy_(2.0 + torch.rand(n, generator=g, dtype=torch.float64, device="cuda"))
+    B0 = torch.randn(nrhs, n, generator=g, dtype=torch.float64, device="cuda")
+    k = n // 2
+    if kind == "zero":
+        R[k, k] = 0.0
+    if kind == "nan":
+        R[n - 1, n - 1] = float("nan")
+    B = B0.clone()
+    ctx.solve_r(R.T, B.T)
+    st = ctx.sync()
+    U_ = torch.triu(R.T)
+    if kind == "nan":
+        assert torch.isnan(B).all()
+        return
+    assert st == (0 if kind == "plain" else ctx_rank())
+    if kind == "zero":                             # x_k = 0, the other equations hold
+        assert (B[:, k] == 0).all()
+        U_[k, k] = 1.0
+        B0[:, k] = (U_[k, k + 1:] @ B[:, k + 1:].T)
+    # row-wise backward error of the blocks' products: 64 + n terms, the block inverses
+    # with condition below (1 + 64 max |R_ij| / 2)^2 of well-scaled rows
+    res = (U_ @ B.T - B0.T).abs()
+    scale = U_.abs() @ B.T.abs() + B0.T.abs()
+    assert (res <= (n + 64) * 16 * U * scale).all()
+
+
+def ctx_rank():
+    from paper_2506_09463_gb300 import abi
+    return abi.SLQR_ERANK
