@@ -11,11 +11,10 @@
 //   exchange      the CTAs' sums of w: added within a cluster by one of its CTAs
 //                 (st.async, mbarrier), the clusters' sums through L2, each slot
 //                 polled until it holds a value (as in panel_grid.cu)
-//   w' = T^T w    by substitution with T^{-1} = striu(V^T V) + diag(1/tau), one
-//                 warp per right-hand side, in every CTA
+//   w' = T^T w    with T formed before (qt_t_kernel), in every CTA
 //   b -= V w'
-// per panel.  What bounds it is latency: the exchange, the 64-step substitution
-// and 16 clocks of the FP64 pipe per warp instruction; V is read once.
+// per panel.  What bounds it is latency: the exchange and 16 clocks of the FP64
+// pipe per warp instruction; V is read once.
 #include "cluster_common.cuh"
 
 #include <algorithm>
@@ -26,6 +25,7 @@ using namespace cl;
 namespace {
 
 constexpr int kQvThreads = 512;
+constexpr int kQvT = 64 * 64;                   // T of a panel
 constexpr int kQvPolls = 5;                     // clusters' sums a lane collects (40 clusters)
 // An unset slot: all ones, a NaN that no arithmetic returns (published values
 // that carry it go out as the canonical NaN).
@@ -51,8 +51,52 @@ __device__ __forceinline__ void cp_async8(void *dst, const void *src) {
 
 }  // namespace
 
+// T of every panel (column-major, zero elsewhere), the inverse of striu(V^T V) +
+// diag(1 / tau), by back-substitution with eight lanes to a column (a tau of 0, an
+// undefined reflector, gives a zero row and column); grid (panels, column groups).
+// In the chain of panels the substitution itself, 64 steps, took 8000 clocks of a
+// panel's 22000; the product with T takes 2000 (4096 x 2048, one right-hand side:
+// 386 -> 295 us with this launch).
+__global__ void __launch_bounds__(128)
+qt_t_kernel(const double *__restrict__ wy, int K, int nb, double *__restrict__ out) {
+  __shared__ double Gs[64][65];
+  __shared__ double ts[64];
+  const int tid = threadIdx.x, l = tid & 7, j = blockIdx.y * 16 + (tid >> 3);
+  const int nbw = min(nb, K - (int)blockIdx.x * nb), top = blockIdx.y * 16 + 16;
+  const double *G = wy + (size_t)blockIdx.x * wy_panel_doubles(nb) + nb * nb, *tau = G + nb * nb;
+  double *T = out + (size_t)blockIdx.x * kQvT + (size_t)j * 64;
+  if (blockIdx.y * 16 >= nbw) {                // (columns past the panel; uniform)
+#pragma unroll
+    for (int u = 0; u < 8; ++u) T[l + 8 * u] = 0.0;
+    return;
+  }
+  for (int idx = tid; idx < 64 * top; idx += 128) {
+    const int i = idx & 63, c = idx >> 6;
+    Gs[i][c] = i < c && c < nbw ? G[i + c * nb] : 0.0;
+    if (c == 0) ts[i] = i < nbw ? tau[i] : 0.0;
+  }
+  __syncthreads();
+  double y[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) y[u] = 0.0;
+#pragma unroll
+  for (int i = 63; i >= 0; --i) {
+    if (i >= top) continue;                    // (uniform)
+    double t = (i == j && l == 0) ? 1.0 : 0.0;
+#pragma unroll
+    for (int u = i / 8; u < 8; ++u)            // (y is zero up to row i and past row j)
+      if (8 * u < top) t = fma(l + 8 * u <= j ? -Gs[i][l + 8 * u] : 0.0, y[u], t);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    t = t * ts[i];
+    if ((i & 7) == l && i <= j) y[i / 8] = t;
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) T[l + 8 * u] = y[u];
+}
+
 struct QtVecParams {
-  const double *A, *up, *Gt;
+  const double *A, *up, *T;
   double *B, *rec;               // rec: [panel][right-hand side][64][clusters], all ones before
   int m, K, nb, lda, ldb, nr, ntop;   // nb: panel width (64, or 32 in 64-column steps)
   int *status;
@@ -66,9 +110,9 @@ qt_vec_kernel(QtVecParams p) {
   constexpr int CG = kQvThreads / R;           // column groups of the update
   extern __shared__ __align__(16) unsigned char qv_smem[];
   double *Vs = (double *)qv_smem;              // [2][64][LD]
-  double *Gs = Vs + 2 * 64 * LD;               // [2][kFxGt]
+  double *Gs = Vs + 2 * 64 * LD;               // [2][kQvT]: T, column-major
   __shared__ double bs[NR][R];
-  __shared__ double s_w[NR][64];               // w, then w'
+  __shared__ double s_w[NR][64], s_wt[NR][64]; // w, w'
   __shared__ double s_part[NR][CG][R];
   __shared__ __align__(16) double s_recv[2][8][16 * NR];
   __shared__ __align__(8) unsigned long long s_mbar[2];
@@ -99,9 +143,9 @@ qt_vec_kernel(QtVecParams p) {
       if (c < nbw && row < p.m && tail) cp_async8(dst + r, col + row);
       else dst[r] = (c < nbw && row == k0 + c) ? p.up[k0 + c] : 0.0;
     }
-    const double *g = p.Gt + (size_t)pnl * kFxGt;
-    double *gd = Gs + (pnl & 1) * kFxGt;
-    for (int idx = tid; idx < kFxGt; idx += kQvThreads) cp_async8(gd + idx, g + idx);
+    const double *g = p.T + (size_t)pnl * kQvT;
+    double *gd = Gs + (pnl & 1) * kQvT;
+    for (int idx = tid; idx < kQvT; idx += kQvThreads) cp_async8(gd + idx, g + idx);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
 
@@ -210,21 +254,23 @@ qt_vec_kernel(QtVecParams p) {
       if (l8 == 0) s_w[k][c] = d;
     }
     __syncthreads();
-    // ---- w' = T^T w: row j of Gt folded into the entries still to come ----------
-    if (warp < NR) {
-      const double *Gt = Gs + buf * kFxGt;
-      double r0 = s_w[warp][lane], r1 = s_w[warp][lane + 32];
-      for (int j = 0; j < min(nbw, 32); ++j) {
-        const double wj = __shfl_sync(0xffffffffu, r0, j);
-        if (lane > j) r0 = fma(-Gt[j * 64 + lane], wj, r0);
-        r1 = fma(-Gt[j * 64 + lane + 32], wj, r1);
+    // ---- w' = T^T w: column c of T, entries l8, l8 + 8, .. up to the diagonal ------
+    {
+      const double *T = Gs + buf * kQvT + c * 64;
+      const int last = (4 * warp + 3) >> 3;
+      double wt[NR];
+#pragma unroll
+      for (int k = 0; k < NR; ++k) wt[k] = 0.0;
+      for (int u = 0; u <= last; ++u) {
+        const double t = T[l8 + 8 * u];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) wt[k] = fma(t, s_w[k][l8 + 8 * u], wt[k]);
       }
-      for (int j = 32; j < nbw; ++j) {
-        const double wj = __shfl_sync(0xffffffffu, r1, j - 32);
-        if (lane + 32 > j) r1 = fma(-Gt[j * 64 + lane + 32], wj, r1);
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        wt[k] = qv_sum8(wt[k]);
+        if (l8 == 0) s_wt[k][c] = wt[k];
       }
-      s_w[warp][lane] = lane < nbw ? Gt[64 * 64 + lane] * r0 : 0.0;
-      s_w[warp][lane + 32] = lane + 32 < nbw ? Gt[64 * 64 + lane + 32] * r1 : 0.0;
     }
     __syncthreads();
     // ---- b -= V w' ----------------------------------------------------------------
@@ -236,8 +282,8 @@ qt_vec_kernel(QtVecParams p) {
         double a0 = 0.0, a1 = 0.0;
 #pragma unroll
         for (int u = 0; u < CP; u += 2) {
-          a0 = fma(V[(g * CP + u) * LD + r], s_w[k][g * CP + u], a0);
-          a1 = fma(V[(g * CP + u + 1) * LD + r], s_w[k][g * CP + u + 1], a1);
+          a0 = fma(V[(g * CP + u) * LD + r], s_wt[k][g * CP + u], a0);
+          a1 = fma(V[(g * CP + u + 1) * LD + r], s_wt[k][g * CP + u + 1], a1);
         }
         s_part[k][g][r] = a0 + a1;
       }
@@ -278,7 +324,7 @@ static const void *qt_kernel(int R, int nr) {
   }
 }
 
-static size_t qt_smem(int R) { return (2 * 64 * (size_t)(R + 8) + 2 * kFxGt) * sizeof(double); }
+static size_t qt_smem(int R) { return (2 * 64 * (size_t)(R + 8) + 2 * kQvT) * sizeof(double); }
 
 slqr_status init_qt_vec_attrs(slqr_ctx *ctx) {
   for (int R : {32, 64, 128})
@@ -316,7 +362,7 @@ size_t qt_vec_bytes(const slqr_ctx *ctx, int m, int K, int nb) {
   int P = 0, cluster = 0;
   if (qt_shape(ctx, m, &P, &cluster) == 0) return 0;
   const size_t np = (size_t)num_panels(K, nb);
-  return np * (kFxGt + 4 * 64 * (size_t)(P / cluster)) * sizeof(double);
+  return np * (kQvT + 4 * 64 * (size_t)(P / cluster)) * sizeof(double);
 }
 
 slqr_status qt_vec(slqr_ctx *ctx, int m, int K, int nb, const double *A, int lda, const double *up,
@@ -325,15 +371,15 @@ slqr_status qt_vec(slqr_ctx *ctx, int m, int K, int nb, const double *A, int lda
   const int np = num_panels(K, nb);
   int P = 0, cluster = 0;
   const int R = qt_shape(ctx, m, &P, &cluster);
-  double *Gt = (double *)work;
+  double *T = (double *)work;
   int slot = prof_begin(ctx, stream);
-  fx_prep(wy, K, nb, Gt, stream);
+  qt_t_kernel<<<dim3(np, 4), 128, 0, stream>>>(wy, K, nb, T);
   prof_end(ctx, stream, slot, kTw, 0.0);
   const int most = R == 128 ? 2 : 4;
   for (int k = 0; k < nrhs; k += most) {
     const int nr = std::min(most, nrhs - k), tr = nr == 3 ? 4 : nr;
     QtVecParams p;
-    p.A = A; p.up = up; p.Gt = Gt; p.B = B + (size_t)k * ldb; p.rec = Gt + (size_t)np * kFxGt;
+    p.A = A; p.up = up; p.T = T; p.B = B + (size_t)k * ldb; p.rec = T + (size_t)np * kQvT;
     p.m = m; p.K = K; p.nb = nb; p.lda = lda; p.ldb = ldb; p.nr = nr; p.ntop = ntop;
     p.status = ctx->d_status; p.spin = ctx->spin_limit;
     cudaError_t e = cudaMemsetAsync(
