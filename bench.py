@@ -44,18 +44,9 @@ FP64_PEAK_TFLOPS = 4 * 152 * 2.070e9 / 1e12
 CPU_SAMPLE_COLS = 512   # oracle sample: leading m x 512 block of each matrix
 # factorization-only timings reported beside the step (N(0,1), seeds 2, 3, 4)
 FACTOR_ONLY_SHAPES = [(16384, 2048, 2), (8192, 8192, 3), (8192, 4096, 4)]
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the two
-# trailing-update kernels, scaled to this program's launches from a one-pass
-# capture of those two kernels alone on a small case larger than L2:
-#   python bench.py --ncu-case 8192 2048 && ncu --metrics dram__bytes_read.sum,\
-#     dram__bytes_write.sum,gpu__time_duration.sum --clock-control none \
-#     -k regex:"gemm_(vtx|upd)_kernel" -c 400 --csv python bench.py --ncu-case 8192 2048
-# There vtx moved 1.119 and upd 0.638 times their algorithmic bytes (vtx: 8 M (N + 64)
-# read; upd: X read and written, V and W' read); times this program's average algorithmic
-# bytes per launch (vtx 52.23 MB, upd 101.72 MB).  Re-measure the same way (never the
-# full-size program with DRAM counters) and reset to None whenever either kernel changes.
-TRAFFIC_PER_LAUNCH = {"vtx": {"dram": 1.119 * 52.23e6, "algorithmic": 52.23e6},
-                      "upd": {"dram": 0.638 * 101.72e6, "algorithmic": 101.72e6}}
+# FP64 products per FP16 digit product of the trailing-update kernels: 34 of the 49
+# products of seven digits (csrc/tc_fp64.cu)
+SPLIT_PRODUCTS = 34
 
 
 def max_over_ranks(ms, dist=None, device="cpu"):
@@ -479,22 +470,26 @@ def run_ours(args, rank, world, local_rank):
 
     # ---- roofline of the dominant kernel (most device time in the timed region) ----
     # the dominant kernel is the family carrying most of the algorithmic flops
-    # (the two trailing-update GEMMs carry equal shares; take the slower one);
-    # panel launches overlap those GEMMs on a second stream, so their event
-    # times are not exclusive
+    # (the two trailing-update products carry equal shares; take the slower one);
+    # panel launches overlap them on a second stream, so their event times are not
+    # exclusive.  Its products run on the tensor cores, SPLIT_PRODUCTS FP16 products
+    # to an FP64 one.
     dom = max(("vtx", "upd"), key=lambda k: prof[k][0])
     dms, dn, dfl = prof[dom]
     achieved = (dfl / dn) / (dms / dn / 1e3) / 1e12 if dn else 0.0
-    tr = TRAFFIC_PER_LAUNCH.get(dom)
-    roofline = {"kernel": dom, "bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
-                "traffic": tr["dram"] if tr else None,
-                "traffic_algorithmic": tr["algorithmic"] if tr else None,
-                "traffic_unit": "bytes per launch (ncu on 8192x2048, scaled to this program's launches)",
-                "peak_source": "derived: FP64 FMA pipe 4 flop/clk/SM x 152 SMs x 2070 MHz",
-                "peak_measured": peaks.get("fp64_fma_tflops"),
-                "frac_of_measured": (achieved / peaks["fp64_fma_tflops"]
-                                     if peaks.get("fp64_fma_tflops") else None)}
+    try:
+        with open(os.path.join(os.path.dirname(os.path.abspath(__file__)),
+                               "MEASURED_PEAKS.json")) as f:
+            tensor = float(json.load(f)["bf16_tflops_sustained"])
+        source = "measured sustained cuBLAS bf16 throughput / %d digit products" % SPLIT_PRODUCTS
+    except (OSError, KeyError, ValueError):
+        tensor, source = 1700.0, "1.7 PFLOP/s bf16 / %d digit products" % SPLIT_PRODUCTS
+    split_peak = tensor / SPLIT_PRODUCTS
+    roofline = {"kernel": dom, "bound": "tensor", "achieved": achieved, "peak": split_peak,
+                "unit": "TFLOP/s", "frac": achieved / split_peak,
+                "traffic": None, "traffic_algorithmic": None,
+                "peak_source": source, "fp64_pipe_peak": FP64_PEAK_TFLOPS,
+                "fp64_pipe_measured": peaks.get("fp64_fma_tflops")}
     kernels = {k: {"ms": v[0], "launches": v[1], "share_of_step_time": v[0] / max(1e-9, ms),
                    "tflops": (v[2] / (v[0] / 1e3) / 1e12) if v[0] > 0 else 0.0}
                for k, v in prof.items()}

@@ -166,11 +166,13 @@ void slqr_set_tuning(int panel_width, int panel_rows_min);
  * Process-wide choice of the panel kernel (no counterpart in the paper):
  *   ctas  0   chosen per panel: a thread-block cluster holds the panel when it
  *             fits (FP32 panels of up to 16 x ~800 rows at width 64; FP64
- *             panels of at most 1024 rows), else the cooperative panel
+ *             panels of at most 1024 rows at width 32; FP64 panels of width 64
+ *             in registers on one or several clusters), else the cooperative
+ *             panel
  *        -1   always the cooperative panel (one grid-wide exchange of partial
  *             sums through L2 per column); this also switches the Q
  *             applications of the mixed-precision refinement to their
- *             cooperative kernel
+ *             cooperative kernel (FP64 panels of width 64 stay on clusters)
  *         1..16  a cluster of that many CTAs wherever the panel's rows fit
  *             their shared memory, else the cooperative panel
  * The cluster panel splits the panel's rows over the CTAs of one cluster,
@@ -340,7 +342,7 @@ slqr_status slqr_apply_qt_stacked(slqr_ctx *ctx, int n, int m_eq, const double *
  * The host arrays are read before the call returns.  The problems must not
  * overlap in memory.  Errors: SLQR_EINVAL, SLQR_ENOMEM, SLQR_ECUDA.
  */
-#define SLQR_FP64 0   /* FP64 throughout (DFMA)                                   */
+#define SLQR_FP64 0   /* FP64 accuracy throughout                                 */
 #define SLQR_FP32 1   /* FP32 factorization + FP64-residual refinement            */
 #define SLQR_TF32 2   /* as SLQR_FP32, the two products of the rank-NB trailing
                          update (W = V^T X and X -= V W') on the tensor cores

@@ -6,7 +6,10 @@
 // applied one by one in the order they were built (each one an
 // update_trailing_non_pivot_row on every right-hand side, Alg. 2).  Here they
 // are applied NB at a time in compact-WY form, B <- B - V T^T (V^T B), using
-// the same tiled DFMA kernels as the trailing update of the factorization.
+// the kernels of the trailing update of the factorization: panels of 64 and at
+// least kFxMinCols right-hand sides on the tensor cores (tc_fp64.cu), fewer in one
+// launch for all panels (qt_vec.cu), the rest, and what the workspace of those does
+// not fit, with the tiled DFMA kernels.
 //
 // The compact-WY store (Vtop, strict upper V^T V, tau per panel) comes from
 // slqr_factor when the caller kept it, or is rebuilt here from (A, up): Vtop

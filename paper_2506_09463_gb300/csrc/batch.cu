@@ -5,7 +5,7 @@
 // update_trailing_non_pivot_row on every later column; Task 1 skip rule),
 // optionally followed by Q^T b and the back-substitution (Section 1: the
 // stored reflectors are reused by the solve); the kernels are in
-// batch_core.cuh.  Problems are independent, so one CTA owns one problem at a
+// batch_core.cuh and, FP64 at the default setting, batch_fx.cu.  Problems are independent, so one CTA owns one problem at a
 // time; persistent CTAs take the next problem from a device-side atomic
 // counter over a list ordered costliest first (longest-processing-time
 // first), the GPU descendant of the paper's shared main_queue of ready tasks

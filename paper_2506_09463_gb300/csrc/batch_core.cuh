@@ -21,7 +21,8 @@
 //    column, each over every (256 / TC)-th row), then W' = T^T W by forward
 //    substitution (one thread per column), then C -= V W' (the same lanes as
 //    W).
-// The FP64 kernel does all arithmetic in FP64 (DFMA).
+// The FP64 kernel does all arithmetic in FP64 (DFMA).  The default FP64 setting runs
+// batch_fx.cu instead, its products on the tensor cores.
 #pragma once
 #include "slqr_internal.cuh"
 
@@ -563,14 +564,6 @@ struct BatchMixedParams {
 // the column scales d_j of the equilibration
 constexpr size_t kBGDoubles = (size_t)kBMaxRows * kBNBMax;
 constexpr size_t kBGtDoubles = kBGDoubles + 3 * kBMaxRows;
-
-// V(i, a) of panel p from the FP32 factorization (rows relative to k0 = p*NB)
-static __device__ __forceinline__ float mixed_v(const float *Af, int m, const double *up, int k0,
-                                         int nbw, int i, int a) {
-  if (a >= nbw || i < a) return 0.f;
-  if (i == a) return (float)up[k0 + a];
-  return Af[SLQR_IDX(k0 + i, k0 + a, m)];
-}
 
 // y <- Q^T y (forward = true) or y <- Q y, panel by panel, FP32 arithmetic.
 // Per panel each thread loads the V entries of its rows (at most two: m <=

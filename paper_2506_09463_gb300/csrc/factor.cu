@@ -22,8 +22,13 @@
 //      gemm_vtx   W_s = V_s^T X_s on row slices s (partials),
 //      tw         W' = T^T W by forward substitution with striu(G), tau,
 //      gemm_upd   X -= V W'.
-//    All three run on the FP64 pipe (DFMA); on GB300 FP64 DMMA issues slower
+//    Here all three run on the FP64 pipe (DFMA); on GB300 FP64 DMMA issues slower
 //    than DFMA, so these are register-tiled DFMA kernels.
+// FP64 panels of 64 columns take faster kernels for both, with the same outputs:
+// panel_grid.cu (the panel in registers on thread-block clusters) and tc_fp64.cu
+// (the update on the tensor cores by exact splitting).  The kernels here serve the
+// other widths and precisions, panels too tall for the clusters, and contexts whose
+// budget does not hold the digit images.
 //
 // Rounding differs from the sequential order (blocked sums, power-of-two
 // scaled norms), so results agree with the sequential H12 to a tolerance,
@@ -1542,8 +1547,8 @@ slqr_status factor_f32(slqr_ctx *ctx, int m, int n, float *A, int lda, double *u
 // The FP64 factorization.  Few columns (n <= 256) have a compact-WY store in
 // panels of 32; unless that width was set (slqr_set_tuning, slqr_autotune) they
 // are factored in panels of 64 all the same, whose panel and update kernels are
-// the faster ones (256 x 128: 0.42 against 0.92 ms), and the store is taken from
-// theirs.
+// the faster ones (256 x 128, factor and solve: 1.55 ms in panels of 32, 0.69 in
+// panels of 64), and the store is taken from theirs.
 static slqr_status factor_fp64(slqr_ctx *ctx, int m, int n, double *A, int lda, double *up,
                                double *wy, cudaStream_t s, int ntop) {
   TuneEntry tuned;

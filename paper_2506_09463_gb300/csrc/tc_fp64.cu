@@ -16,10 +16,10 @@
 // pairs with i + j <= 7 are kept (the first dropped ones are 2^-8 times the
 // rounding above), one accumulator per order in tensor memory, and the eight
 // orders are put together in integer arithmetic before one rounding to FP64.
-// The residual ||A - Q R|| / ||A|| in 128-bit arithmetic: 3.70e-16 with these
+// The residual ||A - Q R|| / ||A|| in 128-bit arithmetic: 3.73e-16 with these
 // kernels, 4.92e-16 with the DFMA kernels of factor.cu (700 x 300 Gaussian),
-// 3.05e-16 against 3.38e-16 (3000 x 260), 2.94e-16 against 2.98e-16
-// (16384 x 260), 6.1e-16 against 9.2e-16 (rows graded over 10^16).
+// 3.08e-16 against 3.38e-16 (3000 x 260), 2.96e-16 against 2.98e-16
+// (16384 x 260), 5.2e-16 against 9.2e-16 (rows graded over 10^16).
 //
 // Why: the FP64 pipe of GB300 does 2 DFMA per SM and clock, 1.2 TFLOP/s, and
 // the products ran at 82-91% of that.  34 FP16 products cost 34/1834 of the
