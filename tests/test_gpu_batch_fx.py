@@ -14,7 +14,9 @@ from test_gpu_batch import U, check_problem, ctx, problem, run_batch  # noqa: F4
 
 pytestmark = pytest.mark.gpu
 
-# problems of one launch: the largest row count picks the kernel
+# problems of one launch: the largest row count and the number of problems (at most
+# 152, 304, more) pick the kernel
+COPIES = [1, 20, 40]
 LAUNCHES = {
     128: [(128, 128), (128, 127), (127, 16), (127, 17), (128, 15), (126, 9), (33, 32), (16, 15)],
     256: [(129, 129), (255, 31), (256, 256), (256, 33), (129, 8), (130, 7), (7, 7), (1, 1)],
@@ -22,18 +24,20 @@ LAUNCHES = {
 }
 
 
+@pytest.mark.parametrize("copies", COPIES)
 @pytest.mark.parametrize("rows", sorted(LAUNCHES))
-def test_edges_against_oracle(ctx, rows):  # noqa: F811
-    ms, ns = zip(*LAUNCHES[rows])
+def test_edges_against_oracle(ctx, rows, copies):  # noqa: F811
+    ms, ns = zip(*LAUNCHES[rows] * copies)
     res = run_batch(ctx, ms, ns, seed=rows)
     assert np.all(res["status"] == 0)
     for i, (m, n) in enumerate(LAUNCHES[rows]):
         check_problem(*problem(res, i, m, n))
 
 
+@pytest.mark.parametrize("copies", COPIES)
 @pytest.mark.parametrize("rows", sorted(LAUNCHES))
-def test_factor_only(ctx, rows):  # noqa: F811
-    ms, ns = zip(*LAUNCHES[rows])
+def test_factor_only(ctx, rows, copies):  # noqa: F811
+    ms, ns = zip(*LAUNCHES[rows] * copies)
     res = run_batch(ctx, ms, ns, seed=rows + 1, with_b=False)
     for i, (m, n) in enumerate(LAUNCHES[rows]):
         if n == 0:
@@ -47,6 +51,8 @@ def test_factor_only(ctx, rows):  # noqa: F811
 
 def _factor(ctx, A_list, setting):  # noqa: F811
     from paper_2506_09463_gb300 import abi
+    given = len(A_list)
+    A_list = A_list + [A_list[0]] * (310 if A_list[0].shape[0] < 256 else 0)   # (every kernel)
     count = len(A_list)
     dev = [torch.from_numpy(np.asfortranarray(A).T.copy()).cuda() for A in A_list]
     ups = [torch.zeros(A.shape[1], dtype=torch.float64, device="cuda") for A in A_list]
@@ -62,7 +68,7 @@ def _factor(ctx, A_list, setting):  # noqa: F811
         ctx.sync()
     finally:
         assert abi.slqr_batch_set_tuning(abi.SLQR_FP64, -1, 0, 0) == abi.SLQR_OK
-    return [d.cpu().numpy().T for d in dev], [u.cpu().numpy() for u in ups]
+    return [d.cpu().numpy().T for d in dev[:given]], [u.cpu().numpy() for u in ups[:given]]
 
 
 @pytest.mark.parametrize("span", [450, 960])
