@@ -25,7 +25,7 @@
 // the products ran at 82-91% of that.  34 FP16 products cost 34/1834 of the
 // same work at the tensor rate, so the products are bound by memory, by the
 // digit extraction and by the reassembly instead.  Both products over a whole
-// 8192 x 8192 factorization: 663 ms on the FP64 pipe, 88 ms here.
+// 8192 x 8192 factorization: 663 ms on the FP64 pipe, 50 ms here.
 //
 // Operand layout: K-major shared-memory images of the digit matrices, written
 // by the producing kernel in the exact (swizzled) form the MMA reads, so that
