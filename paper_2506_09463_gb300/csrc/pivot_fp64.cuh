@@ -15,26 +15,31 @@ __device__ __forceinline__ bool pivot_in_range(double S) {
 __device__ __forceinline__ bool bits_positive(double x) { return __double_as_longlong(x) > 0; }
 
 // s = sqrt(S), cl = -+s, up = x0 - cl and rb = 1 / (up cl) = -1 / (S + |x0| s)
-// for S in that range: a third-order Householder iteration each from the
-// hardware's approximate reciprocal (square root), good to 2^-20 or so, and a
-// Newton correction that takes s to half an ulp (its error enters every entry of
-// the reflector).  14 FP64 operations, all of one warp and so 64 clocks apart;
+// for S in that range, by Newton's iteration from the approximate reciprocal
+// square root and reciprocal that PTX has for FP64:
+//  * s: x^2 = S with the slope kept at its first value (the simplified Newton or
+//    chord iteration; Ortega and Rheinboldt 1970, section 7.1), s <- s + (S - s^2) h
+//    with h = y / 2.  From y = (1 + d) / sqrt(S), s = S y has the relative error d,
+//    the first step leaves -3/2 d^2 - d^3/2 and the second 3/2 d^3: with |d| below
+//    2^-19, 2^-56 of s before the last rounding.
+//  * rb: z <- z + z (1 - b z), whose error is squared (Newton).  The first step
+//    is on the b of the first s, beside the second step of s; it leaves 2^-37,
+//    so the second, on the final b, is exact but for its rounding.
+// Eight FP64 operations one after the other, of one warp and so 64 clocks apart;
 // sqrt() and a division with their range checks take 1600 clocks on an idle
-// pipe.
+// pipe.  s is within 0.55 units in the last place and rb within 3 2^-53 of itself,
+// the error of sqrt, x0 - cl, a product and a division being up to 5 2^-53
+// (tests/test_gpu_pivot.py).
 __device__ __forceinline__ void pivot_fp64(double S, double x0, double *cl, double *up, double *rb) {
   double y, z;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(S));
-  const double ax = fabs(x0);
-  const double s0 = S * y;
-  const double b0 = fma(ax, s0, S);                      // approximate -b, for the seed
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(b0));
-  const double e = fma(-s0, y, 1.0);                     // 1 - S y^2 = 1 - s0^2 / S
-  double s = fma(s0 * e, fma(e, 0.375, 0.5), s0);
-  const double hy = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));   // y / 2
-  s = fma(fma(-s, s, S), hy, s);
-  const double b = fma(ax, s, S);
-  const double f = fma(-b, z, 1.0);
-  *rb = -fma(fma(f, f, f), z, z);
+  const double ax = fabs(x0), h = 0.5 * y;
+  double s = S * y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(fma(ax, s, S)));
+  s = fma(fma(-s, s, S), h, s);
+  z = fma(z, fma(-fma(ax, s, S), z, 1.0), z);
+  s = fma(fma(-s, s, S), h, s);
+  *rb = -fma(z, fma(-fma(ax, s, S), z, 1.0), z);
   const double c = bits_positive(x0) ? -s : s;
   *cl = c;
   *up = x0 - c;
