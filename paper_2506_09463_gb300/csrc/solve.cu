@@ -126,13 +126,16 @@ trsm_step_kernel(const double *__restrict__ A, int lda, int n, int nrhs, double 
     if (r < rows) rhs = B[SLQR_IDX(row_begin + r, r0 + q, ldb)];
     if (r < cols) xsrc = B[SLQR_IDX(col_begin + r, r0 + q, ldb)];
   }
-  // this thread's part of row r of the tile times the vectors in Xs
-  auto product = [&]() {
+  // this thread's part of row r of the tile times the vectors in Xs, from column
+  // `from` on: row r of a block inverse takes no part of the values above it (zero
+  // times one that is not finite would reach the rows below)
+  auto product = [&](int from) {
     double a0 = 0.0, a1 = 0.0;
 #pragma unroll
     for (int c = 0; c < CW; c += 2) {
-      a0 = fma(Rs[cs * CW + c][r], Xs[q][cs * CW + c], a0);
-      a1 = fma(Rs[cs * CW + c + 1][r], Xs[q][cs * CW + c + 1], a1);
+      const int col = cs * CW + c;
+      if (col >= from) a0 = fma(Rs[col][r], Xs[q][col], a0);
+      if (col + 1 >= from) a1 = fma(Rs[col + 1][r], Xs[q][col + 1], a1);
     }
     a0 += a1;
     if (CQ > 1) {
@@ -149,7 +152,7 @@ trsm_step_kernel(const double *__restrict__ A, int lda, int n, int nrhs, double 
     for (int u = 0; u < PER; ++u) Rs[g + u * (kThreads / kTB)][r] = tile[u];
     if (cs == 0) Xs[q][r] = xsrc;
     __syncthreads();
-    rhs -= product();
+    rhs -= product(0);
     if (!diag && rhs_ok && cs == 0 && r < rows) B[SLQR_IDX(row_begin + r, r0 + q, ldb)] = rhs;
     __syncthreads();
   }
@@ -159,7 +162,7 @@ trsm_step_kernel(const double *__restrict__ A, int lda, int n, int nrhs, double 
   for (int u = 0; u < PER; ++u) Rs[g + u * (kThreads / kTB)][r] = inv[u];
   if (cs == 0) Xs[q][r] = (rhs_ok && r < rows) ? rhs : 0.0;
   __syncthreads();
-  const double x = product();
+  const double x = product(r);
   if (rhs_ok && cs == 0 && r < rows) B[SLQR_IDX(row_begin + r, r0 + q, ldb)] = x;
 }
 
@@ -229,7 +232,8 @@ trsm_chain_kernel(const double *__restrict__ A, int lda, int n, double *__restri
   __syncthreads();
   acc = 0.0;
 #pragma unroll
-  for (int u = 0; u < CW; ++u) acc = fma(inv[u], Xs[t & 1][g * CW + u], acc);
+  for (int u = 0; u < CW; ++u)                 // (from the diagonal on, as in the steps)
+    if (g * CW + u >= r) acc = fma(inv[u], Xs[t & 1][g * CW + u], acc);
   const double x = total(acc);
   if (g == 0) {
     const double v = trsm_unset(x) ? __longlong_as_double(0x7fffffffffffffffll) : x;
