@@ -130,6 +130,12 @@ qt_vec_kernel(QtVecParams p) {
     const int k0 = pnl * p.nb;
     return p.ntop > 0 ? row0 + R > p.ntop || (row0 + R > k0 && row0 < k0 + p.nb) : row0 + R > k0;
   };
+  // whether a row is one of panel pnl's: only those are read and changed, as in the
+  // tiled products (zero times a value that is not finite would reach the others)
+  auto panel_row = [&](int pnl, int row) {
+    const int k0 = pnl * p.nb;
+    return row >= k0 && (p.ntop == 0 || row < min(k0 + p.nb, p.K) || row >= p.ntop);
+  };
   // panel pnl's rows of V: the reflector tails, up on the diagonal, zeros above
   // (stacked: the tails are zero down to the rows of C, and not read there)
   auto fetch = [&](int pnl) {
@@ -170,6 +176,7 @@ qt_vec_kernel(QtVecParams p) {
   for (int pnl = 0; pnl < np; ++pnl) {
     const int buf = pnl & 1, nbw = min(p.nb, p.K - pnl * p.nb);
     const bool part_of = takes_part(pnl);               // (uniform over the CTA)
+    const bool whole = row0 >= (p.ntop > 0 ? p.ntop : pnl * p.nb);   // (all rows are the panel's)
     if (pnl + 1 < np && takes_part(pnl + 1)) {
       fetch(pnl + 1);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -186,8 +193,9 @@ qt_vec_kernel(QtVecParams p) {
         double a0 = 0.0, a1 = 0.0;
 #pragma unroll
         for (int i = 0; i < RPL; i += 2) {
-          a0 = fma(V[c * LD + l8 + 8 * i], bs[k][l8 + 8 * i], a0);
-          a1 = fma(V[c * LD + l8 + 8 * (i + 1)], bs[k][l8 + 8 * (i + 1)], a1);
+          const int r0 = l8 + 8 * i, r1 = r0 + 8;
+          if (whole || panel_row(pnl, row0 + r0)) a0 = fma(V[c * LD + r0], bs[k][r0], a0);
+          if (whole || panel_row(pnl, row0 + r1)) a1 = fma(V[c * LD + r1], bs[k][r1], a1);
         }
         part = qv_sum8(a0 + a1);
       }
@@ -262,6 +270,7 @@ qt_vec_kernel(QtVecParams p) {
 #pragma unroll
       for (int k = 0; k < NR; ++k) wt[k] = 0.0;
       for (int u = 0; u <= last; ++u) {
+        if (l8 + 8 * u > c) break;             // (T is zero from there on)
         const double t = T[l8 + 8 * u];
 #pragma unroll
         for (int k = 0; k < NR; ++k) wt[k] = fma(t, s_w[k][l8 + 8 * u], wt[k]);
@@ -294,7 +303,7 @@ qt_vec_kernel(QtVecParams p) {
       double s = s_part[k][0][r];
 #pragma unroll
       for (int g = 1; g < CG; ++g) s += s_part[k][g][r];
-      bs[k][r] -= s;
+      if (whole || panel_row(pnl, row0 + r)) bs[k][r] -= s;
     }
   }
   __syncthreads();
