@@ -105,6 +105,7 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
   unsigned *cm = (unsigned *)(sm + SM::kCm);        // column maxima: this panel's, the next one's
   __shared__ double s_part[RQ][16], s_prow[16], s_sig[16], s_piv[2];
   __shared__ double s_G[16 * 16], s_tau[16], s_up[16];
+  __shared__ __align__(16) unsigned s_mx[16][RQ];   // maxima of the panel's columns below the diagonal
   __shared__ int s_f[16], s_def, s_ecol[SM::CT];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gid = lane >> 2, tq = lane & 3;         // fragment row and column pair
@@ -144,6 +145,17 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
         v[i] = (c < nbw && r < M && !(ntop > 0 && r < nbw && r > c)) ? C[prow(r)] : 0.0;
       }
     }
+    {
+      // the column's own rows set its scale: an entry above the diagonal may be larger
+      // than the norm by more than its square holds
+      unsigned mx = 0;
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (i >= 2 || r0 + 8 * RQ * i >= c) mx = max(mx, fx_hi(v[i]));
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if ((lane & 7) == 0) s_mx[c][rq] = mx;
+    }
     if (c == 0) {
 #pragma unroll
       for (int i = 0; i < 16; ++i) xs[r0 + 8 * RQ * i] = (r0 + 8 * RQ * i > 0) ? v[i] : 0.0;
@@ -152,7 +164,10 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
     for (int j = 0; j < nbw; ++j) {
       const double *x = xs + (j & 1) * PR;
       // a column of extreme scale squares its scaled entries
-      const int E = min(max((int)((cur[k0 + j] >> 20) & 0x7ff) - 1023, -1000), 1022);
+      unsigned jmx = s_mx[j][0];
+#pragma unroll
+      for (int q = 1; q < RQ; ++q) jmx = max(jmx, s_mx[j][q]);
+      const int E = min(max((int)((jmx >> 20) & 0x7ff) - 1023, -1000), 1022);
       const bool extreme = abs(E) > 400;
       if (4 * cg + 3 >= j && 4 * cg < nbw) {
         double a = 0.0;
