@@ -198,7 +198,7 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
       int slot = prof_begin(ctx, stream);
       fx_split_v(A, lda, wyp, k0, nbw, m - k0 - skip, skip, tail, stream);
       prof_end(ctx, stream, slot, kVtx, 0.0);
-      if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip, wyp, gt + (size_t)pnl * kFxGt,
+      if (!fx_update(ctx, A, lda, k0, nbw, m - k0 - skip, skip, wyp, gt + (size_t)pnl * kFxGt,
                      tail, B, ldb, nrhs,
                      cmax + (size_t)pnl * nrhs,
                      pnl + 1 < np ? cmax + (size_t)(pnl + 1) * nrhs : nullptr, tail + fx_v, fx_work,

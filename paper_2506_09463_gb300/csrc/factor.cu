@@ -1419,6 +1419,10 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   auto gram_in_lookahead = [&](int pnl) {
     return pnl + 1 < np && std::min(NB, K - (pnl + 1) * NB) >= kFxMinCols;
   };
+  // (gpart: what panel_kernel would use for its partial terms)
+  auto gram_of = [&](int pnl) {
+    return FxGramBuffers{gram_base + (size_t)pnl * kFxGramBytes, gpart};
+  };
   auto gt_of = [&](int pnl) { return gt_base + (size_t)(pnl & 1) * kFxGt; };
   auto split_v = [&](int pnl, cudaStream_t s) {
     const int k0 = pnl * NB, nbw = std::min(NB, K - k0), skip = skip_of(k0, nbw);
@@ -1431,7 +1435,7 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       fx_split_v(A, lda, wyp, k0, nbw, m - k0 - skip, skip, vbuf[pnl & 1], s);
       prof_end(ctx, s, slot, kVtx, 0.0);
       if (gram)
-        fx_gram(ctx, nbw, m - k0 - skip, wyp, vbuf[pnl & 1], gram_base + (size_t)pnl * kFxGramBytes,
+        fx_gram(ctx, A, lda, k0, nbw, m - k0 - skip, skip, wyp, vbuf[pnl & 1], gram_of(pnl),
                 gt_of(pnl), s);
       else if (!on_grid(pnl))
         fx_prep(wyp, nbw, NB, gt_of(pnl), s);
@@ -1459,12 +1463,13 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       // maxima are not needed any more)
       if (fx && c_end - c_begin >= kFxMinCols) {
         const int skip = skip_of(k0, nbw);
-        if (!fx_update(ctx, k0, nbw, m - k0 - skip, skip,
+        const FxGramBuffers gram = gram_of(pnl);
+        if (!fx_update(ctx, A, lda, k0, nbw, m - k0 - skip, skip,
                        wy_store + (size_t)pnl * wy_panel_doubles(NB), gt_of(pnl), vbuf[pnl & 1],
                        A + (size_t)c_begin * lda, lda, c_end - c_begin,
                        cmax + (size_t)pnl * n + c_begin,
                        pnl + 1 < np ? cmax + (size_t)(pnl + 1) * n + c_begin : nullptr, fxw, fx_work,
-                       us, lookahead && on_grid(pnl) ? gram_base + (size_t)pnl * kFxGramBytes : nullptr))
+                       us, lookahead && on_grid(pnl) ? &gram : nullptr))
           return fail(ctx, SLQR_ENOMEM, "internal: trailing-update workspace too small");
         return check_launch(ctx, "trailing update");
       }

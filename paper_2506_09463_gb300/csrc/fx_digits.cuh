@@ -12,6 +12,23 @@ constexpr int kFxD = 7;                       // digits
 constexpr int kFxOrders = 8;                  // accumulated orders i + j
 constexpr int kFxNonFinite = 1 << 20;         // exponent that stands for Inf / NaN
 
+// Where the splitting loses digits.  A digit product of two vectors is known to 2^-57
+// or so of the product of their largest entries.  An FP64 sum is as accurate as the
+// terms it has: where the largest entries of the two meet small ones of the other (rows
+// that differ in scale), the sum of |terms| is far below that product and the digits of
+// the terms are lost.  So every result is held against a lower bound of its sum of
+// |terms|; one whose bound is below 2^-kFxLoss of the product of the scales is formed
+// again on the FP64 pipe from the operands in FP64.  At the line the error is 2^-51 of
+// the terms, what FP64 leaves of a sum of a hundred.  Row-wise error of the factorization
+// of 330 x 270 with the first 100 rows weighted by 2^13 and 2^33, in units of 2^-53: 7600
+// and 6e9 without this, 190 and 190 with it, 760 and 330 for the same panels in FP64
+// throughout (tests/test_gpu_row_scale.py).  Time: 8192 x 8192 60.0 -> 61.5 ms,
+// 16384 x 2048 20.6 -> 20.8, 1203 x 1001 3.68 -> 3.82, [L^T; C] of 4000 + 1000 17.1 -> 17.7.
+constexpr int kFxLoss = 5;
+
+// The exponent of a vector of zeros, whose digits are exact.
+constexpr int kFxZeroExp = -(1 << 20);
+
 // High word of |x| (sign cleared): ordered as |x|.
 __device__ __forceinline__ uint32_t fx_hi(double x) {
   return (uint32_t)__double2hiint(x) & 0x7fffffffu;
@@ -150,6 +167,17 @@ __device__ __forceinline__ long long fx_four(const uint32_t (&r)[kFxOrders][4], 
   v += (long long)__float2int_rn(__uint_as_float(r[o0][k])) * 16777216;
   return v;
 }
+
+// D += A B, 16 x 8 x 16, FP16 in, FP32 out
+__device__ __forceinline__ void fx_mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                            uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+               "{%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Magnitudes of two FP16 values
+__device__ __forceinline__ uint32_t fx_abs2(uint32_t v) { return v & 0x7fff7fffu; }
 
 // Unit exponent of the totals over slices of RS rows: 56 up to 512 rows, one
 // more for every factor of four.

@@ -163,15 +163,20 @@ int launch_vtx_tc(const float *A, int lda, const double *Vtop, int k0, int M, in
 //                stacked [L^T; C] with that many rows on top; upper: only the
 //                upper triangle of those is read, the rest is zero)
 //   fx_split_v   digit images of the panel's V
-//   fx_update    X -= V T^T V^T X (rows of the panel at k0, ldx, N columns);
+//   fx_update    X -= V T^T V^T X (rows of the panel at k0, ldx, N columns;
+//                the reflectors' tails in A);
 //                cmax: column maxima of X over those rows; cnext (or NULL)
 //                receives the maxima over the rows of the next panel.  False
 //                (nothing launched) when work_bytes is too small.  gram (or
-//                NULL): scratch of kFxGramBytes, zero before; the panel's G is
-//                formed from V's digits and written to wy_panel and Gt first.
+//                NULL): the panel's G is formed from V's digits and written to
+//                wy_panel and Gt first.
 //                Gt: kFxGt doubles, tau_j G[j, .] by rows and tau
 //   fx_gram      the same G and Gt alone, for a panel without such an update
 //   fx_prep      Gt of every panel of a compact-WY store (panels of nb)
+struct FxGramBuffers {
+  void *sums = nullptr;              // kFxGramBytes, zero before
+  double *part = nullptr;            // 2016 doubles to an SM
+};
 constexpr int kFxMinCols = 16;       // narrower updates stay on the FP64 pipe
 slqr_status init_fx_attrs(slqr_ctx *ctx);
 size_t fx_v_bytes(int m);
@@ -180,14 +185,15 @@ void fx_colmax(const double *X, int ldx, int m, int n, int stacked_top, bool upp
                int np, int num_sms, cudaStream_t stream);
 void fx_split_v(const double *A, int lda, const double *Vtop, int k0, int nbw, int M, int skip,
                 void *vbuf, cudaStream_t stream);
-bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy_panel,
-               const double *Gt, const void *vbuf, double *X, int ldx, int N, const unsigned *cmax,
-               unsigned *cnext, void *work, size_t work_bytes, cudaStream_t stream,
-               void *gram = nullptr);
+bool fx_update(slqr_ctx *ctx, const double *A, int lda, int k0, int nbw, int M, int skip,
+               const double *wy_panel, const double *Gt, const void *vbuf, double *X, int ldx, int N,
+               const unsigned *cmax, unsigned *cnext, void *work, size_t work_bytes, cudaStream_t stream,
+               const FxGramBuffers *gram = nullptr);
 constexpr size_t kFxGramBytes = 64 * 64 * 8 + 256;
 constexpr int kFxGt = 64 * 64 + 64;
-void fx_gram(slqr_ctx *ctx, int nbw, int M, double *wy_panel, const void *vbuf, void *gram,
-             double *Gt, cudaStream_t stream);
+void fx_gram(slqr_ctx *ctx, const double *A, int lda, int k0, int nbw, int M, int skip,
+             double *wy_panel, const void *vbuf, const FxGramBuffers &gram, double *Gt,
+             cudaStream_t stream);
 void fx_prep(const double *wy, int K, int nb, double *Gt, cudaStream_t stream);
 
 // B <- Q^T B for fewer than kFxMinCols right-hand sides in one launch for all

@@ -9,7 +9,10 @@
 //
 // e is the exponent of the vector's largest entry, so the rounding of x to
 // this grid is at most 2^(e-56): a quarter of the half-ulp that one FP64
-// operation on that entry commits.  The digits are exact in FP16.  A product
+// operation on that largest entry commits, but more than FP64's on entries far
+// below it.  Results whose terms are all far below the product of the scales are
+// formed again in FP64 (fx_digits.cuh has the rule, each kernel its bound).  The
+// digits are exact in FP16.  A product
 // of two digits is an integer of at most 2^14 in magnitude; the tensor core
 // sums them in FP32, which is exact while the sum stays below 2^24: at most
 // 7 pairs of digits of the same order i + j, over at most 128 terms.  The 34
@@ -19,7 +22,7 @@
 // The residual ||A - Q R|| / ||A|| in 128-bit arithmetic: 3.73e-16 with these
 // kernels, 4.92e-16 with the DFMA kernels of factor.cu (700 x 300 Gaussian),
 // 3.08e-16 against 3.38e-16 (3000 x 260), 2.96e-16 against 2.98e-16
-// (16384 x 260), 5.2e-16 against 9.2e-16 (rows graded over 10^16).
+// (16384 x 260).
 //
 // Why: the FP64 pipe of GB300 does 2 DFMA per SM and clock, 1.2 TFLOP/s, and
 // the products ran at 82-91% of that.  34 FP16 products cost 34/1834 of the
@@ -41,6 +44,7 @@
 
 #include <cuda_fp16.h>
 #include <algorithm>
+#include <climits>
 
 namespace slqr {
 
@@ -52,18 +56,173 @@ constexpr int kFxWTile = kFxD * 32 * 128;             // 28672 B: 32 columns
 constexpr int kFxXStage = kFxD * 128 * 64;            // 57344 B: 128 columns x 32 rows
 constexpr int kFxStage = kFxXStage + kFxV1Chunk;
 constexpr size_t kFxVtxSmem = 2 * (size_t)kFxStage + 1024;
-constexpr size_t kFxUpdSmem = (size_t)kFxV2Tile + 2 * kFxWTile + 1024;
 constexpr int kFxMaxPer = 32;                // column tiles of a CTA of the update
+constexpr int kFxLostWords = kFxWorkers * 8; // of a column tile: a warp's 8 columns, a bit a row
+constexpr size_t kFxUpdSmem =
+    (size_t)kFxV2Tile + 2 * kFxWTile + 1024 + kFxMaxPer * kFxLostWords * sizeof(unsigned);
 
 // D = F32, A = B = F16, both K-major, M = 128; N is added per MMA
 constexpr uint32_t kIdescF16 = (1u << 4) | ((128u >> 4) << 24);
 
 __device__ __forceinline__ uint32_t fx_idesc(int n) { return kIdescF16 | ((uint32_t)(n >> 3) << 17); }
 
+// The panel's V in FP64: rows < nbw in Vtop (ld 64, zero above the diagonal), the
+// others at tail[i + a ld]
+struct FxPanel {
+  const double *Vtop, *tail;
+  int ld, nbw, M, skip;                // skip > 0: [L^T; C], the top rows hold the pivots only
+};
+
+// out[k] = sum_i V(i, a0 + k) x_i for k < 8 on the FP64 pipe, by a warp (x: the column at
+// the panel's first row).  Bound by the pipe: a load of x and eight of V (coalesced) to
+// eight FMAs of 16 clocks each.
+static __device__ __noinline__ void fx_dots8(FxPanel p, const double *x, int a0, double *out) {
+  const int lane = threadIdx.x & 31, na = min(8, p.nbw - a0);
+  double acc[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k] = 0.0;
+  for (int i = lane; i < p.nbw; i += 32) {
+    const double xi = x[i];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < na) acc[k] = fma(p.Vtop[(a0 + k) * 64 + i], xi, acc[k]);
+  }
+  // (128 rows of x at a time: where they are zero, as in a banded or block matrix, V is
+  // not read)
+  const double *v = p.tail + (size_t)a0 * p.ld;
+  for (int i0 = p.nbw + lane; i0 - lane < p.M; i0 += 128) {
+    double xi[4];
+    bool any = false;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      xi[t] = i0 + 32 * t < p.M ? x[p.skip + i0 + 32 * t] : 0.0;
+      any |= (unsigned long long)__double_as_longlong(xi[t]) << 1 != 0;
+    }
+    if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int i = min(i0 + 32 * t, p.M - 1);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < na) acc[k] = fma(v[(size_t)k * p.ld + i], xi[t], acc[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if (lane == 0) out[k] = acc[k];
+  }
+  __syncwarp();
+}
+// the same for this thread's reflector a, of a panel of few rows
+constexpr int kFxFewRows = 192;
+static __device__ __noinline__ double fx_dot1(FxPanel p, const double *x, int a) {
+  double s = p.Vtop[a * 65] * x[a];
+  if (p.skip == 0) {
+#pragma unroll 4
+    for (int i = a + 1; i < p.nbw; ++i) s = fma(p.Vtop[a * 64 + i], x[i], s);
+  }
+  const double *v = p.tail + (size_t)a * p.ld;
+#pragma unroll 4
+  for (int i = p.nbw; i < p.M; ++i) s = fma(v[i], x[p.skip + i], s);
+  return s;
+}
+
+// sum_a V(i, a) W'(a, c) for four columns c .. c + 3 (w: W' of column c, nc of them) and
+// this thread's row
+struct FxFour { double v[4]; };
+static __device__ __noinline__ FxFour fx_row4(FxPanel p, const double *w, int nc, int i) {
+  FxFour s = {{0.0, 0.0, 0.0, 0.0}};
+  const double *v = i < p.nbw ? p.Vtop + i : p.tail + min(i, p.M - 1);
+  const size_t ld = i < p.nbw ? 64 : p.ld;
+#pragma unroll 4
+  for (int a = 0; a < p.nbw; ++a) {
+    const double t = v[a * ld];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s.v[k] = fma(t, w[min(k, nc - 1) * 64 + a], s.v[k]);
+  }
+  return s;
+}
+
+// The entries of X -= V W' that fx_upd_kernel's digits left out, by the warp (of its 32
+// rows, i this thread's) that found them: rows[t * kFxLostWords + k] for column c0 + 32 t + k.
+static __device__ __noinline__ void fx_lost_entries(FxPanel p, const double *Wf, double *X, int ldx,
+                                                    int N, int i, int c0, int T,
+                                                    const unsigned *rows, unsigned *cnext) {
+  const int lane = threadIdx.x & 31;
+  for (int b = 0; b < 2 * T; b += 32) {                  // a lane to a tile's four columns
+    const int mine = b + lane;
+    const uint4 m = mine < 2 * T
+                        ? *(const uint4 *)(rows + (mine >> 1) * kFxLostWords + (mine & 1) * 4)
+                        : make_uint4(0, 0, 0, 0);
+    unsigned todo = __ballot_sync(0xffffffffu, (m.x | m.y | m.z | m.w) != 0);
+    for (; todo; todo &= todo - 1) {
+      const int src = __ffs(todo) - 1, t = (b + src) >> 1, u = (b + src) & 1;
+      const int c = c0 + 32 * t + 4 * u;
+      unsigned w[4] = {m.x, m.y, m.z, m.w};
+      double *xp = X + i + (i >= p.nbw ? p.skip : 0) + (size_t)c * ldx;
+      int n = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        w[k] = __shfl_sync(0xffffffffu, w[k], src);
+        n += __popc(w[k]);
+      }
+      auto store = [&](int k, double s) {
+        const double v = xp[(size_t)k * ldx] - s;
+        xp[(size_t)k * ldx] = v;
+        if (cnext && i >= 64) atomicMax(cnext + c + k, fx_hi(v));
+      };
+      if (n > 16) {
+        const FxFour s = fx_row4(p, Wf + (size_t)c * 64, min(4, N - c), i);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (w[k] >> lane & 1) store(k, s.v[k]);
+      } else {
+        // four entries at a time, two reflectors a lane: one round trip of loads
+        for (; n > 0; n -= 4) {
+          int row[4], col[4];
+          double s[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            row[e] = -1;
+            col[e] = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (row[e] < 0 && w[k]) {
+                row[e] = __ffs(w[k]) - 1;
+                col[e] = k;
+                w[k] &= w[k] - 1;
+              }
+            const int r = i - lane + max(row[e], 0);
+            const double *v = r < p.nbw ? p.Vtop + r : p.tail + min(r, p.M - 1);
+            const size_t ld = r < p.nbw ? 64 : p.ld;
+            const double *wc = Wf + (size_t)min(c + col[e], N - 1) * 64;
+            s[e] = 0.0;
+            if (row[e] >= 0) {
+              if (lane < p.nbw) s[e] = v[lane * ld] * wc[lane];
+              if (lane + 32 < p.nbw) s[e] = fma(v[(lane + 32) * ld], wc[lane + 32], s[e]);
+            }
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[e] += __shfl_xor_sync(0xffffffffu, s[e], o);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (lane == row[e]) store(col[e], s[e]);
+        }
+      }
+    }
+  }
+}
+
 // The Gram terms of a panel beside (or, with no columns, instead of) V^T X
 struct FxGram {
   unsigned long long *sum;             // [c][a], zero before; NULL: none
   unsigned *arrived;                   // zero before
+  FxPanel p;
+  double *part;                        // [slice][c (c - 1) / 2 + a]: terms formed in FP64
   double *G;                           // the compact-WY store's G (tau follows it)
   double *Gt;                          // Gt and tau for the substitution (kFxGt doubles)
   int slices, RS;                      // CTAs, rows of each (a multiple of 128)
@@ -225,7 +384,7 @@ fx_vsplit_kernel(const double *__restrict__ A, int lda, const double *__restrict
     }
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-    const int e = (key == kFxZero) ? 0 : fx_exp(key);
+    const int e = (key == kFxZero) ? kFxZeroExp : fx_exp(key);
     unsigned long long y[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -261,16 +420,27 @@ __device__ __forceinline__ bool fx_wait(uint64_t *bar, int phase) {
 // digits the N side.  With V's wide leading digits the sums are still exact: by
 // Cauchy-Schwarz a product with them is at most (sqrt(2) 1024)^2 over all rows.
 // G is known to 2^-58 of |up_a up_c|; the panel's own sums in FP64 cost it 0.5
-// us of each column step.
+// us of each column step.  That is below FP64's own error in a sum of products unless
+// their magnitudes add up to far less (columns whose large entries are in different
+// rows).  Every CTA forms the sums of |products| over the panel's first kFxGramSample
+// rows from the leading digits (mma.sync), a lower bound; the terms whose bound is below
+// 2^-7 |up_a up_c| (for M > 512 rows 512 / M of it, as of the sum of all) are formed in
+// FP64, each CTA's rows by itself, and added by the last one.  Without structure the
+// sample holds 0.16 to 0.64 of 256 / M.
 // Called by every thread of CTAs (gridDim.x - 1, y), y < slices.
 // --------------------------------------------------------------------------
+constexpr int kFxGramSample = 256;
+// the line in products of leading digits: with the sample's share of M rows
+__device__ __forceinline__ float fx_gram_line(int M) {
+  return (float)(1 << (20 - 7)) * 512.f / (float)max(M, 512);
+}
 constexpr int kFxGramChunk = kFxV1Chunk + 4096;       // (a zero digit 7 behind each chunk)
 constexpr int kFxGramShift = 56;                      // units of 2^56 digit products
 
 __device__ __noinline__ void fx_gram_block(const FxGram &gr, int nbw, int M,
                                            const unsigned char *V1, unsigned char *base,
                                            uint32_t taddr, uint64_t *s_full, uint64_t *s_acc,
-                                           const int *s_fa, int *status) {
+                                           uint64_t *s_sample, const int *s_fa, int *status) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int i_begin = blockIdx.y * gr.RS, i_end = min(M, i_begin + gr.RS);
   const int B = (i_end - i_begin + 127) / 128;
@@ -278,6 +448,21 @@ __device__ __noinline__ void fx_gram_block(const FxGram &gr, int nbw, int M,
     *(uint4 *)(base + (idx >> 8) * kFxGramChunk + kFxV1Chunk + (idx & 255) * 16) =
         make_uint4(0, 0, 0, 0);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __shared__ unsigned s_low[64][2], s_any;              // terms to be formed in FP64, by column
+  unsigned char *sample = base + 4 * kFxGramChunk;
+  const int chunks = min(kFxGramSample / 32, (M + 127) / 128 * 4);
+  if (tid < 128) s_low[tid >> 1][tid & 1] = 0;
+  if (tid == 128) s_any = 0;
+  if (tid == 0) {
+    const uint32_t bar = smem_u32(s_sample);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                 ::"r"(bar), "r"(chunks * 4096) : "memory");
+    for (int u = 0; u < chunks; ++u)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes"
+                   " [%0], [%1], %2, [%3];"
+                   ::"r"(smem_u32(sample + u * 4096)), "l"(V1 + (size_t)u * kFxV1Chunk), "r"(4096),
+                   "r"(bar) : "memory");
+  }
   __syncthreads();
   const int q = warp & 3, h = warp >> 2;               // workers: TMEM lanes, 16 columns
   const int a = (q * 32 + lane) & 63;
@@ -318,7 +503,35 @@ __device__ __noinline__ void fx_gram_block(const FxGram &gr, int nbw, int M,
       }
     }
     __syncwarp();
-    ok = fx_wait(s_acc, b);
+    if (b == 0) ok = fx_wait(s_sample, 0);
+    if (b == 0 && ok && warp < kFxWorkers) {
+      // beside the first MMAs: 16 x 16 of the 64 x 64 sums to a warp (at most 2^21 by
+      // Cauchy-Schwarz, so exact)
+      const int gid = lane >> 2, tq = lane & 3, ar = q * 16 + gid, cr = h * 16 + gid;
+      const float line = fx_gram_line(M);
+      float mag[2][4] = {};
+      for (int u = 0; u < chunks; ++u) {
+        auto pair = [&](int row, int grp) {
+          return fx_abs2(*(const uint32_t *)(sample + u * 4096 + row * 64 +
+                                             ((grp * 16) ^ (((row >> 1) & 3) << 4)) + tq * 4));
+        };
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          const uint32_t fa[4] = {pair(ar, 2 * ks), pair(ar + 8, 2 * ks), pair(ar, 2 * ks + 1),
+                                  pair(ar + 8, 2 * ks + 1)};
+#pragma unroll
+          for (int t = 0; t < 2; ++t)
+            fx_mma16816(mag[t], fa, pair(cr + 8 * t, 2 * ks), pair(cr + 8 * t, 2 * ks + 1));
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int r = q * 16 + gid + 8 * ((k >> 1) & 1), c = h * 16 + 8 * (k >> 2) + 2 * tq + (k & 1);
+        if (r < c && c < nbw && mag[k >> 2][k & 3] < line)
+          atomicOr(&s_low[c][r >> 5], 1u << (r & 31)), s_any = 1;
+      }
+    }
+    ok = fx_wait(s_acc, b) && ok;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok && warp < kFxWorkers) {
 #pragma unroll
@@ -340,15 +553,55 @@ __device__ __noinline__ void fx_gram_block(const FxGram &gr, int nbw, int M,
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
   if (!ok && tid == 0) {
-    mbar_wait(smem_u32(s_full), (uint32_t)((B - 1) & 1));   // let the copies in flight land
+    mbar_wait(smem_u32(s_sample), 0);                       // let the copies in flight land
+    mbar_wait(smem_u32(s_full), (uint32_t)((B - 1) & 1));
     atomicCAS(status, 0, SLQR_ETIMEOUT);
   }
+  // (s_low is complete: a barrier ended each block)
   if (warp < kFxWorkers) {
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const int c = h * 16 + k;
-      if (a < c) atomicAdd(gr.sum + c * 64 + a, (unsigned long long)tot[k]);
+      if (a < c && !(s_low[c][a >> 5] >> (a & 31) & 1))
+        atomicAdd(gr.sum + c * 64 + a, (unsigned long long)tot[k]);
     }
+  }
+  if (s_any) {
+    // this CTA's rows of those terms in FP64: 64 rows at a time through shared memory (the
+    // chunks are used up), a thread for column c and the a = a8, a8 + 8, ..
+    double *vs = (double *)base;                        // [64][65]
+    const int c = tid >> 3, a8 = tid & 7;
+    double g[8];
+    unsigned mine = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      g[k] = 0.0;
+      if (warp < kFxWorkers) mine |= (s_low[c][k >> 2] >> (a8 + 8 * (k & 3)) & 1) << k;
+    }
+    // ([L^T; C]: no two reflectors meet in the top rows)
+    for (int i0 = gr.p.skip > 0 ? max(i_begin, nbw) : i_begin; i0 < i_end; i0 += 64) {
+      const int rows = min(64, i_end - i0);
+      __syncthreads();
+      for (int idx = tid; idx < 64 * 64; idx += kFxThreads) {
+        const int r = idx & 63, aa = idx >> 6, i = i0 + r;
+        double v = 0.0;
+        if (r < rows && aa < nbw)
+          v = i < nbw ? gr.p.Vtop[aa * 64 + i] : gr.p.tail[(size_t)aa * gr.p.ld + i];
+        vs[r * 65 + aa] = v;
+      }
+      __syncthreads();
+      if (mine)
+        for (int r = 0; r < rows; ++r) {
+          const double x = vs[r * 65 + c];
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (mine >> k & 1) g[k] = fma(vs[r * 65 + a8 + 8 * k], x, g[k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (mine >> k & 1)
+        gr.part[(size_t)blockIdx.y * 2016 + c * (c - 1) / 2 + a8 + 8 * k] = g[k];
   }
   __threadfence();
   __syncthreads();
@@ -366,6 +619,9 @@ __device__ __noinline__ void fx_gram_block(const FxGram &gr, int nbw, int M,
       g = (fa == kFxNonFinite || fc == kFxNonFinite)
               ? __longlong_as_double(0x7ff8000000000000ll)
               : fx_scale((double)t, fa + fc - 110 + kFxGramShift);
+      if (s_low[c][aa >> 5] >> (aa & 31) & 1)            // (a NaN stays one)
+        for (int s = 0; s < gr.slices; ++s)
+          g += __ldcg(gr.part + (size_t)s * 2016 + c * (c - 1) / 2 + aa);
     }
     gr.G[idx] = g;
     const double tau = gr.G[64 * 64 + aa];               // (of the panel's own kernel)
@@ -429,7 +685,7 @@ fx_vtx_kernel(const double *__restrict__ X, int ldx, int k0, int nbw, int skip, 
   const uint32_t taddr = s_taddr;
 
   if (gram) {
-    fx_gram_block(gr, nbw, M, V1, base, taddr, &s_full[0], &s_acc, s_fa, status);
+    fx_gram_block(gr, nbw, M, V1, base, taddr, &s_full[0], &s_acc, &s_empty[0], s_fa, status);
   } else if (warp == kFxWorkers) {                      // ---- the MMAs --------------------
     if (lane == 0) {
       bool ok = true;
@@ -618,15 +874,24 @@ fx_prep_kernel(const double *__restrict__ wy, int K, int nb, double *__restrict_
 // and one FMA per 32 rows still to come.  One warp holds CPW columns (two rows
 // a lane each).  Bound by the FP64 pipe: 96 FMAs a column and the sum of its
 // partials.
+// A W entry whose partials' magnitudes add up to less than 2^-kFxLoss |up_a| max |x_c|, as
+// does its term of row a, may have lost its digits and is formed again from V and X (the
+// columns at the panel's first row).  Without structure that is about 1% of the entries of
+// panels of at most 128 rows, which have one partial, and next to none of others.
+// W' in FP64 replaces the first partial, for the entries of X -= V W' formed again.
 // --------------------------------------------------------------------------
 template <int CPW>
-__global__ void __launch_bounds__(256)
-fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restrict__ wy,
-             const double *__restrict__ Gt, int nbw, unsigned char *__restrict__ Wimg,
-             int *__restrict__ ecol) {
+__global__ void __launch_bounds__(256, 4)
+fx_tw_kernel(double *__restrict__ Wp, int S, int N, FxPanel p, const double *__restrict__ X, int ldx,
+             const unsigned *__restrict__ cmax, const double *__restrict__ Gt,
+             unsigned char *__restrict__ Wimg, int *__restrict__ ecol) {
   constexpr int NB = 64, WARPS = CPW == 1 ? 1 : 8;   // (CPW 1: all threads sum one column)
   __shared__ double G[NB * NB];
-  __shared__ double part[4][NB];
+  __shared__ double part[CPW == 1 ? 4 : 8][NB];
+  __shared__ float psum[4][NB];
+  __shared__ unsigned long long s_low;
+  const double *wy = p.Vtop;
+  const int nbw = p.nbw;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c0 = (blockIdx.x * WARPS + (CPW == 1 ? 0 : warp)) * CPW;
   {
@@ -640,43 +905,114 @@ fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restri
   const double u0 = wy[lane * 65], u1 = wy[(lane + 32) * 65];     // up
   const size_t stride = (size_t)N * NB;
   double r0[CPW], r1[CPW];
+  // A partial's magnitude over 2^(exponents of up_a and max |x_c|), by its bits (o: the
+  // exponents to take off, in the high word); o of reflector and column.
+  auto part_of = [](double v, int o) {
+    return __int_as_float(min(max((int)fx_hi(v) - o, 0), 254 << 20) << 3);
+  };
+  auto off = [](double u, unsigned cm) {
+    return min((int)(fx_hi(u) >> 20) + (int)(cm >> 20) - 1023 - 127, 2000) * (1 << 20);
+  };
+  // whether reflector a's entry, whose partials' magnitudes add up to `sum`, is below the
+  // line, and so is the one term up_a x_a
+  auto low = [&](int c, int a, float sum, double u) {
+    const unsigned cm = cmax[c];
+    if (fx_hi(u) == 0 || cm == 0 || cm >= 0x7ff00000u || sum >= 1.f / (1 << kFxLoss)) return false;
+    return (int)(fx_hi(X[(size_t)c * ldx + a]) >> 20) < (int)(cm >> 20) - kFxLoss;
+  };
+  auto dots = [&](int c, int a0, double *out) { fx_dots8(p, X + (size_t)c * ldx, a0, out); };
+  // of few rows every lane forms its own (V of [L^T; C] has its pivots and C's rows)
+  auto few = [&](int c, bool low0, bool low1, double &r0, double &r1) {
+    if (low0) r0 = fx_dot1(p, X + (size_t)c * ldx, lane);
+    if (low1) r1 = fx_dot1(p, X + (size_t)c * ldx, lane + 32);
+  };
   if constexpr (CPW == 1) {
     const double *src = Wp + (size_t)c0 * NB + (tid & 63);
     double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+    float mg = 0.f;
+    const int o = off(wy[(tid & 63) * 65], cmax[c0]);
+    auto take = [&](double &a, int s) {
+      const double v = src[s * stride];
+      mg += part_of(v, o);
+      a += v;
+    };
     int s = tid >> 6;
     for (; s + 12 < S; s += 16) {
-      a0 += src[s * stride];
-      a1 += src[(s + 4) * stride];
-      a2 += src[(s + 8) * stride];
-      a3 += src[(s + 12) * stride];
+      take(a0, s);
+      take(a1, s + 4);
+      take(a2, s + 8);
+      take(a3, s + 12);
     }
-    for (; s < S; s += 4) a0 += src[s * stride];
+    for (; s < S; s += 4) take(a0, s);
     part[tid >> 6][tid & 63] = (a0 + a1) + (a2 + a3);
+    psum[tid >> 6][tid & 63] = mg;
+    __syncthreads();
+    bool low0 = false, low1 = false;
+    if (warp == 0) {
+      r0[0] = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
+      r1[0] = (part[0][lane + 32] + part[1][lane + 32]) + (part[2][lane + 32] + part[3][lane + 32]);
+      auto ps = [&](int a) { return psum[0][a] + psum[1][a] + psum[2][a] + psum[3][a]; };
+      low0 = low(c0, lane, ps(lane), u0);
+      low1 = low(c0, lane + 32, ps(lane + 32), u1);
+      if (p.M <= kFxFewRows) {
+        few(c0, low0, low1, r0[0], r1[0]);
+        low0 = low1 = false;
+      }
+      const unsigned l0 = __ballot_sync(0xffffffffu, low0), l1 = __ballot_sync(0xffffffffu, low1);
+      if (lane == 0) s_low = (unsigned long long)l1 << 32 | l0;
+    }
+    __syncthreads();
+    if (s_low != 0) {                                  // (uniform)
+      if ((s_low >> (8 * warp)) & 0xff) dots(c0, 8 * warp, part[0] + 8 * warp);
+      __syncthreads();
+      if (low0) r0[0] = part[0][lane];
+      if (low1) r1[0] = part[0][lane + 32];
+    }
+    if (warp > 0) return;
   } else {
+    float m0[CPW], m1[CPW];                            // sums of the partials' magnitudes
 #pragma unroll
     for (int k = 0; k < CPW; ++k) {
       const double *src = Wp + (size_t)min(c0 + k, N - 1) * NB + lane;
       double a0 = 0, a1 = 0, b0 = 0, b1 = 0;
+      m0[k] = m1[k] = 0.f;
+      const unsigned cm = cmax[min(c0 + k, N - 1)];
+      const int o0 = off(u0, cm), o1 = off(u1, cm);
+      auto take = [&](double &a, double &b, int s) {
+        const double v0 = src[s * stride], v1 = src[s * stride + 32];
+        m0[k] += part_of(v0, o0);
+        m1[k] += part_of(v1, o1);
+        a += v0;
+        b += v1;
+      };
       int s = 0;
       for (; s + 1 < S; s += 2) {
-        a0 += src[s * stride];
-        b0 += src[s * stride + 32];
-        a1 += src[(s + 1) * stride];
-        b1 += src[(s + 1) * stride + 32];
+        take(a0, b0, s);
+        take(a1, b1, s + 1);
       }
-      if (s < S) {
-        a0 += src[s * stride];
-        b0 += src[s * stride + 32];
-      }
+      if (s < S) take(a0, b0, s);
       r0[k] = a0 + a1;
       r1[k] = b0 + b1;
     }
-  }
-  __syncthreads();
-  if (warp >= WARPS || c0 >= N) return;
-  if constexpr (CPW == 1) {
-    r0[0] = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
-    r1[0] = (part[0][lane + 32] + part[1][lane + 32]) + (part[2][lane + 32] + part[3][lane + 32]);
+    __syncthreads();
+    if (c0 >= N) return;
+#pragma unroll
+    for (int k = 0; k < CPW; ++k) {
+      if (c0 + k >= N) break;
+      const bool low0 = low(c0 + k, lane, m0[k], u0), low1 = low(c0 + k, lane + 32, m1[k], u1);
+      if (p.M <= kFxFewRows) {
+        few(c0 + k, low0, low1, r0[k], r1[k]);
+        __syncwarp();
+        continue;
+      }
+      const unsigned l0 = __ballot_sync(0xffffffffu, low0), l1 = __ballot_sync(0xffffffffu, low1);
+      if ((l0 | l1) == 0) continue;
+      for (int g = 0; g < 8; ++g)
+        if (((g < 4 ? l0 : l1) >> (8 * (g & 3))) & 0xff) dots(c0 + k, 8 * g, part[warp] + 8 * g);
+      if (low0) r0[k] = part[warp][lane];
+      if (low1) r1[k] = part[warp][lane + 32];
+      __syncwarp();
+    }
   }
   // (on and below the diagonal Gt is zero, but a product with an entry that is
   // not finite would not be)
@@ -708,7 +1044,9 @@ fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restri
     key = __reduce_max_sync(0xffffffffu, key);
     const bool bad =
         __any_sync(0xffffffffu, fx_hi(w0) >= 0x7ff00000u || fx_hi(w1) >= 0x7ff00000u);
-    const int g = (key == kFxZero) ? 0 : fx_exp(key);
+    const int g = (key == kFxZero) ? kFxZeroExp : fx_exp(key);
+    Wp[(size_t)c * NB + lane] = w0;
+    Wp[(size_t)c * NB + lane + 32] = w1;
     unsigned char *dst = Wimg + (size_t)(c >> 5) * kFxWTile + (c & 31) * 128;
     const unsigned long long y0 = fx_digits(w0, g - f0), y1 = fx_digits(w1, g - f1);
     const int sw = (c & 7) << 4;
@@ -732,13 +1070,19 @@ fx_tw_kernel(const double *__restrict__ Wp, int S, int N, const double *__restri
 // one.  A thread owns one row and 8 columns of a tile: TMEM lane = row, so X is
 // read and written in 256-byte runs.  The new values' column maxima (rows >= 64,
 // those of the next panel) go to cnext.
+// An entry is below the line where it and its change are less than 2^-kFxLoss of the
+// row's scale times the column's.  By chance that is one entry in 100 of the top rows and
+// one in 10^4 of the others (one in 8 of the top rows of [L^T; C]); where rows and columns
+// hold their large values in different reflectors it is most entries of a row or of a
+// column.  So three of the thread's four columns, or 3/8 of the warp's rows, count as
+// lost: those entries are left and formed again from V and W' in FP64 (fx_lost_entries).
 // grid: (ceil(M / 128), groups of `per` tiles)
 // --------------------------------------------------------------------------
 __global__ void __launch_bounds__(kFxThreads, 1)
 fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M, int N, int per,
               const unsigned char *__restrict__ V2, const int *__restrict__ erow,
-              const unsigned char *__restrict__ Wimg, const int *__restrict__ ecol,
-              unsigned *__restrict__ cnext, int *status) {
+              const unsigned char *__restrict__ Wimg, const int *__restrict__ ecol, FxPanel p,
+              const double *__restrict__ Wf, unsigned *__restrict__ cnext, int *status) {
   extern __shared__ __align__(1024) unsigned char fx_smem_raw[];
   unsigned char *base = (unsigned char *)(((uintptr_t)fx_smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char *Ws = base + kFxV2Tile;
@@ -752,7 +1096,10 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
   const int i0 = blockIdx.x * 128;
 
   for (int idx = tid; idx < 32 * T; idx += kFxThreads)
-    s_ecol[idx] = t_begin * 32 + idx < N ? ecol[t_begin * 32 + idx] : 0;
+    s_ecol[idx] = t_begin * 32 + idx < N ? ecol[t_begin * 32 + idx] : kFxZeroExp;
+  // entries to be formed again: [column tile][warp][column of 8], a bit a row
+  unsigned *lost_rows = (unsigned *)(Ws + 2 * kFxWTile);
+  for (int idx = tid; idx < T * kFxLostWords; idx += kFxThreads) lost_rows[idx] = 0;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
                  :: "r"(smem_u32(&s_taddr)));
@@ -824,7 +1171,15 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
     const int q = warp & 3, h = warp >> 2;
     const int i = i0 + q * 32 + lane;
     const bool row_ok = i < M;
-    const int er = erow[i] - 56;                         // (defined up to the whole tile)
+    const int ei = erow[i];                              // (defined up to the whole tile)
+    const int er = (ei == kFxZeroExp ? 0 : ei) - 56;
+    // the line: the scales' product is 2^(sh + 56) or up to two binades less
+    const bool live = row_ok && ei != kFxZeroExp;
+    const unsigned line = live ? 1u << (23 - kFxLoss) : 0u, line2 = 2 * line;
+    const unsigned xline = (unsigned)(er + 1078 - kFxLoss) << 21;
+    // (3 of 8 of the rows)
+    const int lost_rows_min = 3 * __popc(__ballot_sync(0xffffffffu, live));
+    unsigned *lost_mine = lost_rows + warp * 8;
     double *xrow = X + k0 + i + (i >= nbw ? skip : 0) + (size_t)(t_begin * 32 + h * 8) * ldx;
     const bool next_row = row_ok && i >= 64;
     int c = t_begin * 32 + h * 8;
@@ -860,6 +1215,8 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           if (lane == 0) fx_arrive(&s_free[buf]);
         }
+        long long tt[4];
+        unsigned low = 0;                                // (of these four: below the line)
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           const int k = u * 4 + kk;
@@ -867,18 +1224,49 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
           // (the leading order sums 64 products).  Orders 0..3 are at most 2^22,
           // 4 and 5 above; of 6 and 7 half a unit is lost, 2^-62 of the bound.
           auto f = [&](int o) { return __uint_as_float(r[o][kk]); };
-          const long long tt =
+          tt[kk] =
               fx_join(fx_small(f(0)) * 256 + fx_small(f(1)), fx_small(f(2)) * 256 + fx_small(f(3)),
                       __float2int_rn(f(4)) * 256 + __float2int_rn(f(5)),
                       (fx_small_half(f(6)) * 256 + fx_small_half(f(7))) * 2, 20);
+          if ((unsigned)((int)(tt[kk] >> 32) + (int)line) < line2 &&
+              (unsigned)__double2hiint(x[k]) * 2u < xline + (unsigned)g[k] * (1u << 21))
+            low |= 1u << kk;
+        }
+        if (__any_sync(0xffffffffu, low != 0)) {
+          // (the quick test's exponents wrap, and it takes in columns of zeros, columns that
+          // are not finite and the ones past the last)
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const int gk = g[u * 4 + kk];
+            if (gk == kFxZeroExp || gk == kFxNonFinite ||
+                (int)(fx_hi(x[u * 4 + kk]) >> 20) >= er + gk + 1078 - kFxLoss)
+              low &= ~(1u << kk);
+          }
+          unsigned lost = __popc(low) >= min(3, N - cw - u * 4) ? low : 0u;
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const unsigned in_col = __ballot_sync(0xffffffffu, low >> kk & 1);
+            if (8 * __popc(in_col) >= lost_rows_min) lost |= low & (1u << kk);
+            const unsigned rows = __ballot_sync(0xffffffffu, lost >> kk & 1);
+            if (lane == kk && rows) lost_mine[t * kFxLostWords + u * 4 + kk] = rows;
+            if (lost >> kk & 1) tt[kk] = 0;
+          }
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const int k = u * 4 + kk;
           const int gk = g[k], sh = er + gk;
           // (uniform: exponents out of the quick form's range are rare)
           if (__all_sync(0xffffffffu, sh >= -1000 && sh <= 900))
-            x[k] -= fx_to_double(tt, sh);
+            x[k] -= fx_to_double(tt[kk], sh);
           else if (gk == kFxNonFinite)
             x[k] = __longlong_as_double(0x7ff8000000000000ll);
-          else
-            x[k] -= fx_scale_slow((double)tt, sh);
+          else if (gk != kFxZeroExp)
+            x[k] -= fx_scale_slow((double)tt[kk], sh);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const int k = u * 4 + kk;
           if (row_ok && cw + k < N) xw[(size_t)k * ldx] = x[k];
           const unsigned mx = __reduce_max_sync(0xffffffffu, next_row ? fx_hi(x[k]) : 0u);
           if (lane == k) mine = mx;
@@ -886,6 +1274,9 @@ fx_upd_kernel(double *__restrict__ X, int ldx, int k0, int nbw, int skip, int M,
       }
       if (cnext && lane < 8 && cw + lane < N && mine) atomicMax(cnext + cw + lane, mine);
     }
+    __syncwarp();
+    fx_lost_entries(p, Wf, X + k0, ldx, N, i, t_begin * 32 + h * 8, T, lost_mine,
+                    cnext);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -941,22 +1332,32 @@ void fx_split_v(const double *A, int lda, const double *Vtop, int k0, int nbw, i
                                                               V2, erow);
 }
 
-static FxGram fx_gram_args(double *wy_panel, void *gram, double *Gt, int M, int ctas) {
+static FxPanel fx_panel(const double *A, int lda, const double *Vtop, int k0, int nbw, int M,
+                        int skip) {
+  return FxPanel{Vtop, A + (size_t)k0 * lda + k0 + skip, lda, nbw, M, skip};
+}
+
+static FxGram fx_gram_args(double *wy_panel, const FxGramBuffers &b, double *Gt, const FxPanel &p,
+                           int ctas) {
   FxGram gr;
-  gr.sum = (unsigned long long *)gram;
+  gr.sum = (unsigned long long *)b.sums;
   gr.arrived = (unsigned *)(gr.sum + 64 * 64);
+  gr.p = p;
+  gr.part = b.part;
   gr.G = wy_panel + 64 * 64;
   gr.Gt = Gt;
-  const int blocks = (M + 127) / 128;
+  const int blocks = (p.M + 127) / 128;
   gr.RS = (blocks + ctas - 1) / ctas * 128;
-  gr.slices = (M + gr.RS - 1) / gr.RS;
+  gr.slices = (p.M + gr.RS - 1) / gr.RS;
   gr.vtx_slices = 0;
   return gr;
 }
 
-void fx_gram(slqr_ctx *ctx, int nbw, int M, double *wy_panel, const void *vbuf, void *gram,
-             double *Gt, cudaStream_t stream) {
-  const FxGram gr = fx_gram_args(wy_panel, gram, Gt, M, ctx->num_sms);
+void fx_gram(slqr_ctx *ctx, const double *A, int lda, int k0, int nbw, int M, int skip,
+             double *wy_panel, const void *vbuf, const FxGramBuffers &gram, double *Gt,
+             cudaStream_t stream) {
+  const FxGram gr = fx_gram_args(wy_panel, gram, Gt, fx_panel(A, lda, wy_panel, k0, nbw, M, skip),
+                                 ctx->num_sms);
   int slot = prof_begin(ctx, stream);
   fx_vtx_kernel<<<dim3(1, gr.slices), kFxThreads, kFxVtxSmem, stream>>>(
       nullptr, 0, 0, nbw, 0, M, 0, 128, (const unsigned char *)vbuf, wy_panel, nullptr, nullptr, gr,
@@ -968,9 +1369,10 @@ void fx_prep(const double *wy, int K, int nb, double *Gt, cudaStream_t stream) {
   fx_prep_kernel<<<num_panels(K, nb), 256, 0, stream>>>(wy, K, nb, Gt);
 }
 
-bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy_panel,
-               const double *Gt, const void *vbuf, double *X, int ldx, int N, const unsigned *cmax,
-               unsigned *cnext, void *work, size_t work_bytes, cudaStream_t stream, void *gram) {
+bool fx_update(slqr_ctx *ctx, const double *A, int lda, int k0, int nbw, int M, int skip,
+               const double *wy_panel, const double *Gt, const void *vbuf, double *X, int ldx, int N, const unsigned *cmax,
+               unsigned *cnext, void *work, size_t work_bytes, cudaStream_t stream,
+               const FxGramBuffers *gram) {
   int RS = 0;
   const int S = fx_slices(M, N, ctx->num_sms, &RS);
   const size_t tiles = ((size_t)M + 127) / 128, wt = ((size_t)N + 31) / 32;
@@ -985,7 +1387,8 @@ bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy
   int slot = prof_begin(ctx, stream);
   // the panel's Gram terms beside it, on the SMs the products leave (a quarter at least)
   const int vt = (N + 127) / 128;
-  FxGram gr = fx_gram_args((double *)wy_panel, gram, (double *)Gt, M,
+  const FxPanel p = fx_panel(A, lda, wy_panel, k0, nbw, M, skip);
+  FxGram gr = fx_gram_args((double *)wy_panel, gram ? *gram : FxGramBuffers{}, (double *)Gt, p,
                            std::max(ctx->num_sms / 4, ctx->num_sms - vt * S));
   gr.vtx_slices = S;
   fx_vtx_kernel<<<dim3(vt + (gram ? 1 : 0), std::max(S, gram ? gr.slices : 0)), kFxThreads,
@@ -994,9 +1397,10 @@ bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy
   prof_end(ctx, stream, slot, kVtx, flops);
   slot = prof_begin(ctx, stream);
   if (N <= 4 * ctx->num_sms)
-    fx_tw_kernel<1><<<N, 256, 0, stream>>>(Wp, S, N, wy_panel, Gt, nbw, Wimg, ecol);
+    fx_tw_kernel<1><<<N, 256, 0, stream>>>(Wp, S, N, p, X + k0, ldx, cmax, Gt, Wimg, ecol);
   else
-    fx_tw_kernel<2><<<(N + 15) / 16, 256, 0, stream>>>(Wp, S, N, wy_panel, Gt, nbw, Wimg, ecol);
+    fx_tw_kernel<2><<<(N + 15) / 16, 256, 0, stream>>>(Wp, S, N, p, X + k0, ldx, cmax, Gt, Wimg,
+                                                       ecol);
   prof_end(ctx, stream, slot, kTw, (double)nbw * nbw * N);
   slot = prof_begin(ctx, stream);
   const int rt = (M + 127) / 128;
@@ -1006,7 +1410,7 @@ bool fx_update(slqr_ctx *ctx, int k0, int nbw, int M, int skip, const double *wy
   const int per = std::min(
       kFxMaxPer, std::max(rt * (int)wt <= ctx->num_sms ? 1 : 4, ((int)wt + groups - 1) / groups));
   fx_upd_kernel<<<dim3(rt, ((int)wt + per - 1) / per), kFxThreads, kFxUpdSmem, stream>>>(
-      X, ldx, k0, nbw, skip, M, N, per, V2, erow, Wimg, ecol, cnext, ctx->d_status);
+      X, ldx, k0, nbw, skip, M, N, per, V2, erow, Wimg, ecol, p, Wp, cnext, ctx->d_status);
   prof_end(ctx, stream, slot, kUpd, flops);
   return true;
 }
