@@ -342,7 +342,7 @@ slqr_status slqr_apply_qt_stacked(slqr_ctx *ctx, int n, int m_eq, const double *
  * The host arrays are read before the call returns.  The problems must not
  * overlap in memory.  Errors: SLQR_EINVAL, SLQR_ENOMEM, SLQR_ECUDA.
  */
-#define SLQR_FP64 0   /* FP64 accuracy throughout                                 */
+#define SLQR_FP64 0   /* FP64 accuracy throughout, row by row as well             */
 #define SLQR_FP32 1   /* FP32 factorization + FP64-residual refinement            */
 #define SLQR_TF32 2   /* as SLQR_FP32, the two products of the rank-NB trailing
                          update (W = V^T X and X -= V W') on the tensor cores

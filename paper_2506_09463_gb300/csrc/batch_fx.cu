@@ -30,6 +30,10 @@ namespace slqr {
 namespace {
 
 constexpr int kBfNB = 16;
+// The line below which digits count as lost (fx_digits.cuh), two binades lower than in
+// tc_fp64.cu: the sums of |products| hold every term here, and V is not scaled by rows
+// again for C -= V W', whose entries are known to 2^-56 of the column's scale.
+constexpr int kBfLoss = 7;
 
 template <int NW>
 struct BfSmem {
@@ -45,13 +49,6 @@ struct BfSmem {
 
 __device__ __forceinline__ uint32_t bf_smem(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void bf_mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
-                                       uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-               "{%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 // A 16-byte chunk (8 columns) of V's digit row r: the two chunks of rows 4..7 of
 // eight swap places, so that eight rows of one chunk meet all banks once.
@@ -85,6 +82,47 @@ __device__ __forceinline__ uint32_t bf_pair(unsigned long long y0, unsigned long
   const uint32_t w1 = byte < 4 ? (uint32_t)y1 : (uint32_t)(y1 >> 32);
   return fx_half2(w0, w1, byte & 3);
 }
+// The panel's V in FP64: reflector a's pivot entry on row a, its tail below (stacked: from
+// row nbw on)
+struct BfPanel {
+  const double *A, *up;                              // A at row k0 of column k0
+  int lda, nbw, skip, M;
+  bool stacked;
+};
+__device__ __forceinline__ int bf_row(const BfPanel &p, int r) { return r + (r >= p.nbw ? p.skip : 0); }
+__device__ __forceinline__ double bf_v(const BfPanel &p, int r, int a) {
+  if (r == a) return p.up[a];
+  return r < a || (p.stacked && r < p.nbw) ? 0.0 : p.A[(size_t)a * p.lda + bf_row(p, r)];
+}
+// out[k] = sum_r V(r, a0 + k) x_r for k < 8 on the FP64 pipe, by a warp; x: a column (at row
+// k0), or V's own column c where c >= 0
+__device__ __noinline__ void bf_dots8(BfPanel p, const double *x, int c, int a0, double *out) {
+  const int lane = threadIdx.x & 31;
+  double acc[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k] = 0.0;
+  for (int r = lane; r < p.M; r += 32) {
+    const double xr = c >= 0 ? bf_v(p, r, c) : x[bf_row(p, r)];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (a0 + k < p.nbw) acc[k] = fma(bf_v(p, r, a0 + k), xr, acc[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if (lane == 0) out[k] = acc[k];
+  }
+  __syncwarp();
+}
+// sum_a V(r, a) W'(a) for this thread's row and column (W'(a) at w[a * ldw])
+__device__ __noinline__ double bf_entry(BfPanel p, const double *w, int ldw, int r) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int a = 0; a < p.nbw; ++a) s = fma(bf_v(p, r, a), w[a * ldw], s);
+  return s;
+}
+
 __device__ __forceinline__ double bf_value(long long t, int sh) {
   if (sh >= -1000 && sh <= 900) return fx_to_double(t, sh);
   return fx_scale_slow((double)t, sh);
@@ -107,6 +145,7 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
   __shared__ double s_G[16 * 16], s_tau[16], s_up[16];
   __shared__ __align__(16) unsigned s_mx[16][RQ];   // maxima of the panel's columns below the diagonal
   __shared__ int s_f[16], s_def, s_ecol[SM::CT];
+  __shared__ double s_dot[NW][8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gid = lane >> 2, tq = lane & 3;         // fragment row and column pair
   const int K = num_reflectors(m, n);
@@ -297,7 +336,7 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
         const bool q_ok = !gram && q < NC;
         const double *C = col_ptr(k0 + nbw + (q_ok ? q : 0));
         const int e = fx_exp_of_hi(q_ok ? cur[k0 + nbw + q] : 0u);
-        float acc[kFxOrders][4];
+        float acc[kFxOrders][4], mag[4] = {0.f, 0.f, 0.f, 0.f};   // (mag: of |leading digits|)
         long long tot[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int o = 0; o < kFxOrders; ++o)
@@ -336,9 +375,13 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
           for (int i = 0; i < kFxD; ++i) {
             uint32_t a[4];
             bf_ldsm4t(a, aa + i * PR * 32);
+            if (i == 0) {
+              const uint32_t m[4] = {fx_abs2(a[0]), fx_abs2(a[1]), fx_abs2(a[2]), fx_abs2(a[3])};
+              fx_mma16816(mag, m, fx_abs2(b[0][0]), fx_abs2(b[0][1]));
+            }
 #pragma unroll
             for (int j = 0; j < kFxD; ++j)
-              if (i + j < kFxOrders) bf_mma(acc[i + j], a, b[j][0], b[j][1]);
+              if (i + j < kFxOrders) fx_mma16816(acc[i + j], a, b[j][0], b[j][1]);
           }
           if ((rb & 7) == 7 || rb == nblk - 1) {         // every 128 rows: still exact
 #pragma unroll
@@ -355,17 +398,48 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
         for (int k = 0; k < 4; ++k) {
           const int a = gid + 8 * (k >> 1), cc = 2 * tq + (k & 1);
           const int fa = s_f[a];
+          if (a >= nbw || fx_hi(s_up[a]) == 0) mag[k] = 1e30f;       // (no such reflector)
           if (gram) {
             const int fc = s_f[T * 8 + cc];
             s_G[a + (T * 8 + cc) * 16] =
                 (fa == kFxNonFinite || fc == kFxNonFinite) ? __longlong_as_double(0x7ff8000000000000ll)
                                                            : bf_value(tot[k], fa + fc - 54);
+            if (a >= T * 8 + cc || T * 8 + cc >= nbw || fa == kFxNonFinite || fc == kFxNonFinite)
+              mag[k] = 1e30f;
+            mag[k] *= 0.25f;                         // (2^20 for |up_a up_c|, and one binade lower)
           } else if ((T - 2) * 8 + cc < NC) {
             const unsigned mx = cur[k0 + nbw + (T - 2) * 8 + cc];
             Wb[a * (CT + 1) + warp * 8 + cc] =
                 (fa == kFxNonFinite || mx >= 0x7ff00000u) ? __longlong_as_double(0x7ff8000000000000ll)
                                                           : bf_value(tot[k], fx_exp_of_hi(mx) + fa - 54);
+            if (fa == kFxNonFinite || mx >= 0x7ff00000u || mx == 0) mag[k] = 1e30f;
+          } else {
+            mag[k] = 1e30f;
           }
+        }
+        // the entries whose |products| add up to less than 2^-kBfLoss of the scales (2^17 in
+        // leading digits; 2^-(kBfLoss + 1) for the Gram terms), again in FP64
+        unsigned low[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          low[k] = __ballot_sync(0xffffffffu, mag[k] < (float)(1 << (17 - kBfLoss)));
+        if (low[0] | low[1] | low[2] | low[3]) {
+          const BfPanel p = {A + (size_t)k0 * lda + k0, s_up, lda, nbw, skip, M, ntop > 0};
+          __syncwarp();
+          for (int cc = 0; cc < 8; ++cc)
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const unsigned bits = low[2 * t + (cc & 1)] >> (cc >> 1) & 0x11111111u;
+              if (bits == 0) continue;
+              const double *X = gram ? nullptr : col_ptr(k0 + nbw + (T - 2) * 8 + cc) + k0;
+              bf_dots8(p, X, gram ? T * 8 + cc : -1, 8 * t, s_dot[warp]);
+              if (lane < 8 && (bits >> (4 * lane) & 1)) {
+                const int a = 8 * t + lane;
+                if (gram) s_G[a + (T * 8 + cc) * 16] = s_dot[warp][lane];
+                else Wb[a * (CT + 1) + warp * 8 + cc] = s_dot[warp][lane];
+              }
+              __syncwarp();
+            }
         }
       }
       __syncthreads();
@@ -399,7 +473,9 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
             for (int d = 0; d < kFxD; ++d)
               *(uint4 *)(Wd + ((size_t)d * CT + tid) * 32 + h * 16) = fx_pack8(y, d);
           }
-          s_ecol[tid] = bad ? kFxNonFinite : g;
+          s_ecol[tid] = bad ? kFxNonFinite : key == kFxZero ? kFxZeroExp : g;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) Wb[j * (CT + 1) + tid] = w[j];   // (for entries formed again)
         }
       }
       __syncthreads();
@@ -462,19 +538,61 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
             bf_ldsm4(a, aa + i * PR * 32);
 #pragma unroll
             for (int j = 0; j < kFxD; ++j)
-              if (i + j < kFxOrders) bf_mma(acc[i + j], a, b[j][0], b[j][1]);
+              if (i + j < kFxOrders) fx_mma16816(acc[i + j], a, b[j][0], b[j][1]);
+          }
+          // An entry is below the line where it and its change are less than 2^-kBfLoss of
+          // the column's scale; half a row of the tile or 3/8 of a column of it count as lost
+          // (as in fx_upd_kernel) and are formed again from V and W' in FP64.
+          long long tt[4];
+          unsigned low = 0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int h = k & 1;
+            // in units of 2^55 digit products, each 2^(g - 113); an order of 16
+            // reflectors is below 2^22 (the leading digits of V count eightfold)
+            auto pair = [&](int o) { return fx_small(acc[o][k]) * 256 + fx_small(acc[o + 1][k]); };
+            tt[k] = fx_join(pair(0), pair(2), pair(4), pair(6), 19);
+            constexpr unsigned kLine = 1u << (25 - kBfLoss);
+            if ((unsigned)((int)(tt[k] >> 32) + (int)kLine) < 2 * kLine &&
+                (int)(fx_hi(xv[k]) >> 20) < g[h] + 1022 - kBfLoss)
+              low |= 1u << k;
+          }
+          if (__any_sync(0xffffffffu, low != 0)) {
+            unsigned in[4], lost = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int r = rb * 16 + gid + 8 * (k >> 1), h = k & 1;
+              if (r >= M || !q_ok[h] || g[h] == kFxNonFinite) low &= ~(1u << k);
+              in[k] = __ballot_sync(0xffffffffu, low >> k & 1);
+            }
+            const int cols_here = min(8, NC - (tile_lo - 2 + tl) * 8), rows_here = min(16, M - rb * 16);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int in_row = __popc(in[k & 2] >> (4 * gid) & 0xf) +
+                                 __popc(in[(k & 2) + 1] >> (4 * gid) & 0xf);
+              const int in_col = __popc((in[k & 1] | in[(k & 1) + 2]) >> tq & 0x11111111u) +
+                                 __popc((in[k & 1] & in[(k & 1) + 2]) >> tq & 0x11111111u);
+              if (2 * in_row >= cols_here || 8 * in_col >= 3 * rows_here) lost |= low & (1u << k);
+            }
+            if (__any_sync(0xffffffffu, lost != 0)) {
+              const BfPanel p = {A + (size_t)k0 * lda + k0, s_up, lda, nbw, skip, M, ntop > 0};
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                if (lost >> k & 1) {
+                  xv[k] -= bf_entry(p, Wb + slot + 2 * tq + (k & 1), CT + 1,
+                                    rb * 16 + gid + 8 * (k >> 1));
+                  tt[k] = 0;
+                }
+            }
           }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int r = rb * 16 + gid + 8 * (k >> 1), h = k & 1;
-            // in units of 2^55 digit products, each 2^(g - 113); an order of 16
-            // reflectors is below 2^22 (the leading digits of V count eightfold)
-            auto pair = [&](int o) { return fx_small(acc[o][k]) * 256 + fx_small(acc[o + 1][k]); };
-            const long long tt = fx_join(pair(0), pair(2), pair(4), pair(6), 19);
             double x;
-            if (!odd_scale) x = xv[k] - fx_to_double(tt, g[h] - 58);
+            if (!odd_scale) x = xv[k] - fx_to_double(tt[k], g[h] - 58);
             else if (g[h] == kFxNonFinite) x = __longlong_as_double(0x7ff8000000000000ll);
-            else x = xv[k] - bf_value(tt, g[h] - 58);
+            else if (g[h] == kFxZeroExp) x = xv[k];
+            else x = xv[k] - bf_value(tt[k], g[h] - 58);
             if (r < M && q_ok[h]) {
               P[h][prow(r)] = x;
               if (rb > 0) mx[h] = max(mx[h], fx_hi(x));  // (rows of the next panel)

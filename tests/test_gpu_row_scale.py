@@ -153,3 +153,39 @@ def test_apply_qt(ctx, nrhs, use_wy, w):  # noqa: F811
     one = np.stack([oracle.apply_qt(F, u, np.ascontiguousarray(B[:, j])) for j in range(nrhs)], 1)
     eo, eg = (float((np.abs(v - want).max(axis=1) / alpha).max()) for v in (one, host(Bd)))
     report(f"qt nrhs={nrhs} wy={use_wy}", w, eo, eg, n)
+
+
+def batch_factor(c, A, copies=1):
+    from paper_2506_09463_gb300 import abi
+    m, n = A.shape
+    Ad = [dev(A) for _ in range(copies)]
+    bd = torch.ones(copies, m, dtype=torch.float64, device="cuda")
+    up = torch.zeros(copies, n, dtype=torch.float64, device="cuda")
+    st = abi.slqr_batch_factor(c.ctx, [m] * copies, [n] * copies, [a.data_ptr() for a in Ad],
+                               [m] * copies, [v.data_ptr() for v in up],
+                               [v.data_ptr() for v in bd], abi.SLQR_FP64, None, None,
+                               torch.cuda.current_stream().cuda_stream)
+    abi.check(c.ctx, st, "slqr_batch_factor")
+    assert c.sync() == 0
+    return host(Ad[0]), host(up[0])
+
+
+# (400 problems of up to 128 rows and 200 of up to 256 run on the smaller CTAs)
+@pytest.mark.parametrize("w", WEIGHTS)
+@pytest.mark.parametrize("m,n,h,copies", [(100, 60, 5, 400), (250, 120, 20, 200),
+                                          (500, 200, 20, 1), (128, 128, 40, 400)])
+def test_batch_heavy_rows_on_top(ctx, m, n, h, copies, w):  # noqa: F811
+    A = heavy_top(m, n, h, w, 8)
+    Fo, upo, _ = oracle.h12_factor(A)
+    F, up = batch_factor(ctx, A, copies)
+    report(f"batch {m}x{n} h={h}", w, row_errors(A, Fo, upo).max(), row_errors(A, F, up).max(), n)
+
+
+@pytest.mark.parametrize("w", WEIGHTS)
+@pytest.mark.parametrize("m,n,copies", [(250, 120, 200), (500, 200, 1)])
+def test_batch_heavy_rows_without_the_first_columns(ctx, m, n, copies, w):  # noqa: F811
+    A = block_sparse(m, n, w, 9)
+    Fo, upo, _ = oracle.h12_factor(A)
+    F, up = batch_factor(ctx, A, copies)
+    report(f"batch block {m}x{n}", w, light_rows_error(A, Fo, upo),
+           light_rows_error(A, F, up), n)
