@@ -106,13 +106,17 @@ slqr_status slqr_check_bounded_wait(slqr_ctx *ctx, unsigned polls, void *stream)
 
 /*
  * Set how many polls a bounded device wait of this context makes before it
- * gives up (1 .. 2^24; 0 restores the default 2^24, about 1.5 s): the panel
- * factorization's polled exchange of per-column records and grid barrier,
+ * reports (1 .. 2^24; 0 restores the default 2^24, about 1.5 s): the panel
+ * factorization's polled exchange of per-column records and grid barrier, the
+ * exchanges of Q^T b and of the back-substitution of few right-hand sides,
  * and the grid barriers of the mixed-precision Q application and triangular
- * solves.  A wait that gives up records SLQR_ETIMEOUT in the status word
- * (slqr_sync; slqr_lstsq_mixed and slqr_lstsq_mixed_ex return it) and its
- * kernel returns, leaving that call's outputs unspecified; the context stays
- * usable.  The tensor-core kernels' mbarrier waits keep the fixed default.
+ * solves.  A wait past the limit records SLQR_ETIMEOUT in the status word
+ * (slqr_sync; slqr_lstsq_mixed and slqr_lstsq_mixed_ex return it).  The
+ * cooperative kernels then return; kernels on thread-block clusters, Q^T b and
+ * the back-substitution go on to 2^24 polls, since other CTAs still send to
+ * the one that waits, and return when those run out.
+ * Either way that call's outputs are unspecified and the context stays usable.
+ * The tensor-core kernels' mbarrier waits keep the fixed default.
  * A failure-detection aid (no counterpart in the paper): with a limit of a
  * few polls the waits run out on purpose.  Not while calls are in flight.
  * Errors: SLQR_EINVAL (polls above 2^24, NULL context).

@@ -179,7 +179,7 @@ __device__ __forceinline__ bool trsm_unset(double v) {
 // took 12.4 us.
 __global__ void __launch_bounds__(kThreads, 1)
 trsm_chain_kernel(const double *__restrict__ A, int lda, int n, double *__restrict__ B, int ldb,
-                  const double *__restrict__ Rinv, double *slots, int *status) {
+                  const double *__restrict__ Rinv, double *slots, int *status, unsigned spin) {
   constexpr int CW = kTB * kTB / kThreads;     // columns of a thread
   __shared__ double Xs[2][kTB];
   __shared__ double part[kThreads / kTB][kTB];
@@ -209,10 +209,10 @@ trsm_chain_kernel(const double *__restrict__ A, int lda, int n, double *__restri
       for (unsigned it = 0;; ++it) {
         asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(slot) : "memory");
         if (!trsm_unset(v) || dead) break;
-        if (it > kSpinLimit) {                 // (only if the grid were not resident)
-          record_status(status, SLQR_ETIMEOUT);
-          dead = true;
-        }
+        // (past the context's limit it reports and goes on waiting, as the blocks above
+        // wait for this one's x)
+        if (it == spin) record_status(status, SLQR_ETIMEOUT);
+        if (it > kSpinLimit) dead = true;
       }
       Xs[b & 1][r] = v;
     }
@@ -296,7 +296,8 @@ extern "C" slqr_status slqr_solve_r(slqr_ctx *ctx, int n, const double *A, int l
   if (chain) {
     slot = prof_begin(ctx, s);
     int *status = ctx->d_status;
-    void *args[] = {&A, &lda, &n, &B, &ldb, &Rinv, &slots, &status};
+    unsigned spin = ctx->spin_limit;
+    void *args[] = {&A, &lda, &n, &B, &ldb, &Rinv, &slots, &status, &spin};
     e = cudaLaunchCooperativeKernel((const void *)trsm_chain_kernel, dim3(nblk, nrhs),
                                     dim3(kThreads), args, 0, s);
     if (e != cudaSuccess)
