@@ -176,7 +176,7 @@ void slqr_set_tuning(int panel_width, int panel_rows_min);
  *        -1   always the cooperative panel (one grid-wide exchange of partial
  *             sums through L2 per column); this also switches the Q
  *             applications of the mixed-precision refinement to their
- *             cooperative kernel (FP64 panels of width 64 stay on clusters)
+ *             cooperative kernel
  *         1..16  a cluster of that many CTAs wherever the panel's rows fit
  *             their shared memory, else the cooperative panel
  * The cluster panel splits the panel's rows over the CTAs of one cluster,

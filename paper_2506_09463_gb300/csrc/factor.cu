@@ -1234,11 +1234,8 @@ static size_t panel_smem_bytes(int nb, int R, size_t elem) {
   return ((size_t)nb * R * elem + 15) / 16 * 16 + (size_t)nb * nb * sizeof(double);
 }
 
-// ntop > 0: A = [L^T; C] with an upper-triangular top block of ntop = n rows
-// (the structure-aware factorization: each panel skips the zero rows between
-// its diagonal block and C).  wy32: compact-WY store in panels of 32 of a
-// factorization in panels of 64 (wy NULL), its blocks on the diagonals of the
-// panels' own.
+// Compact-WY store in panels of 32 of a factorization in panels of 64: its blocks are on
+// the diagonals of the panels' own.
 __global__ void __launch_bounds__(256)
 wy32_kernel(const double *__restrict__ wy, int K, double *__restrict__ out) {
   const int p = blockIdx.x, o = (p & 1) * 32;
@@ -1252,6 +1249,10 @@ wy32_kernel(const double *__restrict__ wy, int K, double *__restrict__ out) {
   if (threadIdx.x < 32) dst[2 * 32 * 32 + threadIdx.x] = src[2 * 64 * 64 + o + threadIdx.x];
 }
 
+// ntop > 0: A = [L^T; C] with an upper-triangular top block of ntop = n rows
+// (the structure-aware factorization: each panel skips the zero rows between
+// its diagonal block and C).  wy32: receives the store in panels of 32 of a
+// factorization in panels of 64 (wy NULL).
 template <typename T, int NB>
 static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, double *up,
                                double *wy, cudaStream_t stream, int ntop = 0,
@@ -1334,6 +1335,11 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   // path T_{i,i} early).
   cudaStream_t aux = ctx->aux_stream;
   unsigned bar_base = 0;
+  // The panel in registers, unless slqr_set_panel_cluster chose another one.  (Its Gram
+  // terms come from the digits of V, so the FP64-pipe path keeps panel_kernel.)
+  auto grid_shape = [&](int M) {
+    return fx && g_panel_cluster == 0 ? grid_panel_shape(ctx, M, rmin) : GridPanelShape();
+  };
   auto launch_panel = [&](int pnl, cudaStream_t s) -> slqr_status {
     const int k0 = pnl * NB;
     const int nbw = std::min(NB, K - k0);
@@ -1362,9 +1368,7 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
       return SLQR_OK;                             // (no grid barrier used)
     }
     if constexpr (std::is_same<T, double>::value && NB == 64) {
-      // (the Gram terms of this panel come from the digits of V, so the FP64-pipe
-      // path keeps the panel below)
-      const GridPanelShape shape = fx ? grid_panel_shape(ctx, M, rmin) : GridPanelShape();
+      const GridPanelShape shape = grid_shape(M);
       if (shape.R > 0) {
         GridPanelParams gp;
         gp.A = A; gp.up = up; gp.wy = wy_store + (size_t)pnl * wy_panel_doubles(NB);
@@ -1413,8 +1417,7 @@ static slqr_status factor_impl(slqr_ctx *ctx, int m, int n, T *A, int lda, doubl
   // where that runs on the tensor cores, else at once
   auto on_grid = [&](int pnl) {
     const int k0 = pnl * NB, nbw = std::min(NB, K - k0);
-    return fx && panel_cluster_ctas(ctx, false, NB, m - k0 - skip_of(k0, nbw), nbw) == 0 &&
-           grid_panel_shape(ctx, m - k0 - skip_of(k0, nbw), rmin).R > 0;
+    return grid_shape(m - k0 - skip_of(k0, nbw)).R > 0;
   };
   auto gram_in_lookahead = [&](int pnl) {
     return pnl + 1 < np && std::min(NB, K - (pnl + 1) * NB) >= kFxMinCols;
