@@ -141,8 +141,11 @@ static slqr_status apply_qt_impl(slqr_ctx *ctx, int m, int n, const double *A, i
   const size_t head_bytes = align_up((wy_doubles + gp_doubles) * 8, 256);
   // few right-hand sides: all panels in one launch (qt_vec.cu); kFxMinCols and
   // up: the products on the tensor cores (tc_fp64.cu); unless the scratch of
-  // either does not fit
-  bool vec = nrhs < kFxMinCols && qt_vec_bytes(ctx, m, K, NB) > 0;
+  // either does not fit.  A launch of qt_vec.cu takes 2 or 4 right-hand sides and
+  // about 28 us, the tiled products 82 to 100 us a panel: so one panel goes to
+  // two launches at most (64 x 32, 15 right-hand sides: 130 us in four, 97 tiled).
+  bool vec = nrhs < kFxMinCols && qt_vec_bytes(ctx, m, K, NB) > 0 &&
+             qt_vec_launches(ctx, m, nrhs) <= 2 * np;
   bool fx = NB == 64 && nrhs >= kFxMinCols;
   const size_t fx_v = align_up(fx_v_bytes(m), 256);
   const size_t fx_work = align_up(fx_work_bytes(m, nrhs, ctx->num_sms), 256);

@@ -374,6 +374,14 @@ size_t qt_vec_bytes(const slqr_ctx *ctx, int m, int K, int nb) {
   return np * (kQvT + 4 * 64 * (size_t)(P / cluster)) * sizeof(double);
 }
 
+static int qt_most(int R) { return R == 128 ? 2 : 4; }
+
+int qt_vec_launches(const slqr_ctx *ctx, int m, int nrhs) {
+  int P = 0, cluster = 0;
+  const int most = qt_most(qt_shape(ctx, m, &P, &cluster));
+  return (nrhs + most - 1) / most;
+}
+
 slqr_status qt_vec(slqr_ctx *ctx, int m, int K, int nb, const double *A, int lda, const double *up,
                    const double *wy, int nrhs, double *B, int ldb, int ntop, void *work,
                    cudaStream_t stream) {
@@ -384,7 +392,7 @@ slqr_status qt_vec(slqr_ctx *ctx, int m, int K, int nb, const double *A, int lda
   int slot = prof_begin(ctx, stream);
   qt_t_kernel<<<dim3(np, 4), 128, 0, stream>>>(wy, K, nb, T);
   prof_end(ctx, stream, slot, kTw, 0.0);
-  const int most = R == 128 ? 2 : 4;
+  const int most = qt_most(R);
   for (int k = 0; k < nrhs; k += most) {
     const int nr = std::min(most, nrhs - k), tr = nr == 3 ? 4 : nr;
     QtVecParams p;

@@ -201,6 +201,7 @@ void fx_prep(const double *wy, int K, int nb, double *Gt, cudaStream_t stream);
 // store; work: qt_vec_bytes (0: m is too tall for it).
 slqr_status init_qt_vec_attrs(slqr_ctx *ctx);
 size_t qt_vec_bytes(const slqr_ctx *ctx, int m, int K, int nb);
+int qt_vec_launches(const slqr_ctx *ctx, int m, int nrhs);
 slqr_status qt_vec(slqr_ctx *ctx, int m, int K, int nb, const double *A, int lda, const double *up,
                    const double *wy, int nrhs, double *B, int ldb, int ntop, void *work,
                    cudaStream_t stream);
