@@ -115,6 +115,17 @@ __device__ __noinline__ void bf_dots8(BfPanel p, const double *x, int c, int a0,
   }
   __syncwarp();
 }
+// the same for this thread's reflector a, of a panel [L^T; C] with few rows of C (or of few
+// rows at all)
+constexpr int kBfFewRows = 32;
+__device__ __noinline__ double bf_dot1(BfPanel p, const double *x, int c, int a) {
+  auto at = [&](int r) { return c >= 0 ? bf_v(p, r, c) : x[bf_row(p, r)]; };
+  double s = p.up[a] * at(a);
+  const int r0 = p.stacked ? p.nbw : a + 1;
+#pragma unroll 4
+  for (int r = r0; r < p.M; ++r) s = fma(bf_v(p, r, a), at(r), s);
+  return s;
+}
 // sum_a V(r, a) W'(a) for this thread's row and column (W'(a) at w[a * ldw])
 __device__ __noinline__ double bf_entry(BfPanel p, const double *w, int ldw, int r) {
   double s = 0.0;
@@ -425,8 +436,18 @@ static __device__ __noinline__ void batch_fx_factor(double *A, int lda, int m, i
           low[k] = __ballot_sync(0xffffffffu, mag[k] < (float)(1 << (17 - kBfLoss)));
         if (low[0] | low[1] | low[2] | low[3]) {
           const BfPanel p = {A + (size_t)k0 * lda + k0, s_up, lda, nbw, skip, M, ntop > 0};
+          const bool few = M <= 8 || (ntop > 0 && M - nbw <= kBfFewRows);
           __syncwarp();
-          for (int cc = 0; cc < 8; ++cc)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (!few || !(low[k] >> lane & 1)) continue;
+            const int a = gid + 8 * (k >> 1), cc = 2 * tq + (k & 1);
+            const double *X = gram ? nullptr : col_ptr(k0 + nbw + (T - 2) * 8 + cc) + k0;
+            const double d = bf_dot1(p, X, gram ? T * 8 + cc : -1, a);
+            if (gram) s_G[a + (T * 8 + cc) * 16] = d;
+            else Wb[a * (CT + 1) + warp * 8 + cc] = d;
+          }
+          for (int cc = few ? 8 : 0; cc < 8; ++cc)
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
               const unsigned bits = low[2 * t + (cc & 1)] >> (cc >> 1) & 0x11111111u;

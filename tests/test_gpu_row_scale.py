@@ -189,3 +189,22 @@ def test_batch_heavy_rows_without_the_first_columns(ctx, m, n, copies, w):  # no
     F, up = batch_factor(ctx, A, copies)
     report(f"batch block {m}x{n}", w, light_rows_error(A, Fo, upo),
            light_rows_error(A, F, up), n)
+
+
+@pytest.mark.parametrize("w", WEIGHTS)
+@pytest.mark.parametrize("n,m_eq", [(60, 3), (98, 40), (300, 150), (40, 0)])
+def test_batch_stacked(ctx, n, m_eq, w):  # noqa: F811
+    """Rows of L spread over w, in any order, over few rows of C and many."""
+    from paper_2506_09463_gb300 import abi
+    A, _ = workloads.slsqp_stack(n, m_eq, seed=n)
+    A = np.array(A)
+    A[:n] *= (w ** np.random.default_rng(n).uniform(0.0, 1.0, n))[:, None]
+    Fo, upo, _ = oracle.h12_factor(A)
+    Ad, up = dev(A), torch.zeros(n, dtype=torch.float64, device="cuda")
+    st = abi.slqr_batch_factor_stacked(ctx.ctx, [n], [m_eq], [Ad.data_ptr()], [n + m_eq],
+                                       [up.data_ptr()], None, abi.SLQR_FP64, None, None,
+                                       torch.cuda.current_stream().cuda_stream)
+    abi.check(ctx.ctx, st, "slqr_batch_factor_stacked")
+    assert ctx.sync() == 0
+    report(f"batch stacked {n}+{m_eq}", w, row_errors(A, Fo, upo).max(),
+           row_errors(A, host(Ad), host(up)).max(), n)
