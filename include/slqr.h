@@ -157,8 +157,11 @@ slqr_status slqr_factor(slqr_ctx *ctx, int m, int n, double *A, int lda, double 
  * paper; its alpha/beta task sizes play this role on the CPU):
  *   panel_width     32 or 64 forces the panel width (0: 32 for n <= 256, else 64)
  *   panel_rows_min  smallest slice of rows one panel CTA holds (0: by panel
- *                   height, 64 below 1536 rows, 128 below 6144, else 192);
- *                   larger values put fewer CTAs on each panel
+ *                   height; the cooperative panel 64 below 1536 rows, 128 below
+ *                   6144, else 192; FP64 panels of width 64 in registers 32 to
+ *                   80 on one cluster of up to 16 CTAs, above 1280 rows the
+ *                   fewest that 64 CTAs hold, up to 256); larger values put
+ *                   fewer CTAs on each panel
  * Changing the panel width changes slqr_panel_width and slqr_wy_size: set it
  * before allocating compact-WY stores, and not while calls are in flight.
  * These overrides take precedence over the per-shape settings of
@@ -343,6 +346,13 @@ slqr_status slqr_apply_qt_stacked(slqr_ctx *ctx, int n, int m_eq, const double *
  * when the steps stop contracting below 1e-10 ||x||, the FP64 noise level of
  * an ill-conditioned problem);
  * b[i][0:n] = x_i, b[i][n:m] is unspecified.
+ * The kernel of SLQR_FP64 problems is chosen for the launch, by its largest
+ * problem and their number (4, 8 or 16 warps to a problem), and each adds its
+ * sums in its own order: the last bits of a problem's results depend on the
+ * batch it is in; the same batch gives the same bits.
+ * Device scratch, kept by the context: the problem table, and for SLQR_FP32 up
+ * to 1.2 MB for every CTA of a launch, three of which an SM holds (two where
+ * that does not fit the device or the context's budget).
  * The host arrays are read before the call returns.  The problems must not
  * overlap in memory.  Errors: SLQR_EINVAL, SLQR_ENOMEM, SLQR_ECUDA.
  */
@@ -590,7 +600,10 @@ slqr_status slqr_lstsq_mixed_ex(slqr_ctx *ctx, int m, int n, const double *A, in
  * Admission is in arrival order and by the context's HBM budget (bytes held
  * by resident factorizations and requests in flight); a request that cannot
  * fit waits until memory is freed, and one larger than the whole budget
- * fails with SLQR_EBUSY.  Admitted FP64 requests with m <= slqr_batch_max_rows()
+ * fails with SLQR_EBUSY.  The contexts the request loop makes for its streams,
+ * batches and mixed lanes have no budget of their own: their workspaces (as
+ * large as the largest request each has served needs; up to 544 MB for a
+ * SLQR_FP32 batch) are kept and not counted.  Admitted FP64 requests with m <= slqr_batch_max_rows()
  * share one persistent batched launch, and so do SLQR_FP32 FACTOR_SOLVE
  * requests of that size; larger FP64 ones run one per stream on a pool of
  * streams; every other mixed-precision request runs on a mixed lane (a helper

@@ -137,7 +137,7 @@ struct BatchSmem {
 // The H12 factorization of one m x n problem by one CTA (see the file
 // header).  T == double: all FP64.  T == float: dot products, updates, the
 // norm, cl, up, b and sigma in FP32 (FP64 for a column whose power-of-two
-// scale is extreme for FP32), up, tau and G stored in FP64.  When
+// scale is extreme for FP32); tau and G stored in T, up in FP64.  When
 // G_out/tau_out are given, each panel's
 // striu(V^T V) and tau are kept there (the mixed path reuses them to apply Q).
 // Bcol (T == double only) is an extra right-hand-side column updated with the

@@ -160,10 +160,6 @@ __device__ __forceinline__ void mbar_expect(unsigned long long *mbar, unsigned b
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                ::"r"((unsigned)__cvta_generic_to_shared(mbar)), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(unsigned long long *mbar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];"
-               ::"r"((unsigned)__cvta_generic_to_shared(mbar)) : "memory");
-}
 // Bounded wait for the phase of the given parity.  Past `report` polls (the
 // context's spin limit) it records SLQR_ETIMEOUT once but goes on waiting, up
 // to kSpinLimit polls, so that normally no store of the column is still in
