@@ -33,8 +33,8 @@
 //    CTA barrier a step, after the multipliers, is left.  In one cluster its
 //    partials are counted apart from the others', so that the pivot starts while
 //    the other columns' sums are still coming.
-// Microseconds a column (with 64 columns): 2.5 at 512 rows, 3.4 at 1100, 3.6 at
-// 2048, 4.2 at 4096; panel_kernel took 9.8 at 8192.
+// Microseconds a column (with 64 columns): 2.5 at 512 rows, 3.5 at 1100, 3.6 at
+// 2048, 4.3 at 4096, 5.7 at 8192, 8.5 at 16384; panel_kernel took 9.8 at 8192.
 #include "cluster_common.cuh"
 #include "pivot_fp64.cuh"
 
@@ -559,8 +559,8 @@ slqr_status init_grid_panel_attrs(slqr_ctx *ctx) {
 }
 
 // Rows per CTA, smallest first.  One cluster up to 16 CTAs of 80 rows (1100 rows:
-// 3.4 us a column, 35 CTAs of 32 rows in clusters of 8 3.5; 1300 rows on CTAs of
-// 96: 3.7 against 3.6).  Above that clusters of 8, 64 CTAs at most while 256 rows
+// 0.1 us a column less than 35 CTAs of 32 rows in clusters of 8; 1300 rows on CTAs of
+// 96: 0.1 more).  Above that clusters of 8, 64 CTAs at most while 256 rows
 // each are enough: the sums of more clusters take longer to arrive than the
 // shorter slices save (8192 rows: 6.2 us a column on 64 CTAs, 7.6 on 104), and the
 // trailing update runs on the other SMs.

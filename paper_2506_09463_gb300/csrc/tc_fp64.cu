@@ -73,46 +73,69 @@ struct FxPanel {
   int ld, nbw, M, skip;                // skip > 0: [L^T; C], the top rows hold the pivots only
 };
 
-// out[k] = sum_i V(i, a0 + k) x_i for k < 8 on the FP64 pipe, by a warp (x: the column at
-// the panel's first row).  Bound by the pipe: a load of x and eight of V (coalesced) to
-// eight FMAs of 16 clocks each.
-static __device__ __noinline__ void fx_dots8(FxPanel p, const double *x, int a0, double *out) {
+// out[k] = sum_i V(i, a0 + k) x_i for k < 8 on the FP64 pipe, by a warp, for C columns x
+// (at the panel's first row, ldx apart; their results 64 apart).  Bound by the pipe: eight
+// loads of V (coalesced) to 8 C FMAs of 16 clocks each, where V comes from L2 ([L^T; C] of
+// 4000 + 1000 with L's rows over 10^6: 37 ms with one column, 31 with two).
+template <int C>
+static __device__ __noinline__ void fx_dots8(FxPanel p, const double *x, size_t ldx, int a0,
+                                             double *out) {
   const int lane = threadIdx.x & 31, na = min(8, p.nbw - a0);
-  double acc[8];
+  double acc[C][8];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc[k] = 0.0;
-  for (int i = lane; i < p.nbw; i += 32) {
-    const double xi = x[i];
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[c][k] = 0.0;
+  auto add = [&](const double *v, size_t ld, const double (&xi)[C]) {
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (k < na) acc[k] = fma(p.Vtop[(a0 + k) * 64 + i], xi, acc[k]);
+      if (k < na) {
+        const double t = v[k * ld];
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[c][k] = fma(t, xi[c], acc[c][k]);
+      }
+  };
+  if (p.skip > 0) {                                    // (the pivots only)
+    if (lane < na) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k == lane)
+#pragma unroll
+          for (int c = 0; c < C; ++c) acc[c][k] = p.Vtop[(a0 + k) * 65] * x[c * ldx + a0 + k];
+    }
+  } else {
+    for (int i = lane; i < p.nbw; i += 32) {
+      double xi[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) xi[c] = x[c * ldx + i];
+      add(p.Vtop + a0 * 64 + i, 64, xi);
+    }
   }
   // (128 rows of x at a time: where they are zero, as in a banded or block matrix, V is
   // not read)
   const double *v = p.tail + (size_t)a0 * p.ld;
   for (int i0 = p.nbw + lane; i0 - lane < p.M; i0 += 128) {
-    double xi[4];
+    double xi[4][C];
     bool any = false;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      xi[t] = i0 + 32 * t < p.M ? x[p.skip + i0 + 32 * t] : 0.0;
-      any |= (unsigned long long)__double_as_longlong(xi[t]) << 1 != 0;
-    }
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        xi[t][c] = i0 + 32 * t < p.M ? x[c * ldx + p.skip + i0 + 32 * t] : 0.0;
+        any |= (unsigned long long)__double_as_longlong(xi[t][c]) << 1 != 0;
+      }
     if (!__any_sync(0xffffffffu, any)) continue;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int i = min(i0 + 32 * t, p.M - 1);
+    for (int t = 0; t < 4; ++t) add(v + min(i0 + 32 * t, p.M - 1), p.ld, xi[t]);
+  }
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k < na) acc[k] = fma(v[(size_t)k * p.ld + i], xi[t], acc[k]);
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[c][k] += __shfl_xor_sync(0xffffffffu, acc[c][k], o);
+      if (lane == 0) out[c * 64 + k] = acc[c][k];
     }
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-    if (lane == 0) out[k] = acc[k];
-  }
   __syncwarp();
 }
 // the same for this thread's reflector a, of a panel of few rows
@@ -137,10 +160,13 @@ static __device__ __noinline__ FxFour fx_row4(FxPanel p, const double *w, int nc
   const double *v = i < p.nbw ? p.Vtop + i : p.tail + min(i, p.M - 1);
   const size_t ld = i < p.nbw ? 64 : p.ld;
 #pragma unroll 4
-  for (int a = 0; a < p.nbw; ++a) {
-    const double t = v[a * ld];
+  for (int a = 0; a < p.nbw; a += 2) {                 // (W' is zero past nbw, V not read there)
+    const double t0 = v[a * ld], t1 = a + 1 < p.nbw ? v[(a + 1) * ld] : 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s.v[k] = fma(t, w[min(k, nc - 1) * 64 + a], s.v[k]);
+    for (int k = 0; k < 4; ++k) {
+      const double2 u = *(const double2 *)(w + min(k, nc - 1) * 64 + a);
+      s.v[k] = fma(t1, u.y, fma(t0, u.x, s.v[k]));
+    }
   }
   return s;
 }
@@ -881,13 +907,13 @@ fx_prep_kernel(const double *__restrict__ wy, int K, int nb, double *__restrict_
 // W' in FP64 replaces the first partial, for the entries of X -= V W' formed again.
 // --------------------------------------------------------------------------
 template <int CPW>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256, CPW == 1 ? 4 : 3)
 fx_tw_kernel(double *__restrict__ Wp, int S, int N, FxPanel p, const double *__restrict__ X, int ldx,
              const unsigned *__restrict__ cmax, const double *__restrict__ Gt,
              unsigned char *__restrict__ Wimg, int *__restrict__ ecol) {
   constexpr int NB = 64, WARPS = CPW == 1 ? 1 : 8;   // (CPW 1: all threads sum one column)
   __shared__ double G[NB * NB];
-  __shared__ double part[CPW == 1 ? 4 : 8][NB];
+  __shared__ double part[CPW == 1 ? 4 : 8 * CPW][NB];
   __shared__ float psum[4][NB];
   __shared__ unsigned long long s_low;
   const double *wy = p.Vtop;
@@ -920,7 +946,6 @@ fx_tw_kernel(double *__restrict__ Wp, int S, int N, FxPanel p, const double *__r
     if (fx_hi(u) == 0 || cm == 0 || cm >= 0x7ff00000u || sum >= 1.f / (1 << kFxLoss)) return false;
     return (int)(fx_hi(X[(size_t)c * ldx + a]) >> 20) < (int)(cm >> 20) - kFxLoss;
   };
-  auto dots = [&](int c, int a0, double *out) { fx_dots8(p, X + (size_t)c * ldx, a0, out); };
   // of few rows every lane forms its own (V of [L^T; C] has its pivots and C's rows)
   auto few = [&](int c, bool low0, bool low1, double &r0, double &r1) {
     if (low0) r0 = fx_dot1(p, X + (size_t)c * ldx, lane);
@@ -963,7 +988,8 @@ fx_tw_kernel(double *__restrict__ Wp, int S, int N, FxPanel p, const double *__r
     }
     __syncthreads();
     if (s_low != 0) {                                  // (uniform)
-      if ((s_low >> (8 * warp)) & 0xff) dots(c0, 8 * warp, part[0] + 8 * warp);
+      if ((s_low >> (8 * warp)) & 0xff)
+        fx_dots8<1>(p, X + (size_t)c0 * ldx, ldx, 8 * warp, part[0] + 8 * warp);
       __syncthreads();
       if (low0) r0[0] = part[0][lane];
       if (low1) r1[0] = part[0][lane + 32];
@@ -996,22 +1022,30 @@ fx_tw_kernel(double *__restrict__ Wp, int S, int N, FxPanel p, const double *__r
     }
     __syncthreads();
     if (c0 >= N) return;
+    bool low0[CPW], low1[CPW];
+    unsigned l0 = 0, l1 = 0;
 #pragma unroll
     for (int k = 0; k < CPW; ++k) {
-      if (c0 + k >= N) break;
-      const bool low0 = low(c0 + k, lane, m0[k], u0), low1 = low(c0 + k, lane + 32, m1[k], u1);
+      const bool in = c0 + k < N;
+      low0[k] = in && low(c0 + k, lane, m0[k], u0);
+      low1[k] = in && low(c0 + k, lane + 32, m1[k], u1);
       if (p.M <= kFxFewRows) {
-        few(c0 + k, low0, low1, r0[k], r1[k]);
-        __syncwarp();
-        continue;
+        few(c0 + k, low0[k], low1[k], r0[k], r1[k]);
+        low0[k] = low1[k] = false;
       }
-      const unsigned l0 = __ballot_sync(0xffffffffu, low0), l1 = __ballot_sync(0xffffffffu, low1);
-      if ((l0 | l1) == 0) continue;
+      l0 |= __ballot_sync(0xffffffffu, low0[k]);
+      l1 |= __ballot_sync(0xffffffffu, low1[k]);
+    }
+    if (l0 | l1) {                                     // the warp's columns together
+      double *dots = part[warp * CPW];
       for (int g = 0; g < 8; ++g)
-        if (((g < 4 ? l0 : l1) >> (8 * (g & 3))) & 0xff) dots(c0 + k, 8 * g, part[warp] + 8 * g);
-      if (low0) r0[k] = part[warp][lane];
-      if (low1) r1[k] = part[warp][lane + 32];
-      __syncwarp();
+        if (((g < 4 ? l0 : l1) >> (8 * (g & 3))) & 0xff)
+          fx_dots8<CPW>(p, X + (size_t)c0 * ldx, c0 + CPW <= N ? ldx : 0, 8 * g, dots + 8 * g);
+#pragma unroll
+      for (int k = 0; k < CPW; ++k) {
+        if (low0[k]) r0[k] = dots[k * NB + lane];
+        if (low1[k]) r1[k] = dots[k * NB + lane + 32];
+      }
     }
   }
   // (on and below the diagonal Gt is zero, but a product with an entry that is
