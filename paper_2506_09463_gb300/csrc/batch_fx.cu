@@ -14,6 +14,9 @@
 //    rows, reading C once and splitting it in registers; the Gram terms of V^T V
 //    are two more such column tiles.  Column maxima for the digits come from the
 //    update before.
+//  * results whose digits may be lost (fx_digits.cuh) are formed again in FP64: W and
+//    Gram entries by the sums of |leading digits| formed beside them, entries of
+//    C -= V W' by their own size and their change's;
 //  * W' = T^T W by substitution, one thread per column, in FP64;
 //  * the back-substitution goes in blocks of 32 rows.
 // CTAs of 4, 8 or 16 warps hold problems of up to 128, 256 or 512 rows, four,
